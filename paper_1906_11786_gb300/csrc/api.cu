@@ -415,7 +415,7 @@ bool tc_gemm_path(bg_dtype dt, int H) {
 
 struct BwdWs {
   size_t dM, Wt, part;                 // fp32 SIMT path
-  size_t dMb, dMT, Wp, ETa, tpart;     // bf16 path with tensor-core GEMMs
+  size_t dMb, Wp, ETa, tpart;          // bf16 path with tensor-core GEMMs
   size_t super;                        // supernode edges (after everything else)
   size_t total;
 };
@@ -430,7 +430,6 @@ BwdWs bwd_ws(const bg_plan* p, bg_dtype dt, int H) {
   if (tc_gemm_path(dt, H)) {
     size_t q = 0;
     w.dMb = q; q += al(n * p->P * H * 2);
-    w.dMT = q; q += al(n * p->P * H * 2);
     w.Wp = q; q += al((size_t)p->P * H * H * 2);
     w.ETa = q; q += al((size_t)(H + 16) * n * 2);
     w.tpart = q; q += al(sizeof(float) * bg::gemm_tn_part_floats(p->P * H, H + 16, (int64_t)n));
@@ -470,7 +469,7 @@ GgnnFwdWs ggnn_fwd_ws(const bg_plan* p, bg_dtype dt, int H) {
 struct GgnnBwdWs {
   size_t gi, gh, dgi, dgh, dX, g, part, prop;
   size_t Ybf, dgib, dghb, dgiT, dghT, YTa, ETa, WihT, WhhT, tpart;  // tensor-core GEMM path
-  size_t dXT, dMT, Wk, tcpart, split, sup, dWs, dbs;  // and with the band kernel (bf16 Y saved)
+  size_t dXb, dMb, Wk, tcpart, split, sup, dWs, dbs;  // and with the band kernel (bf16 Y saved)
   size_t total;
 };
 size_t tc_part_floats(const bg_plan* p, int H, int T);
@@ -498,8 +497,8 @@ GgnnBwdWs ggnn_bwd_ws(const bg_plan* p, bg_dtype dt, int H, int T) {
     w.WhhT = o; o += al((size_t)3 * H * H * 2);
     w.tpart = o; o += al(sizeof(float) * gru_tpart_floats(p, H, T));
     if (ybf) {
-      w.dXT = o; o += al(n * H * 2);
-      w.dMT = o; o += al((size_t)p->P * H * n * 2);
+      w.dXb = o; o += al(n * H * 2);
+      w.dMb = o; o += al((size_t)p->P * H * n * 2);
       w.Wk = o; o += bg::band_tc_w_bytes(p, H);
       w.tcpart = o; o += al(sizeof(float) * tc_part_floats(p, H, T));
       w.split = o; o += al(sizeof(float) * bg::band_tc_split_floats(p, H));
@@ -587,7 +586,7 @@ TcFwdWs tc_fwd_ws(const bg_plan* p, int H) {
   return w;
 }
 struct TcBwdWs {
-  size_t g, dXT, dMT, dgiT, dhnT, WihT, WhhT, Wk, part, split, sup, dWs, dbs, total;
+  size_t g, dXb, dMb, dgiT, dhnT, WihT, WhhT, Wk, part, split, sup, dWs, dbs, total;
 };
 size_t tc_part_floats(const bg_plan* p, int H, int T) {
   const int64_t K = (int64_t)T * p->n_pad();
@@ -600,8 +599,8 @@ TcBwdWs tc_bwd_ws(const bg_plan* p, int H, int T) {
   TcBwdWs w{};
   size_t o = 0;
   w.g = o; o += al(sizeof(float) * n * H);
-  w.dXT = o; o += al(n * H * 2);
-  w.dMT = o; o += al((size_t)p->P * H * TN * 2);
+  w.dXb = o; o += al(n * H * 2);
+  w.dMb = o; o += al((size_t)p->P * H * TN * 2);
   w.dgiT = o; o += al((size_t)3 * H * TN * 2);
   w.dhnT = o; o += al((size_t)H * TN * 2);
   w.WihT = o; o += al((size_t)3 * H * H * 2);
@@ -745,7 +744,7 @@ static int propagate_bwd_impl(const bg_plan* p, bg_dtype dt, int H, const void* 
   if (ws_bytes < w.total) return bg_fail(BG_ECAPACITY, "workspace too small");
   BG_TRY(propagate_bwd_band(p, dt, H, E, W, dY, dE, dW, db, accum, ws, ws_bytes, st));
   // the supernode rows and columns (Section 6), added to the band's gradients
-  BG_CUDA(bg::super_bwd(p, bf, H, E, W, dY, nullptr, 0, dE, dW, db, ws + w.super, st));
+  BG_CUDA(bg::super_bwd(p, bf, H, E, W, dY, nullptr, dE, dW, db, ws + w.super, st));
   return BG_OK;
 }
 
@@ -767,7 +766,6 @@ static int propagate_bwd_band(const bg_plan* p, bg_dtype dt, int H, const void* 
     int* status = nullptr;
     BG_TRY(status_word_ptr(&status));
     auto* dMb = reinterpret_cast<__nv_bfloat16*>(ws + w.dMb);
-    auto* dMT = reinterpret_cast<__nv_bfloat16*>(ws + w.dMT);
     auto* Wp = reinterpret_cast<__nv_bfloat16*>(ws + w.Wp);
     auto* ETa = reinterpret_cast<__nv_bfloat16*>(ws + w.ETa);
     float* tpart = reinterpret_cast<float*>(ws + w.tpart);
@@ -783,10 +781,9 @@ static int propagate_bwd_band(const bg_plan* p, bg_dtype dt, int H, const void* 
     }
     KTimer t(BG_KID_DW, st);
     // dW_p, db_p from one split-K product of dM^T with E^T and the GEMM's appended ones row
-    BG_CUDA(bg::prep_transpose_bf16(dMb, 0, dMT, (int)n, PH, 1, st));
     BG_CUDA(bg::prep_transpose_bf16(E, 0, ETa, (int)n, H, 1, st));
-    BG_CUDA(bg::gemm_tn(dMT, (int64_t)n, ETa, (int64_t)n, PH, H, (int64_t)n, 1, dW, db, accum,
-                        tpart, tpf, status, st));
+    BG_CUDA(bg::gemm_tn(dMb, PH, 1, ETa, (int64_t)n, PH, H, (int64_t)n, 1, dW, db, accum, tpart, tpf,
+                        status, st));
     return BG_OK;
   }
   float* dM = reinterpret_cast<float*>(ws + w.dM);
@@ -912,8 +909,7 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
       if (addend) BG_CUDA(bg::super_fwd(p, 1, H, Ei(t), prm->W, prm->b, addend, 1, st));
       {
         KTimer tm(BG_KID_BAND_FWD, st);
-        BG_CUDA(bg::band_tc_fwd_core(p, H, ETa + (size_t)t * n, (int64_t)TN, WT,
-                                     prm->b ? b2T : nullptr, prm->b, nullptr, Yi(t),
+        BG_CUDA(bg::band_tc_fwd_core(p, H, Ei(t), WT, prm->b ? b2T : nullptr, prm->b, nullptr, Yi(t),
                                      YTa + (size_t)t * n, (int64_t)TN, split, addend, status, st));
       }
       KTimer tm(BG_KID_GRU_FWD, st);
@@ -961,8 +957,7 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
       if (addend) BG_CUDA(bg::super_fwd(p, 1, H, Et, prm->W, prm->b, addend, 1, st));
       {
         KTimer tm(BG_KID_BAND_FWD, st);
-        BG_CUDA(bg::band_tc_fwd_core(p, H, ETa + (size_t)t * n, (int64_t)TN, WT,
-                                     prm->b ? b2T : nullptr, prm->b, nullptr, Yb,
+        BG_CUDA(bg::band_tc_fwd_core(p, H, Et, WT, prm->b ? b2T : nullptr, prm->b, nullptr, Yb,
                                      YTa + (size_t)t * n, (int64_t)TN,
                                      bg::band_tc_split_floats(p, H) ? split : nullptr, addend,
                                      status, st));
@@ -1022,8 +1017,9 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     const __nv_bfloat16* ETa = reinterpret_cast<const __nv_bfloat16*>(sv + sl.ETa);
     const __nv_bfloat16* YTa = reinterpret_cast<const __nv_bfloat16*>(sv + sl.YTa);
     float* g = reinterpret_cast<float*>(wsc + wl.g);
-    __nv_bfloat16* dXT = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dXT);
-    __nv_bfloat16* dMT = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dMT);
+    __nv_bfloat16* dXb = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dXb);
+    __nv_bfloat16* dMb = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dMb);
+    const size_t PH = (size_t)p->P * H;
     __nv_bfloat16* dgiT = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dgiT);
     __nv_bfloat16* dhnT = reinterpret_cast<__nv_bfloat16*>(wsc + wl.dhnT);
     __nv_bfloat16* WihT = reinterpret_cast<__nv_bfloat16*>(wsc + wl.WihT);
@@ -1050,18 +1046,17 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
       {
         KTimer tm(BG_KID_GRU_BWD, st);
         BG_CUDA(bg::gru_bwd_tc(H, (int)n, p->n_real, Yi(t), Ei(t), Wih, Whh, WihT, WhhT, prm->b_ih,
-                               prm->b_hh, gin, g, dXT, (int64_t)n, dgiT + (size_t)t * n,
+                               prm->b_hh, gin, g, dXb, dgiT + (size_t)t * n,
                                dhnT + (size_t)t * n, (int64_t)TN, status, st));
       }
       {
         KTimer tm(BG_KID_BAND_BWD, st);
-        BG_CUDA(bg::band_tc_bwd_core(p, H, dXT, (int64_t)n, Wk, g, 1, dMT + (size_t)t * n,
-                                     (int64_t)TN, split, status, st));
+        BG_CUDA(bg::band_tc_bwd_core(p, H, dXb, Wk, g, 1, dMb + (size_t)t * n * PH, split,
+                                     status, st));
       }
       // the supernode rows and columns: dE(t) and their share of dW, db (summed over the steps)
       if (sup)
-        BG_CUDA(bg::super_bwd(p, 1, H, Ei(t), prm->W, nullptr, dXT, (int64_t)n, g, dWs, dbs,
-                              wsc + wl.sup, st, t < T - 1));
+        BG_CUDA(bg::super_bwd(p, 1, H, Ei(t), prm->W, nullptr, dXb, g, dWs, dbs, wsc + wl.sup, st, t < T - 1));
       gin = g;
     }
     const int acc = (flags & BG_ACCUM) ? 1 : 0;
@@ -1069,10 +1064,10 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     // dW_p, db_p over all steps and nodes; dW_ih, db_ih; dW_hh, db_hh, whose r and z rows take
     // the input-side gate gradients (equal to the hidden-side ones there) and n rows dh_n
     const bg::TNProblem probs[4] = {
-        {dMT, (int64_t)TN, ETa, (int64_t)TN, p->P * H, 1, gr->dW, gr->db},
-        {dgiT, (int64_t)TN, YTa, (int64_t)TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
-        {dgiT, (int64_t)TN, ETa, (int64_t)TN, 2 * H, 0, gr->dW_hh, gr->db_hh},
-        {dhnT, (int64_t)TN, ETa, (int64_t)TN, H, 0, gr->dW_hh + (size_t)2 * H * H,
+        {dMb, (int64_t)PH, 1, ETa, (int64_t)TN, p->P * H, 1, gr->dW, gr->db},
+        {dgiT, (int64_t)TN, 0, YTa, (int64_t)TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
+        {dgiT, (int64_t)TN, 0, ETa, (int64_t)TN, 2 * H, 0, gr->dW_hh, gr->db_hh},
+        {dhnT, (int64_t)TN, 0, ETa, (int64_t)TN, H, 0, gr->dW_hh + (size_t)2 * H * H,
          gr->db_hh + 2 * H}};
     BG_CUDA(bg::gemm_tn_multi(probs, 4, H, (int64_t)TN, acc, part, pf, status, st));
     if (sup) {
@@ -1114,8 +1109,8 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     auto* dghT = reinterpret_cast<__nv_bfloat16*>(wsc + w.dghT);
     auto* WihT = reinterpret_cast<__nv_bfloat16*>(wsc + w.WihT);
     auto* WhhT = reinterpret_cast<__nv_bfloat16*>(wsc + w.WhhT);
-    auto* dXT = reinterpret_cast<__nv_bfloat16*>(wsc + w.dXT);
-    auto* dMT = reinterpret_cast<__nv_bfloat16*>(wsc + w.dMT);
+    auto* dXb = reinterpret_cast<__nv_bfloat16*>(wsc + w.dXb);
+    auto* dMb = reinterpret_cast<__nv_bfloat16*>(wsc + w.dMb);
     void* Wk = wsc + w.Wk;
     float* tcpart = reinterpret_cast<float*>(wsc + w.tcpart);
     float* split = bg::band_tc_split_floats(p, H) ? reinterpret_cast<float*>(wsc + w.split)
@@ -1143,33 +1138,30 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
         BG_CUDA(bg::gru_bwd_gates_tc(H, n, p->n_real, Yt, Et, Wih, Whh, prm->b_ih, prm->b_hh, gin,
                                      gout, dgib, dghb, dgiT + (size_t)t * nn,
                                      dghT + (size_t)t * nn, (int64_t)TN, status, st));
-        BG_CUDA(bg::gemm_bf16_tn_outT(dgib, 3 * H, WihT, 3 * H, n, H, 3 * H, dXT, (int64_t)nn,
-                                      status, st));
+        BG_CUDA(bg::gemm_bf16_tn_outb(dgib, 3 * H, WihT, 3 * H, n, H, 3 * H, dXb, H, status, st));
         BG_CUDA(bg::gemm_bf16_tn(dghb, 3 * H, 0, WhhT, 3 * H, 0, n, H, 3 * H, 1, gout, H, 0,
                                  nullptr, 0, 1, status, st));
       }
       {
         KTimer tm(BG_KID_BAND_BWD, st);
-        BG_CUDA(bg::band_tc_bwd_core(p, H, dXT, (int64_t)nn, Wk, gout, 1, dMT, (int64_t)nn, split,
-                                     status, st));
+        BG_CUDA(bg::band_tc_bwd_core(p, H, dXb, Wk, gout, 1, dMb, split, status, st));
       }
       {
         KTimer tm(BG_KID_DW, st);
-        BG_CUDA(bg::gemm_tn(dMT, (int64_t)nn, ETa + (size_t)t * nn, (int64_t)TN, p->P * H, H,
-                            (int64_t)nn, 1, gr->dW, gr->db, t == T - 1 ? acc : 1, tcpart,
+        BG_CUDA(bg::gemm_tn(dMb, (int64_t)p->P * H, 1, ETa + (size_t)t * nn, (int64_t)TN,
+                            p->P * H, H, (int64_t)nn, 1, gr->dW, gr->db, t == T - 1 ? acc : 1, tcpart,
                             tc_part_floats(p, H, T), status, st));
       }
       // the supernode rows and columns: dE(t) and their share of dW, db (summed over the steps)
       if (sup)
-        BG_CUDA(bg::super_bwd(p, 1, H, Et, prm->W, nullptr, dXT, (int64_t)nn, gout, dWs, dbs,
-                              wsc + w.sup, st, t < T - 1));
+        BG_CUDA(bg::super_bwd(p, 1, H, Et, prm->W, nullptr, dXb, gout, dWs, dbs, wsc + w.sup, st, t < T - 1));
       gin = gout;
       gout = gout == dX ? g : dX;
     }
     KTimer tm(BG_KID_DW, st);
     const bg::TNProblem probs[2] = {
-        {dgiT, (int64_t)TN, YTa, (int64_t)TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
-        {dghT, (int64_t)TN, ETa, (int64_t)TN, 3 * H, 0, gr->dW_hh, gr->db_hh}};
+        {dgiT, (int64_t)TN, 0, YTa, (int64_t)TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
+        {dghT, (int64_t)TN, 0, ETa, (int64_t)TN, 3 * H, 0, gr->dW_hh, gr->db_hh}};
     BG_CUDA(bg::gemm_tn_multi(probs, 2, H, (int64_t)TN, acc, tcpart, tc_part_floats(p, H, T),
                               status, st));
     if (sup) {
@@ -1266,8 +1258,8 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     // GEMM appends the ones column)
     KTimer tm(BG_KID_DW, st);
     const bg::TNProblem probs[2] = {
-        {dgiT, TN, YTa, TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
-        {dghT, TN, ETa, TN, 3 * H, 0, gr->dW_hh, gr->db_hh}};
+        {dgiT, TN, 0, YTa, TN, 3 * H, 0, gr->dW_ih, gr->db_ih},
+        {dghT, TN, 0, ETa, TN, 3 * H, 0, gr->dW_hh, gr->db_hh}};
     BG_CUDA(bg::gemm_tn_multi(probs, 2, H, TN, 1, reinterpret_cast<float*>(wsc + w.tpart),
                               gru_tpart_floats(p, H, T), status, st));
   }

@@ -9,7 +9,7 @@
 // 256, where bf16 integers stop being exact).  pre_p never leaves the SM.
 // Backward (transposed band): the same kernel with the transposed tiles, dY instead of E and W_p
 // instead of W_p^T gives dE_j += sum_p (A^T dY)_p W_p^T; dM_p = A_p^T dY is also written (bf16,
-// transposed) for the weight gradient.
+// [n][P H]) for the weight gradient.
 //
 // The second product runs as kind::tf32 straight from the fp32 pre_p (W_p staged as fp32), so no
 // thread touches pre_p between the two products and no MMA issuer waits on a conversion.  The
@@ -61,7 +61,6 @@ using namespace tc;
 namespace {
 
 constexpr int kTile = 128;     // rows per tile = UMMA M
-constexpr int kAtom = 64;      // bf16 per 128-byte swizzle row
 
 // Block size S: a 128-row tile sees a window of C1 128-column chunks of the state (and of its
 // bit tiles): rows [row0, row0 + 128) only couple to columns in block-rows kr - 1 .. kr + 1 of
@@ -82,8 +81,9 @@ struct Cfg {
   static constexpr bool GM = S == 512 && SW == 64;
   static constexpr int NH = H / SW;
   static constexpr int C1 = band_chunks(S);                   // 128-column chunks per type
-  static constexpr int ATOM_X = SW * 128;                     // 64 nodes x SW state columns
-  static constexpr int XWIN = 2 * C1 * ATOM_X;                // one half's window, 64-node atoms
+  static constexpr int XROW = SW * 2;                         // bytes of one node's slice
+  static constexpr int XCHUNK = 128 * XROW;                   // 128 nodes x SW state columns
+  static constexpr int XWIN = C1 * XCHUNK;                    // one half's window
   static constexpr int NXB = XWIN <= 48 * 1024 ? 2 : 1;       // state-window buffers
   // W ring stages: at H <= 64, S <= 128 the small window leaves room for a deeper ring (the second
   // issuer's W stages come from L2, and it gates the release of the pre_p units); measured best
@@ -96,8 +96,11 @@ struct Cfg {
   static constexpr int WJ = SW / WK;                          // stages per job
   static constexpr int WSTAGE = (WK / 32) * H * 128;
   static constexpr int DEG = kTile * 128;                     // 128 rows x 64 bf16
-  static constexpr int NDEG = GM ? 0 : (NH > 1 ? 1 : 2);      // deg buffers
-  static constexpr int B2 = GM ? 0 : H * 128;                 // H rows x 64 bf16
+  // forward: deg buffers and H rows x 64 bf16 of bias; backward: the dM_p staging tile instead
+  static constexpr int NDEG = (GM || BWD) ? 0 : (NH > 1 ? 1 : 2);
+  static constexpr int B2 = (GM || BWD) ? 0 : H * 128;
+  static constexpr bool DMS = BWD && !(GM && H > 64);         // (no room for it at H = 128, S = 512)
+  static constexpr int DM = DMS ? kTile * SW * 2 : 0;
   static constexpr int OFF_X = 0;
   static constexpr int OFF_W = OFF_X + NXB * XWIN;
   static constexpr int OFF_DEG = OFF_W + NW * WSTAGE;
@@ -108,7 +111,8 @@ struct Cfg {
   static constexpr int NM = GM ? 0 : (C1 > 6 ? 2 : (NM0 > 2 ? NM0 : 2));
   // ring sizes as divisors (the GM shapes have no deg or mask ring; their code paths are off)
   static constexpr int NDEGD = NDEG > 0 ? NDEG : 1, NMD = NM > 0 ? NM : 1;
-  static constexpr int OFF_M = OFF_B2 + B2;
+  static constexpr int OFF_DM = OFF_B2 + B2;
+  static constexpr int OFF_M = OFF_DM + DM;
   static constexpr int OFF_BAR = OFF_M + NM * MSTAGE;
   static constexpr int SMEM = OFF_BAR + 1024 + 1024;          // barriers + 1 KB alignment slack
   // TMEM columns: Y (H), two 64-column pre_p units used by the jobs (half, type) in turn, so that
@@ -225,9 +229,10 @@ template <int H, int S, bool BWD>
 __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
     k_band_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
               const __grid_constant__ CUtensorMap tm_deg, const __grid_constant__ CUtensorMap tm_b2,
-              const uint32_t* __restrict__ maskI, float* __restrict__ out,
-              __nv_bfloat16* __restrict__ outb, __nv_bfloat16* __restrict__ outT, int64_t ld_outT,
-              __nv_bfloat16* __restrict__ dMT, int64_t ld_mt, const Sched sc, int P, int has_bias,
+              const __grid_constant__ CUtensorMap tm_dm, const uint32_t* __restrict__ maskI,
+              float* __restrict__ out, __nv_bfloat16* __restrict__ outb,
+              __nv_bfloat16* __restrict__ outT, int64_t ld_outT, __nv_bfloat16* __restrict__ dM,
+              const Sched sc, int P, int has_bias,
               int bias_f16, int accumulate, int* status) {
   using C = Cfg<H, S, BWD>;
   extern __shared__ uint8_t smem_raw[];
@@ -325,9 +330,9 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
           ++n_x[xb];
           ++xi;
           mbar_expect_tx(&bars->x_full[xb], C::XWIN);
-          for (int a = 0; a < 2 * C::C1; ++a)
-            tma_load_2d(xwin + xb * C::XWIN + a * C::ATOM_X, &tm_x, &bars->x_full[xb],
-                        ws + a * kAtom, C::SW * hh);
+          for (int a = 0; a < C::C1; ++a)
+            tma_load_2d(xwin + xb * C::XWIN + a * C::XCHUNK, &tm_x, &bars->x_full[xb], C::SW * hh,
+                        ws + a * 128);
         }
         // per job: K-columns SW hh .. of W_p^T in WJ stages of WK / 32 atoms
         {
@@ -389,7 +394,8 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
     // pre_p = sum over the window chunks of A_{tile,p,j} X_j (N = SW): one t_full wait per group
     // of chunks, then an unbroken MMA stream
     const bool leader = elect_one_sync();
-    constexpr uint32_t idesc = idesc_bf16_f32(kTile, C::SW);
+    // B is the window itself, row-major: N = SW columns contiguous, one row per K index
+    constexpr uint32_t idesc = idesc_bf16_f32(kTile, C::SW) | kIdescBMN;
     uint32_t c = 0, slot = 0, gi = 0, xi = 0;
     // expander group of chunk x + NA (the next user of the slot chunk x frees): job (x + NA) / C1
     // mod 2, kept as a group and a position within the job
@@ -405,7 +411,8 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
         if (!mbar_wait(&bars->x_full[xb], (xi / C::NXB) & 1, status, 204, abort)) { ok = false; break; }
         ++xi;
         // descriptors differ from the window's first one only in the start-address field
-        const uint64_t xdesc = desc_sw128_kmajor(smem_u32(xwin + xb * C::XWIN));
+        const uint32_t xaddr = smem_u32(xwin + xb * C::XWIN);
+        const uint64_t xdesc = C::SW == 64 ? desc_sw128_mnmajor(xaddr, 1024) : desc_sw64_mnmajor(xaddr);
         for (; jb < seg_end && ok; ++jb, ++c) {
           const uint32_t d1 = tmem + C::D1COL0 + (c % C::NB) * 64;
           for (int g = 0; g < C::G; ++g, ++gi) {
@@ -413,14 +420,14 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
             tc_fence_after();
             for (int j = g * C::CG; j < (g + 1) * C::CG; ++j) {
               const uint32_t a = tmem + C::ACOL + slot * 64;
-              const uint64_t jdesc = xdesc + (uint64_t)((2 * j * C::ATOM_X) >> 4);
+              const uint64_t jdesc = xdesc + (uint64_t)((j * C::XCHUNK) >> 4);
               // S = 32: the tile's rows couple to window columns [0, 192) only, so the last four
               // K steps of the second chunk would multiply all-zero A tiles
               const int kk_end = (S == 32 && j == C::C1 - 1) ? 4 : kTile / 16;
 #pragma unroll
               for (int kk = 0; kk < kTile / 16; ++kk)
                 if (leader && kk < kk_end)
-                  mma_ts(d1, a + kk * 8, jdesc + (uint64_t)(((kk / 4) * C::ATOM_X + (kk % 4) * 32) >> 4),
+                  mma_ts(d1, a + kk * 8, jdesc + (uint64_t)((kk * 16 * C::XROW) >> 4),
                          idesc, (j == 0 && kk == 0) ? 0u : 1u);
               if (leader) tc_commit(&bars->a_empty[slot][nx_g]);
               slot = slot + 1 == (uint32_t)C::NA ? 0 : slot + 1;
@@ -589,6 +596,7 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
     grid_dep_wait();  // outputs (and the accumulated dE) may still be in use by the previous kernel
     const int r = threadIdx.x - 128 * (1 + C::NE);
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    uint8_t* dms = smem + C::OFF_DM + (warp & 3) * 32 * C::XROW;
     uint32_t c = 0;
     int i = 0;
     for (int w = blockIdx.x; w < sc.n_items && !*abort; w += gridDim.x, ++i) {
@@ -614,17 +622,27 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 #pragma unroll
         for (int j = 0; j < C::SW / 2; ++j)
           pk[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-        // dM_p (bf16) transposed, dMT[(p*H + h) * ld_mt + row], as 4-byte words of two rows: a
-        // lane pair swaps its packed (h, h + 1) pairs, then the even lane stores column h of rows
-        // (row, row + 1) and the odd lane column h + 1 of rows (row - 1, row)
-        const bool odd = lane & 1;
+        if constexpr (!C::DMS) {
+          uint4* d = reinterpret_cast<uint4*>(dM + ((size_t)row * P + p) * H + C::SW * hh);
 #pragma unroll
-        for (int j = 0; j < C::SW / 2; ++j) {
-          const uint32_t other = __shfl_xor_sync(0xffffffffu, pk[j], 1);
-          const uint32_t word = odd ? __byte_perm(other, pk[j], 0x7632) : __byte_perm(pk[j], other, 0x5410);
-          *reinterpret_cast<uint32_t*>(dMT + ((size_t)p * H + C::SW * hh + 2 * j + odd) * ld_mt +
-                                       (row & ~1)) = word;
+          for (int j = 0; j < C::SW / 8; ++j)
+            d[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+          continue;
         }
+        // dM_p (bf16, row-major) through this warp's 32-row staging tile, one bulk store per job
+        // (a thread's own row as 16-byte global stores would touch 32 lines per instruction)
+        if (lane == 0) tma_store_wait_read<0>();  // the previous job's copy has left the tile
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < C::SW / 8; ++j) {
+          const int sw = C::SW == 64 ? (j ^ (lane & 7)) : (j ^ ((lane >> 1) & 3));
+          *reinterpret_cast<uint4*>(dms + lane * C::XROW + sw * 16) =
+              make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0)
+          tma_store_2d(&tm_dm, dms, p * H + C::SW * hh, k * kTile + (warp & 3) * 32);
       }
       if (!ok) break;
       if (!mbar_wait(&bars->y_full, i & 1, status, 402, abort, 64)) break;
@@ -712,6 +730,7 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
         }
       }
     }
+    if (BWD && lane == 0) tma_store_wait_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -897,9 +916,9 @@ Sched make_sched(int n_tiles, int jobs, int sms, bool can_split) {
 
 template <int H, int S, bool BWD>
 cudaError_t launch_s(const bg_plan* p, const CUtensorMap& tx, const CUtensorMap& tw,
-                     const CUtensorMap& tdeg, const CUtensorMap& tb2, float* out,
-                     __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
-                     __nv_bfloat16* dMT, int64_t ld_mt, int has_bias, int accumulate,
+                     const CUtensorMap& tdeg, const CUtensorMap& tb2, const CUtensorMap& tdm,
+                     float* out, __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
+                     __nv_bfloat16* dM, int has_bias, int accumulate,
                      float* split, const float* addend, const float* b32, int* status,
                      cudaStream_t st) {
   using C = Cfg<H, S, BWD>;
@@ -916,7 +935,7 @@ cudaError_t launch_s(const bg_plan* p, const CUtensorMap& tx, const CUtensorMap&
   sc.bias_f16 = p->max_deg > 256 ? 1 : 0;
   const int grid = std::min(sc.n_items, sms);
   e = launch_pdl(k_band_tc<H, S, BWD>, dim3(grid), dim3(C::THREADS), C::SMEM, st, tx, tw, tdeg,
-                 tb2, BWD ? p->d_maskTI : p->d_maskI, out, outb, outT, ld_outT, dMT, ld_mt, sc,
+                 tb2, tdm, BWD ? p->d_maskTI : p->d_maskI, out, outb, outT, ld_outT, dM, sc,
                  p->P, has_bias, p->max_deg > 256 ? 1 : 0, accumulate, status);
   note_launch();
   if (e != cudaSuccess || sc.ksplit == 1) return e;
@@ -932,13 +951,13 @@ cudaError_t launch_s(const bg_plan* p, const CUtensorMap& tx, const CUtensorMap&
 // at S in {32, 64, 128} (its state-slice window at S = 256 leaves no room for the mask ring).
 template <int H, bool BWD>
 cudaError_t launch(const bg_plan* p, const CUtensorMap& tx, const CUtensorMap& tw,
-                   const CUtensorMap& tdeg, const CUtensorMap& tb2, float* out,
-                   __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
-                   __nv_bfloat16* dMT, int64_t ld_mt, int has_bias, int accumulate, float* split,
+                   const CUtensorMap& tdeg, const CUtensorMap& tb2, const CUtensorMap& tdm,
+                   float* out, __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
+                   __nv_bfloat16* dM, int has_bias, int accumulate, float* split,
                    const float* addend, const float* b32, int* status, cudaStream_t st) {
 #define BG_BAND_S(SV)                                                                            \
-  return launch_s<H, SV, BWD>(p, tx, tw, tdeg, tb2, out, outb, outT, ld_outT, dMT, ld_mt,      \
-                              has_bias, accumulate, split, addend, b32, status, st);
+  return launch_s<H, SV, BWD>(p, tx, tw, tdeg, tb2, tdm, out, outb, outT, ld_outT, dM, has_bias, \
+                              accumulate, split, addend, b32, status, st);
   switch (p->S) {
     case 32: BG_BAND_S(32)
     case 64: BG_BAND_S(64)
@@ -984,6 +1003,21 @@ bool make_map_ld(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols,
   return r == CUDA_SUCCESS;
 }
 
+bool make_map_box(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
+                  uint32_t box_cols, uint32_t box_rows) {
+  auto fn = encode_fn();
+  if (!fn || (box_cols != 64 && box_cols != 32)) return false;
+  cuuint64_t dims[2] = {cols, rows};
+  cuuint64_t strides[1] = {ld * 2};
+  cuuint32_t box[2] = {box_cols, box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
+                  box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 int gemm_tn_num_sms() { return num_sms(); }
 
 bool make_map_3d(CUtensorMap* m, const void* base, uint64_t batch, uint64_t rows, uint64_t cols,
@@ -1023,6 +1057,8 @@ cudaError_t band_tc_prep_w(const bg_plan* p, int H, const void* W, int bwd, void
   return cudaGetLastError();
 }
 
+// (The first n H bf16 elements are not used; the size is what callers have always been asked for,
+// and what the allocation-free entry point's limit is checked against.)
 size_t band_tc_fwd_ws_bytes(const bg_plan* p, int dtype, int H) {
   if (!p || dtype != 1) return 0;
   const size_t n = (size_t)p->n_pad();
@@ -1044,20 +1080,20 @@ size_t band_tc_split_floats(const bg_plan* p, int H) {
   return sc.ksplit > 1 ? (size_t)sc.ksplit * sc.part_rows * H : 0;
 }
 
-cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* XT, int64_t ld_x,
-                             const void* Wk, const __nv_bfloat16* b2T, const float* b32,
-                             float* out, __nv_bfloat16* outb, __nv_bfloat16* outT,
-                             int64_t ld_outT, float* split, const float* addend, int* status,
+cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, const void* Wk,
+                             const __nv_bfloat16* b2T, const float* b32, float* out,
+                             __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
+                             float* split, const float* addend, int* status,
                              cudaStream_t st) {
   const int n = p->n_pad(), P = p->P;
   CUtensorMap tx, tw, tdeg, tb2;
-  if (!make_map_ld(&tx, XT, H, n, ld_x, H < 64 ? 32 : 64) ||
+  if (!make_map_box(&tx, X, n, H, H, H < 64 ? 32 : 64, kTile) ||
       !make_map_w(&tw, Wk, P, H) || !make_map(&tdeg, p->d_deg2, n, 64, kTile) ||
-      !make_map(&tb2, b2T ? b2T : XT, H, 64, H))
+      !make_map(&tb2, b2T ? b2T : X, H, 64, H))
     return cudaErrorInvalidValue;
   const int hb = b2T != nullptr;
 #define BG_FWD(HV)                                                                                \
-  return launch<HV, false>(p, tx, tw, tdeg, tb2, out, outb, outT, ld_outT, nullptr, 0, hb, 0,     \
+  return launch<HV, false>(p, tx, tw, tdeg, tb2, tw, out, outb, outT, ld_outT, nullptr, hb, 0,    \
                            split, addend, b32, status, st);
   switch (H) {
     case 32: BG_FWD(32)
@@ -1068,16 +1104,17 @@ cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* XT, i
 #undef BG_FWD
 }
 
-cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dYT, int64_t ld_y,
-                             const void* Wk, float* dE, int accumulate, __nv_bfloat16* dMT,
-                             int64_t ld_mt, float* split, int* status, cudaStream_t st) {
+cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, const void* Wk,
+                             float* dE, int accumulate, __nv_bfloat16* dM, float* split,
+                             int* status, cudaStream_t st) {
   const int n = p->n_pad(), P = p->P;
-  CUtensorMap tx, tw;
-  if (!make_map_ld(&tx, dYT, H, n, ld_y, H < 64 ? 32 : 64) ||
-      !make_map_w(&tw, Wk, P, H))
+  CUtensorMap tx, tw, tdm;
+  const int sw = H < 64 ? 32 : 64;
+  if (!make_map_box(&tx, dY, n, H, H, sw, kTile) || !make_map_w(&tw, Wk, P, H) ||
+      !make_map_box(&tdm, dM, n, (uint64_t)P * H, (uint64_t)P * H, sw, 32))
     return cudaErrorInvalidValue;
 #define BG_BWD(HV)                                                                                \
-  return launch<HV, true>(p, tx, tw, tw, tw, dE, nullptr, nullptr, 0, dMT, ld_mt, 0, accumulate,  \
+  return launch<HV, true>(p, tx, tw, tw, tw, tdm, dE, nullptr, nullptr, 0, dM, 0, accumulate,     \
                           split, nullptr, nullptr, status, st);
   switch (H) {
     case 32: BG_BWD(32)
@@ -1115,20 +1152,18 @@ cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, c
                         float* Y, char* ws, size_t ws_bytes, int* status, cudaStream_t st) {
   if (ws_bytes < band_tc_fwd_ws_bytes(p, 1, H)) return cudaErrorInvalidValue;
   const int n = p->n_pad();
-  __nv_bfloat16* ET = reinterpret_cast<__nv_bfloat16*>(ws);
   void* WT = ws + al256((size_t)n * H * 2);
   __nv_bfloat16* b2T = reinterpret_cast<__nv_bfloat16*>(ws + al256((size_t)n * H * 2) +
                                                         band_tc_w_bytes(p, H));
   float* split = reinterpret_cast<float*>(ws + al256((size_t)n * H * 2) + band_tc_w_bytes(p, H) +
                                           al256((size_t)H * 64 * 2));
-  // E [n][H] -> ET [H][n];  W_p [H_in][H_out] -> W_p^T in the kernel's operand type;  bias split
-  cudaError_t e = prep_transpose_bf16(E, 0, ET, n, H, 1, st);
-  if (e == cudaSuccess) e = band_tc_prep_w(p, H, W, 0, WT, st);
+  // W_p [H_in][H_out] -> W_p^T in the kernel's operand type;  bias split
+  cudaError_t e = band_tc_prep_w(p, H, W, 0, WT, st);
   if (e == cudaSuccess && b) e = prep_bias_split(p, b, b2T, H, status, st);
   if (e != cudaSuccess) return e;
   ProfSpan span(BG_KID_BAND_FWD, st);
-  return band_tc_fwd_core(p, H, ET, n, WT, b ? b2T : nullptr, b, Y, nullptr, nullptr, 0,
-                          band_tc_split_floats(p, H) ? split : nullptr, nullptr, status, st);
+  return band_tc_fwd_core(p, H, static_cast<const __nv_bfloat16*>(E), WT, b ? b2T : nullptr, b, Y,
+                          nullptr, nullptr, 0, band_tc_split_floats(p, H) ? split : nullptr, nullptr, status, st);
 }
 
 cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, const float* dY,
@@ -1137,9 +1172,9 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
   if (ws_bytes < band_tc_bwd_ws_bytes(p, 1, H)) return cudaErrorInvalidValue;
   const int n = p->n_pad(), P = p->P;
   size_t o = 0;
-  __nv_bfloat16* dYT = reinterpret_cast<__nv_bfloat16*>(ws + o);
+  __nv_bfloat16* dYb = reinterpret_cast<__nv_bfloat16*>(ws + o);
   o += al256((size_t)n * H * 2);
-  __nv_bfloat16* dMT = reinterpret_cast<__nv_bfloat16*>(ws + o);
+  __nv_bfloat16* dM = reinterpret_cast<__nv_bfloat16*>(ws + o);
   o += al256((size_t)P * H * n * 2);
   __nv_bfloat16* ETa = reinterpret_cast<__nv_bfloat16*>(ws + o);
   o += al256((size_t)(H + 16) * n * 2);
@@ -1149,11 +1184,11 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
   const size_t part_floats = gemm_tn_part_floats(P * H, H + 16, (int64_t)n);
   o += al256(sizeof(float) * part_floats);
   float* split = band_tc_split_floats(p, H) ? reinterpret_cast<float*>(ws + o) : nullptr;
-  cudaError_t e = prep_transpose_bf16(dY, 1, dYT, n, H, 1, st);
+  cudaError_t e = f32_to_bf16(dY, dYb, (int64_t)n * H, st);
   if (e == cudaSuccess) e = band_tc_prep_w(p, H, W, 1, Wk, st);
   if (e == cudaSuccess) {
     ProfSpan span(BG_KID_BAND_BWD, st);
-    e = band_tc_bwd_core(p, H, dYT, n, Wk, dE, accum, dMT, n, split, status, st);
+    e = band_tc_bwd_core(p, H, dYb, Wk, dE, accum, dM, split, status, st);
   }
   if (e != cudaSuccess) return e;
   // E^T; the weight-gradient product appends its ones row, which turns the bias gradient into
@@ -1162,7 +1197,8 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
   if (e != cudaSuccess) return e;
   // dW_p[h][h'] (+)= sum_nodes E[node][h] dM_p[node][h'],  db_p[h'] (+)= sum_nodes dM_p[node][h']
   ProfSpan span(BG_KID_DW, st);
-  return gemm_tn(dMT, n, ETa, n, P * H, H, n, 1, dW, db, accum, part, part_floats, status, st);
+  return gemm_tn(dM, (int64_t)P * H, 1, ETa, n, P * H, H, n, 1, dW, db, accum, part, part_floats,
+                 status, st);
 }
 
 int band_tc_upload(bg_plan* p, cudaStream_t st) {
@@ -1191,7 +1227,6 @@ cudaError_t band_tc_preload_fwd(const bg_plan* p) {
   cudaFuncAttributes a;
   cudaError_t e = cudaSuccess;
   auto take = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  take(cudaFuncGetAttributes(&a, k_transpose_bf16<__nv_bfloat16>));
   take(cudaFuncGetAttributes(&a, k_prep_w));
   take(cudaFuncGetAttributes(&a, k_bias_split));
   take(cudaFuncGetAttributes(&a, k_band_split_fixup));

@@ -25,7 +25,7 @@ size_t band_tc_w_bytes(const bg_plan* p, int H);
 cudaError_t band_tc_prep_w(const bg_plan* p, int H, const void* W, int bwd, void* Wk,
                            cudaStream_t st);
 // Kernel-level entry points used by the fused GGNN steps (operands already in kernel layout):
-//   XT: [H][>= n_pad] bf16 transposed states (row stride ld_x); Wk: band_tc_prep_w(bwd = 0);
+//   X: [n_pad][H] bf16 states; Wk: band_tc_prep_w(bwd = 0);
 //   b2T: [H][64] bf16 bias split or NULL.  Outputs (each optional): out fp32 [n][H],
 //   outb bf16 [n][H], outT bf16 [H][ld_outT].
 //   split: fp32 scratch of band_tc_split_floats(p, H) floats (may be NULL: no tile splitting) for
@@ -35,15 +35,16 @@ cudaError_t band_tc_prep_w(const bg_plan* p, int H, const void* W, int bwd, void
 size_t band_tc_split_floats(const bg_plan* p, int H);
 //   b32: the fp32 bias [P][H] (or NULL) beside its split b2T; the S = 512 kernels at 64-column
 //   slices add the bias in their epilogue from it.
-cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* XT, int64_t ld_x,
-                             const void* Wk, const __nv_bfloat16* b2T, const float* b32,
-                             float* out, __nv_bfloat16* outb, __nv_bfloat16* outT,
-                             int64_t ld_outT, float* split, const float* addend, int* status,
+cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, const void* Wk,
+                             const __nv_bfloat16* b2T, const float* b32, float* out,
+                             __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
+                             float* split, const float* addend, int* status,
                              cudaStream_t st);
-//   dYT: [H][>= n_pad] bf16; Wk: band_tc_prep_w(bwd = 1); dE fp32 (+)=; dMT: [P*H][ld_mt] bf16.
-cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dYT, int64_t ld_y,
-                             const void* Wk, float* dE, int accumulate, __nv_bfloat16* dMT,
-                             int64_t ld_mt, float* split, int* status, cudaStream_t st);
+//   dY: [n_pad][H] bf16; Wk: band_tc_prep_w(bwd = 1); dE fp32 (+)=; dM: [n_pad][P*H] bf16, 16-byte
+//   aligned.
+cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, const void* Wk,
+                             float* dE, int accumulate, __nv_bfloat16* dM, float* split,
+                             int* status, cudaStream_t st);
 // out[c * ld_out + r] = bf16(in[r][c]) for `batch` consecutive R x Cc matrices (in fp32 or bf16;
 // ld_out <= 0 means R; batches are R*Cc apart on both sides).
 cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* out, int R, int Cc,

@@ -69,6 +69,7 @@ struct TNGroups {
   int it_end[kMaxGroups];  // cumulative work-item counts
   int M[kMaxGroups];
   int prow[kMaxGroups];
+  int a_mn[kMaxGroups];    // A stored [K][M] (MN-major operand) instead of [M][K]
 };
 
 template <int BN>
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(192, 1)
   const int ntiles = min(C::MT, (M + 127) / 128 - mt0);    // 1 .. MT
   const CUtensorMap* tmA = &grp.a[g];
   const CUtensorMap* tmB = &grp.b[g];
+  const bool a_mn = grp.a_mn[g] != 0;
   const int kc0 = split * per_split;
   const int kc1 = min(kchunks, kc0 + per_split);
   // the last 16 rows of every stage's B: row Hout all bf16 ones, the rest zeros (128 bytes a row;
@@ -134,8 +136,15 @@ __global__ void __launch_bounds__(192, 1)
       ++issued[s];
       mbar_expect_tx(&full[s], ntiles * C::A_BYTES + C::BROWS * 128);
       uint8_t* st = smem + s * C::STAGE;
-      for (int m = 0; m < ntiles; ++m)
-        tma_load_2d(st + m * C::A_BYTES, tmA, &full[s], kc * 64, (mt0 + m) * 128);
+      for (int m = 0; m < ntiles; ++m) {
+        if (a_mn) {
+          // 64 K rows of 128 M elements, as two blocks of 64 (one swizzle row each)
+          tma_load_2d(st + m * C::A_BYTES, tmA, &full[s], (mt0 + m) * 128, kc * 64);
+          tma_load_2d(st + m * C::A_BYTES + 8192, tmA, &full[s], (mt0 + m) * 128 + 64, kc * 64);
+        } else {
+          tma_load_2d(st + m * C::A_BYTES, tmA, &full[s], kc * 64, (mt0 + m) * 128);
+        }
+      }
       tma_load_2d(st + C::MT * C::A_BYTES, tmB, &full[s], kc * 64, blockIdx.y * BN);
     }
     if (*abort)
@@ -145,8 +154,9 @@ __global__ void __launch_bounds__(192, 1)
   } else if (warp == 1) {
     // the whole warp runs the loop (uniform operands); one elected lane issues
     const bool leader = elect_one_sync();
-    constexpr uint32_t idesc = idesc_bf16_f32(128, C::N1);
-    constexpr uint32_t idesc2 = idesc_bf16_f32(128, BN > 256 ? BN - 256 : 16);
+    const uint32_t mn = a_mn ? kIdescAMN : 0u;
+    const uint32_t idesc = idesc_bf16_f32(128, C::N1) | mn;
+    const uint32_t idesc2 = idesc_bf16_f32(128, BN > 256 ? BN - 256 : 16) | mn;
     for (int kc = kc0, it = 0; kc < kc1; ++kc, ++it) {
       const int s = it % C::STAGES;
       if (!mbar_wait(&full[s], (it / C::STAGES) & 1, status, 502, abort)) break;
@@ -158,7 +168,8 @@ __global__ void __launch_bounds__(192, 1)
           const uint32_t acc = (kc > kc0 || kk > 0) ? 1u : 0u;
           const uint64_t bd = desc_sw128_kmajor(b + kk * 32);
           for (int m = 0; m < ntiles; ++m) {
-            const uint64_t ad = desc_sw128_kmajor(a + m * C::A_BYTES + kk * 32);
+            const uint64_t ad = a_mn ? desc_sw128_mnmajor(a + m * C::A_BYTES + kk * 2048, 8192)
+                                     : desc_sw128_kmajor(a + m * C::A_BYTES + kk * 32);
             mma_ss(tmem + m * C::TCOLS, ad, bd, idesc, acc);
             if (BN > 256)
               mma_ss(tmem + m * C::TCOLS + 256, ad, desc_sw128_kmajor(b + 256 * 128 + kk * 32),
@@ -283,10 +294,10 @@ struct BatchArgs {
   int64_t sBias;
   int accumulate;
   int vec;  // C rows (and bias) 16-byte aligned: each thread stores its row as float4
-  // instead of C: the product rounded to bf16 and stored transposed, CT[n * ldT + m] (batch 1,
-  // no bias, no accumulation; M even, N a multiple of 32, ldT even)
-  __nv_bfloat16* CT;
-  int64_t ldT;
+  // instead of C: the product rounded to bf16, Cb[m * ldb16 + n] (batch 1, no bias, no
+  // accumulation; N a multiple of 32, ldb16 of 8)
+  __nv_bfloat16* Cb;
+  int64_t ldb16;
 };
 
 template <int BN>
@@ -361,14 +372,12 @@ __global__ void __launch_bounds__(192, 2)
     __syncwarp();
     for (uint32_t t = 0; t < (1u << 24) && !mbar_try(drain, 0); ++t) {
     }
-  } else if (warp >= 2 && g.CT) {
-    // thread = row m, 32 consecutive columns per round; a lane pair (rows m, m + 1) swaps its
-    // packed column pairs so that each lane stores 4-byte words of two rows of one column
+  } else if (warp >= 2 && g.Cb) {
+    // thread = row m, 32 consecutive columns per round, rounded and stored as 4 x 16 bytes
     const int q = warp & 3;
     if (mbar_wait(done, 0, status, 513, abort, 128)) {
       tc_fence_after();
       const int m = mt * 128 + q * 32 + lane;
-      const bool odd = lane & 1;
 #pragma unroll 1
       for (int c0 = 0; c0 < BN; c0 += 32) {
         const int n0 = nt * BN + c0;
@@ -377,16 +386,17 @@ __global__ void __launch_bounds__(192, 2)
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + c0, v);
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + c0 + 16, v + 16);
         tmem_wait_ld();
-        __nv_bfloat16* base = g.CT + (size_t)(n0 + odd) * g.ldT + (m & ~1);
-        const bool live = (m & ~1) < g.M;
+        if (m >= g.M) continue;
+        uint32_t pk[16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-          const uint32_t pk = *reinterpret_cast<uint32_t*>(&h2);
-          const uint32_t other = __shfl_xor_sync(0xffffffffu, pk, 1);
-          const uint32_t word = odd ? __byte_perm(other, pk, 0x7632) : __byte_perm(pk, other, 0x5410);
-          if (live) *reinterpret_cast<uint32_t*>(base + (size_t)(2 * j) * g.ldT) = word;
+          pk[j] = *reinterpret_cast<uint32_t*>(&h2);
         }
+        uint4* dst = reinterpret_cast<uint4*>(g.Cb + (size_t)m * g.ldb16 + n0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
       }
     }
   } else if (warp >= 2 && g.vec) {
@@ -484,7 +494,7 @@ namespace {
 cudaError_t gemm_bf16_tn_any(const void* A, int64_t lda, int64_t sA, const void* B, int64_t ldb,
                              int64_t sB, int M, int N, int K, int batch, float* Cout, int64_t ldc,
                              int64_t sC, const float* bias, int64_t sBias, int accumulate,
-                             __nv_bfloat16* CT, int64_t ldT, int* status, cudaStream_t st) {
+                             __nv_bfloat16* Cb, int64_t ldb16, int* status, cudaStream_t st) {
   if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
   if (K <= 0 || (lda % 8) || (ldb % 8) || (sA % 8) || (sB % 8)) return cudaErrorInvalidValue;
   const int BN = N <= 64 ? 64 : N <= 128 ? 128 : N <= 192 ? 192 : 256;
@@ -496,7 +506,7 @@ cudaError_t gemm_bf16_tn_any(const void* A, int64_t lda, int64_t sA, const void*
   const int vec = (reinterpret_cast<uintptr_t>(Cout) % 16 == 0) && ldc % 4 == 0 && sC % 4 == 0 &&
                   (!bias || (reinterpret_cast<uintptr_t>(bias) % 16 == 0 && sBias % 4 == 0));
   BatchArgs g{M, N, (K + 63) / 64, a3 ? 1 : 0, b3 ? 1 : 0, Cout, ldc, sC, bias, sBias, accumulate,
-              vec, CT, ldT};
+              vec, Cb, ldb16};
   dim3 grid((M + 127) / 128, (N + BN - 1) / BN, batch);
   cudaError_t e;
 #define BG_GEMM16_CASE(BNV)                                                                    \
@@ -524,12 +534,12 @@ cudaError_t gemm_bf16_tn(const void* A, int64_t lda, int64_t sA, const void* B, 
                           accumulate, nullptr, 0, status, st);
 }
 
-cudaError_t gemm_bf16_tn_outT(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N,
-                              int K, __nv_bfloat16* CT, int64_t ldT, int* status, cudaStream_t st) {
-  if (!CT || (M % 2) || (N % 32) || (ldT % 2) || ldT < M ||
-      (reinterpret_cast<uintptr_t>(CT) % 4))
+cudaError_t gemm_bf16_tn_outb(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N,
+                              int K, __nv_bfloat16* Cb, int64_t ldb16, int* status,
+                              cudaStream_t st) {
+  if (!Cb || (N % 32) || (ldb16 % 8) || ldb16 < N || (reinterpret_cast<uintptr_t>(Cb) % 16))
     return cudaErrorInvalidValue;
-  return gemm_bf16_tn_any(A, lda, 0, B, ldb, 0, M, N, K, 1, nullptr, 0, 0, nullptr, 0, 0, CT, ldT,
+  return gemm_bf16_tn_any(A, lda, 0, B, ldb, 0, M, N, K, 1, nullptr, 0, 0, nullptr, 0, 0, Cb, ldb16,
                           status, st);
 }
 
@@ -551,13 +561,15 @@ cudaError_t gemm_tn_multi(const TNProblem* pr, int n, int Hout, int64_t K, int a
   const int MT = N <= 256 ? 2 : 1;  // M tiles per CTA (GCfg::MT)
   int mt = 0, Mtot = 0;
   for (int g = 0; g < n; ++g) {
-    if (!make_map_ld(&grp.a[g], pr[g].A, pr[g].M, K, pr[g].lda, 128) ||
+    if (!(pr[g].a_mn ? make_map_ld(&grp.a[g], pr[g].A, K, pr[g].M, pr[g].lda, 64)
+                     : make_map_ld(&grp.a[g], pr[g].A, pr[g].M, K, pr[g].lda, 128)) ||
         !make_map_ld(&grp.b[g], pr[g].B, N - 16, K, pr[g].ldb, N - 16))
       return cudaErrorInvalidValue;
     mt += ((pr[g].M + 127) / 128 + MT - 1) / MT;
     grp.it_end[g] = mt;
     grp.M[g] = o.M[g] = pr[g].M;
     grp.prow[g] = o.prow[g] = Mtot;
+    grp.a_mn[g] = pr[g].a_mn;
     o.out[g] = pr[g].out;
     o.bias[g] = pr[g].bias;
     o.mode[g] = pr[g].mode;
@@ -626,10 +638,10 @@ cudaError_t wait_selftest(int* status, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t gemm_tn(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int Hout,
-                    int64_t K, int mode, float* out, float* bias, int accumulate, float* part,
-                    size_t part_floats, int* status, cudaStream_t st) {
-  const TNProblem pr{A, lda, B, ldb, M, mode, out, bias};
+cudaError_t gemm_tn(const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb, int M,
+                    int Hout, int64_t K, int mode, float* out, float* bias, int accumulate,
+                    float* part, size_t part_floats, int* status, cudaStream_t st) {
+  const TNProblem pr{A, lda, a_mn, B, ldb, M, mode, out, bias};
   return gemm_tn_multi(&pr, 1, Hout, K, accumulate, part, part_floats, status, st);
 }
 

@@ -14,14 +14,15 @@ namespace bg {
 size_t gemm_tn_part_floats(int M, int N, int64_t K);
 
 // Reduces over K (nodes, possibly several steps concatenated) the outer products
-//   G[m][n] = sum_k A[m][k] B'[n][k]    A: [M][K] bf16 (row stride lda), B: [Hout][K] bf16
+//   G[m][n] = sum_k A[m][k] B'[n][k]    A: [M][K] bf16 (row stride lda), or with a_mn != 0 stored
+//   transposed, [K][M] (row stride lda, a multiple of 8); B: [Hout][K] bf16
 // where B' is B with a row of ones (row Hout) and 15 zero rows appended by the kernel, so column
 // Hout of G is the row sum of A (a bias gradient).  Output (accumulate != 0 adds):
 //   mode 0: out[m][n] = G[m][n] (n < Hout), bias[m] = G[m][Hout]
 //   mode 1: m = p*Hout + o: out[p][n][o] = G[m][n], bias[m] = G[m][Hout]   (bias may be NULL)
 // Hout in {32, 64, 128, 256}.  Deterministic: fixed split layout and summation order.
-cudaError_t gemm_tn(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int Hout,
-                    int64_t K, int mode, float* out, float* bias, int accumulate, float* part,
+cudaError_t gemm_tn(const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb, int M,
+                    int Hout, int64_t K, int mode, float* out, float* bias, int accumulate, float* part,
                     size_t part_floats, int* status, cudaStream_t st);
 
 // Up to four such problems with the same K and Hout in one launch (one wave over all their M
@@ -29,6 +30,7 @@ cudaError_t gemm_tn(const void* A, int64_t lda, const void* B, int64_t ldb, int 
 struct TNProblem {
   const void* A;
   int64_t lda;
+  int a_mn;
   const void* B;
   int64_t ldb;
   int M;
@@ -48,10 +50,11 @@ cudaError_t gemm_bf16_tn(const void* A, int64_t lda, int64_t sA, const void* B, 
                          int64_t sB, int M, int N, int K, int batch, float* C, int64_t ldc,
                          int64_t sC, const float* bias, int64_t sBias, int accumulate, int* status,
                          cudaStream_t st);
-// The same product (batch 1, no bias) rounded to bf16 and stored transposed: CT[n * ldT + m].  M
-// even, N a multiple of 32, ldT even and >= M, CT 4-byte aligned.
-cudaError_t gemm_bf16_tn_outT(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N,
-                              int K, __nv_bfloat16* CT, int64_t ldT, int* status, cudaStream_t st);
+// The same product (batch 1, no bias) rounded to bf16: Cb[m * ldb16 + n].  N a multiple of 32, ldb16
+// a multiple of 8, Cb 16-byte aligned.
+cudaError_t gemm_bf16_tn_outb(const void* A, int64_t lda, const void* B, int64_t ldb, int M, int N,
+                              int K, __nv_bfloat16* Cb, int64_t ldb16, int* status,
+                              cudaStream_t st);
 
 // 2-D bf16 tensor map over row-major [rows][cols] with row stride ld elements; box {64, box_rows};
 // 128-byte swizzle; reads outside the array return zero.
@@ -60,6 +63,10 @@ bool make_map_f32(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols
                   uint32_t box_rows);
 bool make_map_ld(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
                  uint32_t box_rows);
+// The same with boxes {box_cols, box_rows}, box_cols 64 (128-byte swizzle) or 32 (64-byte swizzle):
+// one box row is one swizzle row.
+bool make_map_box(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
+                  uint32_t box_cols, uint32_t box_rows);
 int gemm_tn_num_sms();
 // 3-D variant: [batch][rows][cols] with row stride ld and batch stride sbatch (elements).
 bool make_map_3d(CUtensorMap* m, const void* base, uint64_t batch, uint64_t rows, uint64_t cols,

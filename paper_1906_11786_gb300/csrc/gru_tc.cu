@@ -6,10 +6,11 @@
 //
 // Pre-activations live in TMEM: [r|z] = Y Wi_rz^T + E Wh_rz^T (2H columns: both products
 // accumulate into one tile), Wi_n x (H) and Wh_n h (H).  The forward epilogue applies the gates
-// and writes E(t+1) row-major and transposed (the next band product's operand).  The backward
+// and writes E(t+1) row-major (the next band product's operand) and transposed (the weight
+// gradients').  The backward
 // recomputes the same products, forms the gate gradients in registers, writes them back into the
 // TMEM columns it has just read as the bf16 A operand of dX = dgi W_ih and dH = dgh W_hh (chained
-// MMAs that accumulate into the freed Wi_n x / Wh_n h columns), and stores dX^T (the
+// MMAs that accumulate into the freed Wi_n x / Wh_n h columns), and stores dX (the
 // transposed-band operand), the running state gradient and dgi^T, dgh^T for the weight gradients.
 //
 // Both kernels are persistent (one CTA per SM) and warp-specialised: warp 0 streams 128-row
@@ -150,10 +151,6 @@ __device__ __forceinline__ void store_T_pairs(__nv_bfloat16* dst, int64_t ld, in
 __device__ __forceinline__ void store_T4(__nv_bfloat16* dst, int64_t ld, int row, int h0,
                                          const uint32_t* pk) {
   store_T_pairs<4>(dst, ld, row, h0, pk);
-}
-__device__ __forceinline__ void store_T8(__nv_bfloat16* dst, int64_t ld, int row, int h0,
-                                         const uint32_t* pk) {
-  store_T_pairs<8>(dst, ld, row, h0, pk);
 }
 
 template <int KH>
@@ -389,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                  const __grid_constant__ CUtensorMap tG,
                  const float* __restrict__ b_ih, const float* __restrict__ b_hh,
                  float* __restrict__ gout,
-                 __nv_bfloat16* __restrict__ dXT, int64_t ld_x, __nv_bfloat16* __restrict__ dgiT,
+                 __nv_bfloat16* __restrict__ dX, __nv_bfloat16* __restrict__ dgiT,
                  __nv_bfloat16* __restrict__ dhnT, int64_t ld_g, int n_tiles, int n_real,
                  int* status) {
   extern __shared__ uint8_t smem_raw[];
@@ -557,7 +554,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t px[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) px[j] = pk2(__uint_as_float(vx[2 * j]), __uint_as_float(vx[2 * j + 1]));
-      store_T8(dXT, ld_x, row, h0, px);
+      uint4* dx = reinterpret_cast<uint4*>(dX + (size_t)row * KH + h0);
+      dx[0] = make_uint4(px[0], px[1], px[2], px[3]);
+      dx[1] = make_uint4(px[4], px[5], px[6], px[7]);
       float4* go = reinterpret_cast<float4*>(gout + (size_t)row * KH + h0);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
@@ -1051,7 +1050,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const __grid_constant__ CUtensorMap tWihT, const __grid_constant__ CUtensorMap tWhhT,
               const __grid_constant__ CUtensorMap tG, const float* __restrict__ b_ih,
               const float* __restrict__ b_hh, float* __restrict__ gout,
-              __nv_bfloat16* __restrict__ dXT, int64_t ld_x, __nv_bfloat16* __restrict__ dgiT,
+              __nv_bfloat16* __restrict__ dX, __nv_bfloat16* __restrict__ dgiT,
               __nv_bfloat16* __restrict__ dhnT, int64_t ld_g, int n_tiles, int n_real,
               int* status) {
   extern __shared__ uint8_t smem_raw[];
@@ -1261,7 +1260,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t px[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) px[j] = pk2(__uint_as_float(vx[2 * j]), __uint_as_float(vx[2 * j + 1]));
-        store_T8(dXT, ld_x, row, h0, px);
+        uint4* dx = reinterpret_cast<uint4*>(dX + (size_t)row * H + h0);
+        dx[0] = make_uint4(px[0], px[1], px[2], px[3]);
+        dx[1] = make_uint4(px[4], px[5], px[6], px[7]);
         // this thread stored the direct term of these columns above
         float4* go = reinterpret_cast<float4*>(gout + (size_t)row * H + h0);
 #pragma unroll
@@ -1342,7 +1343,7 @@ cudaError_t gru_bwd_tc(int H, int n_pad, int n_real, const __nv_bfloat16* Y,
                        const __nv_bfloat16* E, const __nv_bfloat16* W_ih,
                        const __nv_bfloat16* W_hh, const __nv_bfloat16* W_ihT,
                        const __nv_bfloat16* W_hhT, const float* b_ih, const float* b_hh,
-                       const float* gin, float* gout, __nv_bfloat16* dXT, int64_t ld_x,
+                       const float* gin, float* gout, __nv_bfloat16* dX,
                        __nv_bfloat16* dgiT, __nv_bfloat16* dhnT, int64_t ld_g, int* status,
                        cudaStream_t st) {
   if (!gru_tc_supported(H) || n_pad % 128) return cudaErrorInvalidValue;
@@ -1363,7 +1364,7 @@ cudaError_t gru_bwd_tc(int H, int n_pad, int n_real, const __nv_bfloat16* Y,
   const int n_tiles = n_pad / 128;
   const int grid = std::min(n_tiles, gemm_tn_num_sms());
   e = launch_pdl(kern, dim3(grid), dim3(kThreads), smem, st, tY, tE, tWi, tWh, tWiT, tWhT, tG, b_ih,
-                 b_hh, gout, dXT, ld_x, dgiT, dhnT, ld_g, n_tiles, n_real, status);
+                 b_hh, gout, dX, dgiT, dhnT, ld_g, n_tiles, n_real, status);
   note_launch();
   return e;
 }

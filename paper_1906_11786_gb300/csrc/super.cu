@@ -62,12 +62,12 @@ __global__ void k_super_fwd(const int32_t* __restrict__ rows, const int32_t* __r
 }
 
 // Backward: one CTA per source row r, thread h = state column h.  dY is fp32 [n][H] (dYT NULL)
-// or bf16 transposed [H][ld] (dYT).  Wt[p][o][i] = W[p][i][o] (fp32).
+// or bf16 [n][H] (dYb).  Wt[p][o][i] = W[p][i][o] (fp32).
 __global__ void k_super_bwd(const int32_t* __restrict__ rows, const int32_t* __restrict__ poff,
                             const int32_t* __restrict__ pair_type,
                             const int32_t* __restrict__ pair_off, const int32_t* __restrict__ dst,
-                            const float* __restrict__ dY, const __nv_bfloat16* __restrict__ dYT,
-                            int64_t ld, const float* __restrict__ Wt, int H,
+                            const float* __restrict__ dY, const __nv_bfloat16* __restrict__ dYb,
+                            const float* __restrict__ Wt, int H,
                             float* __restrict__ dE, float* __restrict__ dMs) {
   extern __shared__ float g[];  // [H]: the current pair's dM_p[u]
   const int r = blockIdx.x, h = threadIdx.x;
@@ -76,7 +76,7 @@ __global__ void k_super_bwd(const int32_t* __restrict__ rows, const int32_t* __r
     float acc = 0.f;
     for (int e = pair_off[k]; e < pair_off[k + 1]; ++e) {
       const int v = dst[e];
-      acc += dYT ? __bfloat162float(dYT[(size_t)h * ld + v]) : dY[(size_t)v * H + h];
+      acc += dYb ? __bfloat162float(dYb[(size_t)v * H + h]) : dY[(size_t)v * H + h];
     }
     dMs[(size_t)k * H + h] = acc;
     __syncthreads();
@@ -250,7 +250,7 @@ cudaError_t super_fwd(const bg_plan* p, int bf16, int H, const void* E, const vo
 }
 
 cudaError_t super_bwd(const bg_plan* p, int bf16, int H, const void* E, const void* W,
-                      const float* dY, const __nv_bfloat16* dYT, int64_t ld, float* dE, float* dW,
+                      const float* dY, const __nv_bfloat16* dYb, float* dE, float* dW,
                       float* db, char* ws, cudaStream_t st, bool weights_ready) {
   if (!p->sup_rows_out) return cudaSuccess;
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -260,7 +260,7 @@ cudaError_t super_bwd(const bg_plan* p, int bf16, int H, const void* E, const vo
   if (!weights_ready) e = transpose_weights(bf16, W, Wt, p->P, H, st);
   if (e != cudaSuccess) return e;
   k_super_bwd<<<p->sup_rows_out, H, sizeof(float) * H, st>>>(
-      p->d_sout_rows, p->d_sout_poff, p->d_pair_type, p->d_pair_off, p->d_sout_dst, dY, dYT, ld,
+      p->d_sout_rows, p->d_sout_poff, p->d_pair_type, p->d_pair_off, p->d_sout_dst, dY, dYb,
       Wt, H, dE, dMs);
   note_launch();
   if (bf16)

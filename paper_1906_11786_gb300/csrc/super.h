@@ -25,10 +25,10 @@ cudaError_t super_fwd(const bg_plan* p, int bf16, int H, const void* E, const vo
 size_t super_bwd_ws_bytes(const bg_plan* p, int H);
 // Backward: dE[u] += sum_p dM_p[u] W_p^T, dW_p += E[u]^T dM_p[u], db_p += dM_p[u] (db may be
 // NULL) over the supernode edges, dM_p[u] = sum over edges (u -> v, p) of dY[v].  dY fp32
-// [n_pad][H], or (dY NULL) dYT bf16 [H][ld].  weights_ready: ws already holds W^T from an
+// [n_pad][H], or (dY NULL) dYb bf16 [n_pad][H].  weights_ready: ws already holds W^T from an
 // earlier call with the same W (the GGNN steps reuse it).
 cudaError_t super_bwd(const bg_plan* p, int bf16, int H, const void* E, const void* W,
-                      const float* dY, const __nv_bfloat16* dYT, int64_t ld, float* dE, float* dW,
+                      const float* dY, const __nv_bfloat16* dYb, float* dE, float* dW,
                       float* db, char* ws, cudaStream_t st, bool weights_ready = false);
 
 }  // namespace bg

@@ -121,6 +121,25 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* m, uin
       : "memory");
 }
 
+// 2-D tile shared -> global as one bulk group of the calling thread, and the waits on that thread's
+// groups: until shared memory has been read (at most N groups still reading), or until every
+// write is done.  The hardware completes bulk copies without help from other threads, so these
+// waits end by themselves.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, const void* src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(m)),
+               "r"(smem_u32(src)), "r"(x), "r"(y)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void tma_store_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void tma_store_wait_all() {
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+
 // 1-D bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
@@ -234,6 +253,33 @@ __device__ __forceinline__ uint64_t desc_sw128_kmajor(uint32_t start) {
   d |= (uint64_t)2 << 61;                            // layout: 128-byte swizzle
   return d;
 }
+
+// The same for an MN-major operand: rows of 64 consecutive M (or N) elements (128 bytes, 128-byte
+// swizzle), one row per K index; 8-row groups 1024 bytes apart along K (stride byte offset) and
+// blocks of 64 M/N elements `block_bytes` apart (leading byte offset).
+__device__ __forceinline__ uint64_t desc_sw128_mnmajor(uint32_t start, uint32_t block_bytes) {
+  uint64_t d = 0;
+  d |= (uint64_t)((start >> 4) & 0x3FFFu);
+  d |= (uint64_t)((block_bytes >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)(1024u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// MN-major with rows of 32 elements (64 bytes, 64-byte swizzle), 8-row groups 512 bytes apart.
+__device__ __forceinline__ uint64_t desc_sw64_mnmajor(uint32_t start) {
+  uint64_t d = 0;
+  d |= (uint64_t)((start >> 4) & 0x3FFFu);
+  d |= (uint64_t)(512u >> 4) << 16;
+  d |= (uint64_t)(512u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)4 << 61;
+  return d;
+}
+
+// Instruction-descriptor bits for an MN-major A or B operand (K-major without them).
+constexpr uint32_t kIdescAMN = 1u << 15, kIdescBMN = 1u << 16;
 
 // Instruction descriptor of tcgen05.mma kind::f16: bf16 A and B, fp32 accumulator, both K-major,
 // shape M x N.
