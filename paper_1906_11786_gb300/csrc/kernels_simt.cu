@@ -2,10 +2,14 @@
 // GRU gates, layout conversion, readout and Adam.  Every kernel is bounds-checked by its index
 // arithmetic; none waits on another block.
 #include <atomic>
+#include <type_traits>
 
 #include "kernels.h"
+#include "tc_util.cuh"
 
 namespace bg {
+
+using tc::grid_dep_wait;
 
 static std::atomic<long long> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -32,10 +36,15 @@ inline int grid_for(int64_t n, int threads) {
 constexpr int GT = 64;   // output tile edge
 constexpr int GK = 16;   // k step
 
+// 64 x 64 tile, 4 x 4 outputs per thread.  The next K step's operands are on their way in registers
+// while the current one is multiplied from shared memory (two buffers, one barrier a step): with the
+// loads in front of each step the loop was latency-bound (four 512 x 64 x 64 products 15.4 us
+// against 8.2; six products of 3,008 rows at H = 96 198 us against 134, ncu).
 template <typename TA, typename TB>
 __global__ void __launch_bounds__(256) k_gemm(Gemm g, int splits, int kchunk, float* part) {
-  __shared__ float As[GK][GT + 4];
-  __shared__ float Bs[GK][GT + 4];
+  __shared__ __align__(16) float As[2][GK][GT + 4];
+  __shared__ __align__(16) float Bs[2][GK][GT + 4];
+  grid_dep_wait();
   const TA* A = static_cast<const TA*>(g.A);
   const TB* B = static_cast<const TB*>(g.B);
   const int b = blockIdx.z / splits, s = blockIdx.z % splits;
@@ -50,33 +59,46 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, int splits, int kchunk, fl
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  for (int k0 = kbeg; k0 < kend; k0 += GK) {
+  float ra[4], rb[4];
+  auto fetch = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      int idx = tid + 256 * q;
-      int mm, kk;
-      if (a_k_fast) { kk = idx % GK; mm = idx / GK; } else { mm = idx % GT; kk = idx / GT; }
-      int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < g.M && k < kend) ? ld(A, b * g.sAb + m * g.sAm + k * g.sAk) : 0.f;
-      int nn;
-      if (b_n_fast) { nn = idx % GT; kk = idx / GT; } else { kk = idx % GK; nn = idx / GK; }
-      int n = n0 + nn;
-      k = k0 + kk;
-      Bs[kk][nn] = (n < g.N && k < kend) ? ld(B, b * g.sBb + k * g.sBk + n * g.sBn) : 0.f;
+      const int idx = tid + 256 * q;
+      const int am = a_k_fast ? idx / GK : idx % GT, ak = a_k_fast ? idx % GK : idx / GT;
+      const int m = m0 + am, k = k0 + ak;
+      ra[q] = (m < g.M && k < kend) ? ld(A, b * g.sAb + m * g.sAm + k * g.sAk) : 0.f;
+      const int bn = b_n_fast ? idx % GT : idx / GK, bk = b_n_fast ? idx / GT : idx % GK;
+      const int n = n0 + bn, kb = k0 + bk;
+      rb[q] = (n < g.N && kb < kend) ? ld(B, b * g.sBb + kb * g.sBk + n * g.sBn) : 0.f;
     }
-    __syncthreads();
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int idx = tid + 256 * q;
+      As[buf][a_k_fast ? idx % GK : idx / GT][a_k_fast ? idx / GK : idx % GT] = ra[q];
+      Bs[buf][b_n_fast ? idx / GT : idx % GK][b_n_fast ? idx % GT : idx / GK] = rb[q];
+    }
+  };
+  if (kbeg < kend) {
+    fetch(kbeg);
+    stage(0);
+  }
+  __syncthreads();
+  for (int k0 = kbeg, buf = 0; k0 < kend; k0 += GK, buf ^= 1) {
+    const bool more = k0 + GK < kend;
+    if (more) fetch(k0 + GK);
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      float a[4], bb[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty * 4 + r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) bb[c] = Bs[kk][tx * 4 + c];
+      const float4 av = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
+      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
+      const float a[4] = {av.x, av.y, av.z, av.w}, bb[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] += a[r] * bb[c];
     }
+    if (more) stage(buf ^ 1);
     __syncthreads();
   }
 #pragma unroll
@@ -99,6 +121,7 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, int splits, int kchunk, fl
 }
 
 __global__ void k_gemm_reduce(Gemm g, int splits, const float* part) {
+  grid_dep_wait();
   int64_t total = (int64_t)g.batch * g.M * g.N;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -115,6 +138,31 @@ __global__ void k_gemm_reduce(Gemm g, int splits, const float* part) {
 }
 
 // ------------------------------------------------------------------------------------ layout
+// Rows of whole 16-byte chunks: one chunk per thread, its row by one 32-bit division.  Bound by HBM
+// (both arrays once).  The element-wise form below divides a 64-bit index per element: at 72k x 64
+// fp32 it packs in 26.6 us and unpacks in 22.6, this one in 8.0 and 6.9 (ncu).
+__global__ void __launch_bounds__(256) k_pack16(const uint4* __restrict__ Eo, uint4* __restrict__ Eb,
+                                                const int32_t* __restrict__ gather, int n_real,
+                                                uint32_t total, uint32_t chunks) {
+  grid_dep_wait();
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= total) return;
+  const uint32_t q = t / chunks, c = t - q * chunks;
+  Eb[t] = q < (uint32_t)n_real ? Eo[(size_t)gather[q] * chunks + c] : make_uint4(0u, 0u, 0u, 0u);
+}
+
+__global__ void __launch_bounds__(256) k_unpack16(const uint4* __restrict__ Eb,
+                                                  uint4* __restrict__ Eo,
+                                                  const int32_t* __restrict__ gather,
+                                                  uint32_t total, uint32_t chunks) {
+  grid_dep_wait();
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x;
+  if (t >= total) return;
+  const uint32_t q = t / chunks, c = t - q * chunks;
+  Eo[(size_t)gather[q] * chunks + c] = Eb[t];
+}
+
+// Any row size and alignment, element by element.
 template <typename T>
 __global__ void k_pack(const T* Eo, T* Eb, const int32_t* gather, int n_real, int64_t total,
                        int H) {
@@ -137,76 +185,151 @@ __global__ void k_unpack(const T* Eb, T* Eo, const int32_t* gather, int64_t tota
 }
 
 // ------------------------------------------------------------------------------------ band
-// One warp per row; lanes hold columns lane + 32 q.  The mask word is read by every lane (a
-// broadcast) and its set bits are walked in order, so the summation order is fixed.
+// Sums rows of a [*][H] array (H = 32 HQ; lanes hold columns lane + 32 q) in the order they are
+// pushed, four rows' loads at a time: one row after another the sum waited out a memory latency per
+// edge (30k rows of 50 edges at H = 64: 193.7 us against 67.6, which is 5.7 TB/s from L2, ncu).
+template <int HQ>
+struct RowSum {
+  const float* src;
+  float acc[HQ];
+  int64_t r[4];
+  int n;
+  __device__ __forceinline__ void clear() {
+    n = 0;
+    r[0] = r[1] = r[2] = r[3] = 0;
+#pragma unroll
+    for (int q = 0; q < HQ; ++q) acc[q] = 0.f;
+  }
+  __device__ __forceinline__ void push(int64_t row) {
+    r[0] = r[1]; r[1] = r[2]; r[2] = r[3]; r[3] = row;
+    if (++n == 4) {
+      float v[4][HQ];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < HQ; ++q) v[i][q] = src[r[i] * (32 * HQ) + 32 * q];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < HQ; ++q) acc[q] += v[i][q];
+      n = 0;
+    }
+  }
+  __device__ __forceinline__ void finish() {  // the last n < 4 rows
+    float v[3][HQ];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < n) {
+        const int64_t row = n == 3 ? r[1 + i] : n == 2 ? r[2 + (i & 1)] : r[3];
+#pragma unroll
+        for (int q = 0; q < HQ; ++q) v[i][q] = src[row * (32 * HQ) + 32 * q];
+      }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (i < n)
+#pragma unroll
+        for (int q = 0; q < HQ; ++q) acc[q] += v[i][q];
+    n = 0;
+  }
+};
+
+// One warp per row.  Each lane reads one mask word of the row (in the order diagonal, type, word),
+// and the set bits of the words are walked in that order, so the summation order is fixed.
+template <int HQ>
 __global__ void __launch_bounds__(256) k_band_fwd_gather(const uint32_t* __restrict__ masks,
                                                          const float* __restrict__ M,
                                                          float* __restrict__ Y, int K, int S,
-                                                         int P, int H) {
+                                                         int P) {
+  grid_dep_wait();
   const int lane = threadIdx.x & 31;
   const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int64_t n_pad = (int64_t)K * S;
   if (i >= n_pad) return;
-  const int k = (int)(i / S), r = (int)(i % S), W32 = S / 32, HQ = H / 32;
-  float acc[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-  for (int e = 0; e < 3; ++e) {
-    const int kb = k + e - 1;
-    if (kb < 0 || kb >= K) continue;
-    for (int p = 0; p < P; ++p) {
-      const uint32_t* row = masks + ((((int64_t)k * 3 + e) * P + p) * S + r) * W32;
-      for (int w = 0; w < W32; ++w) {
-        uint32_t word = row[w];
-        while (word) {
-          const int c = __ffs(word) - 1;
-          word &= word - 1;
-          const float* m = M + ((int64_t)p * n_pad + (int64_t)kb * S + w * 32 + c) * H;
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (q < HQ) acc[q] += m[lane + 32 * q];
-        }
+  const int k = (int)(i / S), r = (int)(i % S), W32 = S / 32, nw = 3 * P * W32;
+  RowSum<HQ> sum;
+  sum.src = M + lane;
+  sum.clear();
+  for (int f0 = 0; f0 < nw; f0 += 32) {
+    const int f = f0 + lane;
+    uint32_t word = 0;
+    int64_t base = 0;  // row of M of the word's bit 0
+    if (f < nw) {
+      const int w = f % W32, ep = f / W32, e = ep / P, p = ep - e * P, kb = k + e - 1;
+      if (kb >= 0 && kb < K) {
+        word = masks[((((int64_t)k * 3 + e) * P + p) * S + r) * W32 + w];
+        base = (int64_t)p * n_pad + (int64_t)kb * S + w * 32;
+      }
+    }
+    uint32_t full = __ballot_sync(0xffffffffu, word != 0);
+    while (full) {
+      const int l = __ffs(full) - 1;
+      full &= full - 1;
+      uint32_t bits = __shfl_sync(0xffffffffu, word, l);
+      const int64_t b0 = __shfl_sync(0xffffffffu, base, l);
+      while (bits) {
+        sum.push(b0 + __ffs(bits) - 1);
+        bits &= bits - 1;
       }
     }
   }
+  sum.finish();
 #pragma unroll
-  for (int q = 0; q < 8; ++q)
-    if (q < HQ) Y[i * H + lane + 32 * q] = acc[q];
+  for (int q = 0; q < HQ; ++q) Y[i * (32 * HQ) + lane + 32 * q] = sum.acc[q];
 }
 
-template <typename TO>
+// The same over the transposed tiles, one sum per type; the next type's words are read while the
+// current one's rows are summed (3 S / 32 <= 48 words: two per lane).
+template <int HQ, typename TO>
 __global__ void __launch_bounds__(256) k_band_bwd_gather(const uint32_t* __restrict__ masksT,
                                                          const float* __restrict__ dY,
-                                                         TO* __restrict__ dM, int K, int S,
-                                                         int P, int H) {
+                                                         TO* __restrict__ dM, int K, int S, int P) {
+  grid_dep_wait();
   const int lane = threadIdx.x & 31;
   const int64_t j = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int64_t n_pad = (int64_t)K * S;
   if (j >= n_pad) return;
-  const int kj = (int)(j / S), c = (int)(j % S), W32 = S / 32, HQ = H / 32;
+  const int kj = (int)(j / S), c = (int)(j % S), W32 = S / 32, nw = 3 * W32;
+  RowSum<HQ> sum;
+  sum.src = dY + lane;
+  int64_t base[2];
+  bool in[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int f = lane + 32 * h, e = f / W32, kb = kj + e - 1;
+    in[h] = f < nw && kb >= 0 && kb < K;
+    base[h] = (int64_t)kb * S + (f - e * W32) * 32;
+  }
+  auto words = [&](int p, uint32_t (&w)[2]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int f = lane + 32 * h, e = f / W32;
+      w[h] = in[h] ? masksT[((((int64_t)kj * 3 + e) * P + p) * S + c) * W32 + f - e * W32] : 0u;
+    }
+  };
+  uint32_t cur[2], nxt[2] = {0u, 0u};
+  words(0, cur);
   for (int p = 0; p < P; ++p) {
-    float acc[8];
+    if (p + 1 < P) words(p + 1, nxt);
+    sum.clear();
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-    for (int e = 0; e < 3; ++e) {
-      const int kb = kj + e - 1;
-      if (kb < 0 || kb >= K) continue;
-      const uint32_t* row = masksT + ((((int64_t)kj * 3 + e) * P + p) * S + c) * W32;
-      for (int w = 0; w < W32; ++w) {
-        uint32_t word = row[w];
-        while (word) {
-          const int t = __ffs(word) - 1;
-          word &= word - 1;
-          const float* g = dY + ((int64_t)kb * S + w * 32 + t) * H;
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (q < HQ) acc[q] += g[lane + 32 * q];
+    for (int h = 0; h < 2; ++h) {
+      uint32_t full = __ballot_sync(0xffffffffu, cur[h] != 0);
+      while (full) {
+        const int l = __ffs(full) - 1;
+        full &= full - 1;
+        uint32_t bits = __shfl_sync(0xffffffffu, cur[h], l);
+        const int64_t b0 = __shfl_sync(0xffffffffu, base[h], l);
+        while (bits) {
+          sum.push(b0 + __ffs(bits) - 1);
+          bits &= bits - 1;
         }
       }
     }
+    sum.finish();
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (q < HQ) st(dM, (j * P + p) * H + lane + 32 * q, acc[q]);
+    for (int q = 0; q < HQ; ++q) st(dM, (j * P + p) * (32 * HQ) + lane + 32 * q, sum.acc[q]);
+    cur[0] = nxt[0];
+    cur[1] = nxt[1];
   }
 }
 
@@ -232,6 +355,7 @@ __global__ void k_f32_to_bf16(const float* __restrict__ x, __nv_bfloat16* __rest
 // Four elements per thread: one 16-byte load, one 8-byte store (x 16-byte and y 8-byte aligned,
 // n4 = n / 4 groups; the caller converts the n % 4 tail with k_f32_to_bf16).
 __global__ void k_f32_to_bf16_x4(const float4* __restrict__ x, uint2* __restrict__ y, int64_t n4) {
+  grid_dep_wait();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n4;
        t += (int64_t)gridDim.x * blockDim.x) {
     const float4 v = x[t];
@@ -242,6 +366,7 @@ __global__ void k_f32_to_bf16_x4(const float4* __restrict__ x, uint2* __restrict
 
 template <typename T>
 __global__ void k_transpose_w(const T* W, float* Wt, int P, int H) {
+  grid_dep_wait();
   int64_t total = (int64_t)P * H * H;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -254,6 +379,7 @@ __global__ void k_transpose_w(const T* W, float* Wt, int P, int H) {
 }
 
 __global__ void k_colsum_part(const float* X, int64_t rows, int cols, int64_t chunk, float* part) {
+  grid_dep_wait();
   int col = blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= cols) return;
   int64_t r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
@@ -263,6 +389,7 @@ __global__ void k_colsum_part(const float* X, int64_t rows, int cols, int64_t ch
 }
 
 __global__ void k_colsum_reduce(const float* part, int splits, int cols, float* out, int accum) {
+  grid_dep_wait();
   int col = blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= cols) return;
   float s = 0.f;
@@ -276,6 +403,7 @@ __device__ __forceinline__ float sigm(float x) { return 1.f / (1.f + __expf(-x))
 template <typename T>
 __global__ void k_gru_fwd(const float* gi, const float* gh, const T* E, T* En, int n_real,
                           int64_t total, int H) {
+  grid_dep_wait();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
     int64_t i = t / H;
@@ -293,6 +421,7 @@ __global__ void k_gru_fwd(const float* gi, const float* gh, const T* E, T* En, i
 template <typename T>
 __global__ void k_gru_bwd(const float* gi, const float* gh, const T* E, const float* dHn,
                           float* dgi, float* dgh, float* dHd, int n_real, int64_t total, int H) {
+  grid_dep_wait();
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
     int64_t i = t / H;
@@ -427,11 +556,15 @@ __global__ void k_add(float* d, const float* s, int64_t n) {
 cudaError_t gemm(const Gemm& g, float* part, size_t part_floats, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   int tiles = ((g.N + GT - 1) / GT) * ((g.M + GT - 1) / GT) * g.batch;
+  // Few tiles: K split over more blocks, at least 64 of it each (four steps of the loop).  The second
+  // launch costs about 3.5 us, so K below 256 is not split.  The two products of the 512-node fp32
+  // backward (512 x 64 x 256, and 64 x 64 x 512 for four types) take 15.4 us and 7.2 for their
+  // reductions; with the split from K > 512 on and the old loop 161.7 us (ncu).
   int splits = 1;
-  if (g.K > 512 && tiles < 304) {
+  if (g.K >= 256 && tiles < 304 && part) {
     splits = (304 + tiles - 1) / tiles;
     splits = splits > 64 ? 64 : splits;
-    int maxk = (g.K + 255) / 256;
+    int maxk = g.K / 64;
     if (splits > maxk) splits = maxk;
     while (splits > 1 && (size_t)splits * g.batch * g.M * g.N > part_floats) --splits;
   }
@@ -440,26 +573,46 @@ cudaError_t gemm(const Gemm& g, float* part, size_t part_floats, cudaStream_t st
   splits = (g.K + kchunk - 1) / kchunk;
   if (splits < 1) splits = 1;
   dim3 grid((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, g.batch * splits);
+  cudaError_t e;
   if (g.a_bf16 && g.b_bf16)
-    k_gemm<__nv_bfloat16, __nv_bfloat16><<<grid, 256, 0, st>>>(g, splits, kchunk, part);
+    e = launch_pdl(k_gemm<__nv_bfloat16, __nv_bfloat16>, grid, dim3(256), 0, st, g, splits, kchunk, part);
   else if (g.a_bf16)
-    k_gemm<__nv_bfloat16, float><<<grid, 256, 0, st>>>(g, splits, kchunk, part);
+    e = launch_pdl(k_gemm<__nv_bfloat16, float>, grid, dim3(256), 0, st, g, splits, kchunk, part);
   else if (g.b_bf16)
-    k_gemm<float, __nv_bfloat16><<<grid, 256, 0, st>>>(g, splits, kchunk, part);
+    e = launch_pdl(k_gemm<float, __nv_bfloat16>, grid, dim3(256), 0, st, g, splits, kchunk, part);
   else
-    k_gemm<float, float><<<grid, 256, 0, st>>>(g, splits, kchunk, part);
+    e = launch_pdl(k_gemm<float, float>, grid, dim3(256), 0, st, g, splits, kchunk, part);
   note_launch();
-  if (splits > 1) {
+  if (e == cudaSuccess && splits > 1) {
     int64_t total = (int64_t)g.batch * g.M * g.N;
-    k_gemm_reduce<<<grid_for(total, 256), 256, 0, st>>>(g, splits, part);
+    e = launch_pdl(k_gemm_reduce, dim3(grid_for(total, 256)), dim3(256), 0, st, g, splits,
+                   (const float*)part);
     note_launch();
   }
-  return cudaGetLastError();
+  return e;
+}
+
+// Rows of H elements of `esize` bytes as whole 16-byte chunks: the number per row, 0 where the rows
+// or the arrays are not so aligned, or the chunks exceed 32 bits.
+static uint32_t row_chunks(const void* a, const void* b, int64_t rows, int H, int esize) {
+  const uintptr_t m = reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b);
+  const int64_t bytes = (int64_t)H * esize;
+  return (m % 16 == 0 && bytes % 16 == 0 && rows * (bytes / 16) < (int64_t)1 << 31)
+             ? (uint32_t)(bytes / 16) : 0;
 }
 
 cudaError_t pack_states(int bf16, const void* Eo, void* Eb, const int32_t* gather, int n_real,
                         int n_pad, int H, cudaStream_t st) {
   int64_t total = (int64_t)n_pad * H;
+  if (const uint32_t c = row_chunks(Eo, Eb, n_pad, H, bf16 ? 2 : 4)) {
+    const uint32_t n = (uint32_t)n_pad * c;
+    if (!n) return cudaSuccess;
+    cudaError_t e = launch_pdl(k_pack16, dim3((n + 255) / 256), dim3(256), 0, st,
+                               static_cast<const uint4*>(Eo), static_cast<uint4*>(Eb), gather, n_real,
+                               n, c);
+    note_launch();
+    return e;
+  }
   if (bf16)
     k_pack<<<grid_for(total, 256), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(Eo),
                                                  static_cast<__nv_bfloat16*>(Eb), gather, n_real,
@@ -475,6 +628,13 @@ cudaError_t unpack_states(int bf16, const void* Eb, void* Eo, const int32_t* gat
                           int H, cudaStream_t st) {
   int64_t total = (int64_t)n_real * H;
   if (total == 0) return cudaSuccess;
+  if (const uint32_t c = row_chunks(Eb, Eo, n_real, H, bf16 ? 2 : 4)) {
+    const uint32_t n = (uint32_t)n_real * c;
+    cudaError_t e = launch_pdl(k_unpack16, dim3((n + 255) / 256), dim3(256), 0, st,
+                               static_cast<const uint4*>(Eb), static_cast<uint4*>(Eo), gather, n, c);
+    note_launch();
+    return e;
+  }
   if (bf16)
     k_unpack<<<grid_for(total, 256), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(Eb),
                                                    static_cast<__nv_bfloat16*>(Eo), gather, total,
@@ -486,6 +646,24 @@ cudaError_t unpack_states(int bf16, const void* Eb, void* Eo, const int32_t* gat
   return cudaGetLastError();
 }
 
+namespace {
+// f(integral_constant<int, H / 32>) for H a multiple of 32 up to 256
+template <typename F>
+cudaError_t with_hq(int H, F f) {
+  switch (H / 32) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    case 8: return f(std::integral_constant<int, 8>{});
+    default: return cudaErrorInvalidValue;
+  }
+}
+}  // namespace
+
 cudaError_t preload_fwd_simt() {
   // CUDA loads kernels lazily, on first launch; this loads the ones the SIMT forward launches
   cudaFuncAttributes a;
@@ -496,33 +674,43 @@ cudaError_t preload_fwd_simt() {
   take(cudaFuncGetAttributes(&a, k_gemm<float, __nv_bfloat16>));
   take(cudaFuncGetAttributes(&a, k_gemm<float, float>));
   take(cudaFuncGetAttributes(&a, k_gemm_reduce));
-  take(cudaFuncGetAttributes(&a, k_band_fwd_gather));
+  for (int H = 32; H <= 256; H += 32)
+    take(with_hq(H, [&](auto hq) {
+      return cudaFuncGetAttributes(&a, k_band_fwd_gather<decltype(hq)::value>);
+    }));
   return e;
 }
 
 cudaError_t band_fwd_gather(const uint32_t* masks, const float* M, float* Y, int K, int S, int P,
                             int H, cudaStream_t st) {
-  int64_t rows = (int64_t)K * S;
-  k_band_fwd_gather<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(masks, M, Y, K, S, P, H);
+  const dim3 grid((unsigned)(((int64_t)K * S + 7) / 8));
+  cudaError_t e = with_hq(H, [&](auto hq) {
+    return launch_pdl(k_band_fwd_gather<decltype(hq)::value>, grid, dim3(256), 0, st, masks, M, Y, K, S, P);
+  });
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t band_bwd_gather(const uint32_t* masksT, const float* dY, float* dM, int K, int S,
                             int P, int H, cudaStream_t st) {
-  int64_t rows = (int64_t)K * S;
-  k_band_bwd_gather<float><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(masksT, dY, dM, K, S, P, H);
+  const dim3 grid((unsigned)(((int64_t)K * S + 7) / 8));
+  cudaError_t e = with_hq(H, [&](auto hq) {
+    return launch_pdl(k_band_bwd_gather<decltype(hq)::value, float>, grid, dim3(256), 0, st, masksT, dY,
+                      dM, K, S, P);
+  });
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t band_bwd_gather_bf16(const uint32_t* masksT, const float* dY, __nv_bfloat16* dM, int K,
                                  int S, int P, int H, cudaStream_t st) {
-  int64_t rows = (int64_t)K * S;
-  k_band_bwd_gather<__nv_bfloat16><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(masksT, dY, dM, K,
-                                                                               S, P, H);
+  const dim3 grid((unsigned)(((int64_t)K * S + 7) / 8));
+  cudaError_t e = with_hq(H, [&](auto hq) {
+    return launch_pdl(k_band_bwd_gather<decltype(hq)::value, __nv_bfloat16>, grid, dim3(256), 0, st,
+                      masksT, dY, dM, K, S, P);
+  });
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t wperm(const void* W, __nv_bfloat16* Wp, int P, int H, cudaStream_t st) {
@@ -537,9 +725,10 @@ cudaError_t f32_to_bf16(const float* x, __nv_bfloat16* y, int64_t n, cudaStream_
   const int64_t n4 = (reinterpret_cast<uintptr_t>(x) % 16 == 0 && reinterpret_cast<uintptr_t>(y) % 8 == 0)
                          ? n / 4 : 0;
   if (n4 > 0) {
-    k_f32_to_bf16_x4<<<grid_for(n4, 256), 256, 0, st>>>(reinterpret_cast<const float4*>(x),
-                                                        reinterpret_cast<uint2*>(y), n4);
+    cudaError_t e = launch_pdl(k_f32_to_bf16_x4, dim3(grid_for(n4, 256)), dim3(256), 0, st,
+                               reinterpret_cast<const float4*>(x), reinterpret_cast<uint2*>(y), n4);
     note_launch();
+    if (e != cudaSuccess) return e;
   }
   if (n > 4 * n4) {
     k_f32_to_bf16<<<grid_for(n - 4 * n4, 256), 256, 0, st>>>(x + 4 * n4, y + 4 * n4, n - 4 * n4);
@@ -550,57 +739,64 @@ cudaError_t f32_to_bf16(const float* x, __nv_bfloat16* y, int64_t n, cudaStream_
 
 cudaError_t transpose_weights(int bf16, const void* W, float* Wt, int P, int H, cudaStream_t st) {
   int64_t total = (int64_t)P * H * H;
+  cudaError_t e;
   if (bf16)
-    k_transpose_w<<<grid_for(total, 256), 256, 0, st>>>(static_cast<const __nv_bfloat16*>(W), Wt,
-                                                        P, H);
+    e = launch_pdl(k_transpose_w<__nv_bfloat16>, dim3(grid_for(total, 256)), dim3(256), 0, st,
+                   static_cast<const __nv_bfloat16*>(W), Wt, P, H);
   else
-    k_transpose_w<<<grid_for(total, 256), 256, 0, st>>>(static_cast<const float*>(W), Wt, P, H);
+    e = launch_pdl(k_transpose_w<float>, dim3(grid_for(total, 256)), dim3(256), 0, st,
+                   static_cast<const float*>(W), Wt, P, H);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t colsum(const float* X, int64_t rows, int cols, float* out, int accumulate, float* part,
                    size_t part_floats, cudaStream_t st) {
-  int splits = (int)((rows + 1023) / 1024);
+  // 32 rows a block up to 256 blocks (one block of 512 rows added them one latency after another:
+  // 32.3 us against 3.9)
+  int splits = (int)((rows + 31) / 32);
   if (splits > 256) splits = 256;
   while (splits > 1 && (size_t)splits * cols > part_floats) --splits;
   if (splits < 1) splits = 1;
   if ((size_t)splits * cols > part_floats) return cudaErrorInvalidValue;  // partials always used
   int64_t chunk = (rows + splits - 1) / splits;
   dim3 grid((cols + 255) / 256, splits);
-  k_colsum_part<<<grid, 256, 0, st>>>(X, rows, cols, chunk, part);
+  cudaError_t e = launch_pdl(k_colsum_part, grid, dim3(256), 0, st, X, rows, cols, chunk, part);
   note_launch();
-  k_colsum_reduce<<<(cols + 255) / 256, 256, 0, st>>>(part, splits, cols, out, accumulate);
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_colsum_reduce, dim3((cols + 255) / 256), dim3(256), 0, st, (const float*)part, splits,
+                 cols, out, accumulate);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t gru_fwd_gates(int bf16, const float* gi, const float* gh, const void* E, void* En,
                           int n_real, int n_pad, int H, cudaStream_t st) {
-  int64_t total = (int64_t)n_pad * H;
+  const int64_t total = (int64_t)n_pad * H;
+  cudaError_t e;
   if (bf16)
-    k_gru_fwd<<<grid_for(total, 256), 256, 0, st>>>(gi, gh, static_cast<const __nv_bfloat16*>(E),
-                                                    static_cast<__nv_bfloat16*>(En), n_real,
-                                                    total, H);
+    e = launch_pdl(k_gru_fwd<__nv_bfloat16>, dim3(grid_for(total, 256)), dim3(256), 0, st, gi, gh,
+                   static_cast<const __nv_bfloat16*>(E), static_cast<__nv_bfloat16*>(En), n_real, total, H);
   else
-    k_gru_fwd<<<grid_for(total, 256), 256, 0, st>>>(gi, gh, static_cast<const float*>(E),
-                                                    static_cast<float*>(En), n_real, total, H);
+    e = launch_pdl(k_gru_fwd<float>, dim3(grid_for(total, 256)), dim3(256), 0, st, gi, gh,
+                   static_cast<const float*>(E), static_cast<float*>(En), n_real, total, H);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t gru_bwd_gates(int bf16, const float* gi, const float* gh, const void* E,
                           const float* dHn, float* dgi, float* dgh, float* dHd, int n_real,
                           int n_pad, int H, cudaStream_t st) {
-  int64_t total = (int64_t)n_pad * H;
+  const int64_t total = (int64_t)n_pad * H;
+  cudaError_t e;
   if (bf16)
-    k_gru_bwd<<<grid_for(total, 256), 256, 0, st>>>(gi, gh, static_cast<const __nv_bfloat16*>(E),
-                                                    dHn, dgi, dgh, dHd, n_real, total, H);
+    e = launch_pdl(k_gru_bwd<__nv_bfloat16>, dim3(grid_for(total, 256)), dim3(256), 0, st, gi, gh,
+                   static_cast<const __nv_bfloat16*>(E), dHn, dgi, dgh, dHd, n_real, total, H);
   else
-    k_gru_bwd<<<grid_for(total, 256), 256, 0, st>>>(gi, gh, static_cast<const float*>(E), dHn, dgi,
-                                                    dgh, dHd, n_real, total, H);
+    e = launch_pdl(k_gru_bwd<float>, dim3(grid_for(total, 256)), dim3(256), 0, st, gi, gh,
+                   static_cast<const float*>(E), dHn, dgi, dgh, dHd, n_real, total, H);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t readout_loss(int bf16, const void* ET, const float* w_out, const float* target,
