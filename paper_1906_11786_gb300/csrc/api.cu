@@ -902,8 +902,7 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
     float* addend = p->sup_rows_in ? reinterpret_cast<float*>(wsc + wl.addend) : nullptr;
     BG_CUDA(cudaMemcpyAsync(Ei(0), E0, n * H * 2, cudaMemcpyDeviceToDevice, st));
     BG_CUDA(bg::prep_transpose_bf16(E0, 0, ETa, (int)n, H, 1, st, (int64_t)TN));
-    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 0, WT, st));
-    if (prm->b) BG_CUDA(bg::prep_bias_split(p, prm->b, b2T, H, status, st));
+    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 0, WT, prm->b, b2T, status, st));
     for (int t = 0; t < T; ++t) {
       // the supernode rows' messages, which the band kernel adds before it rounds Y
       if (addend) BG_CUDA(bg::super_fwd(p, 1, H, Ei(t), prm->W, prm->b, addend, 1, st));
@@ -948,8 +947,7 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
                                             al((size_t)H * 64 * 2));
     float* addend = p->sup_rows_in ? reinterpret_cast<float*>(wsc + w.addend) : nullptr;
     BG_CUDA(bg::prep_transpose_bf16(E0, 0, ETa, (int)n, H, 1, st, (int64_t)TN));
-    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 0, WT, st));
-    if (prm->b) BG_CUDA(bg::prep_bias_split(p, prm->b, b2T, H, status, st));
+    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 0, WT, prm->b, b2T, status, st));
     for (int t = 0; t < T; ++t) {
       const auto* Et = reinterpret_cast<const __nv_bfloat16*>(sv + saved_E_off(p, dt, H, t));
       auto* En = reinterpret_cast<__nv_bfloat16*>(sv + saved_E_off(p, dt, H, t + 1));
@@ -1033,7 +1031,7 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     BG_CUDA(bg::prep_transpose_bf16(Wih, 0, WihT, 3 * H, H, 1, st));
     BG_CUDA(bg::prep_transpose_bf16(Whh, 0, WhhT, 3 * H, H, 1, st));
     void* Wk = wsc + wl.Wk;
-    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 1, Wk, st));
+    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 1, Wk, nullptr, nullptr, status, st));
     const bool sup = p->n_super_edges() > 0;
     float* dWs = reinterpret_cast<float*>(wsc + wl.dWs);
     float* dbs = reinterpret_cast<float*>(wsc + wl.dbs);
@@ -1119,7 +1117,7 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     const auto* Whh = static_cast<const __nv_bfloat16*>(prm->W_hh);
     BG_CUDA(bg::prep_transpose_bf16(Wih, 0, WihT, 3 * H, H, 1, st));
     BG_CUDA(bg::prep_transpose_bf16(Whh, 0, WhhT, 3 * H, H, 1, st));
-    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 1, Wk, st));
+    BG_CUDA(bg::band_tc_prep_w(p, H, prm->W, 1, Wk, nullptr, nullptr, status, st));
     const bool sup = p->n_super_edges() > 0;
     float* dWs = reinterpret_cast<float*>(wsc + w.dWs);
     float* dbs = reinterpret_cast<float*>(wsc + w.dbs);

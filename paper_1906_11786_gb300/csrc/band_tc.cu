@@ -747,6 +747,7 @@ template <typename T>
 __global__ void k_transpose_bf16(const T* __restrict__ in, __nv_bfloat16* __restrict__ out, int R,
                                  int Cc, int64_t in_batch, int64_t out_batch, int64_t ld_out) {
   __shared__ float tile[32][33];
+  grid_dep_wait();
   in += blockIdx.z * in_batch;
   out += blockIdx.z * out_batch;
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
@@ -771,14 +772,21 @@ __global__ void k_transpose_bf16(const T* __restrict__ in, __nv_bfloat16* __rest
 // Second-product weights in the band kernel's operand layout, for each type p:
 //   forward  out[p][o][i] = W[p][i][o]   (W_p^T, K-major in i)
 //   backward out[p][i][o] = W[p][i][o]   (W_p as given, K-major in o)
-// as fp32 (the tf32 product's B operand).
-__global__ void k_prep_w(const __nv_bfloat16* __restrict__ W, float* __restrict__ out, int P, int H,
-                         int transpose) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)P * H * H) return;
-  const int64_t p = t / ((int64_t)H * H);
-  const int a = (int)((t / H) % H), c = (int)(t % H);
-  out[t] = __bfloat162float(transpose ? W[(p * H + c) * H + a] : W[(p * H + a) * H + c]);
+// as fp32 (the tf32 product's B operand).  Blocks beyond P H H / 256 do the bias split (b2T not
+// NULL): one launch instead of two before every propagation.
+__device__ void bias_split(const float* b, uint16_t* b2T, int P, int H, int f16, int* status, int t);
+__global__ void __launch_bounds__(256) k_prep_w(const __nv_bfloat16* __restrict__ W,
+                                                float* __restrict__ out, int P, int H, int transpose,
+                                                const float* __restrict__ b,
+                                                uint16_t* __restrict__ b2T, int f16, int* status) {
+  grid_dep_wait();
+  const uint32_t t = blockIdx.x * 256u + threadIdx.x, HH = (uint32_t)(H * H), total = (uint32_t)P * HH;
+  if (t < total) {
+    const uint32_t p = t / HH, r = t - p * HH, a = r / (uint32_t)H, c = r - a * (uint32_t)H;
+    out[t] = __bfloat162float(transpose ? W[p * HH + c * H + a] : W[t]);
+  } else if (b2T && t - total < (uint32_t)H * 64u) {
+    bias_split(b, b2T, P, H, f16, status, (int)(t - total));
+  }
 }
 
 // Outputs of the split tiles: Y = sum over the ksplit slices of `part` (fixed order), written like
@@ -828,10 +836,8 @@ __global__ void k_band_split_fixup(const float* __restrict__ part, int ksplit, i
 // both fp16 (f16 != 0; the in-degrees are then fp16 too).  fp16 holds magnitudes up to 65504: a
 // finite bias beyond that is recorded in the status word (code 2, site 120) and the product is
 // then not to be trusted.
-__global__ void k_bias_split(const float* __restrict__ b, uint16_t* __restrict__ b2T, int P, int H,
-                             int f16, int* status) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= H * 64) return;
+__device__ void bias_split(const float* __restrict__ b, uint16_t* __restrict__ b2T, int P, int H,
+                           int f16, int* status, int t) {
   const int h = t / 64, q = t % 64, p = q % 32;
   float x = 0.f;
   if (p < P && b) x = b[p * H + h];
@@ -1048,13 +1054,14 @@ size_t band_tc_w_bytes(const bg_plan* p, int H) {
 }
 
 cudaError_t band_tc_prep_w(const bg_plan* p, int H, const void* W, int bwd, void* Wk,
-                           cudaStream_t st) {
-  const int64_t n = (int64_t)p->P * H * H;
-  const int blocks = (int)((n + 255) / 256);
-  const auto* w = static_cast<const __nv_bfloat16*>(W);
-  k_prep_w<<<blocks, 256, 0, st>>>(w, static_cast<float*>(Wk), p->P, H, !bwd);
+                           const float* b, __nv_bfloat16* b2T, int* status, cudaStream_t st) {
+  const int64_t n = (int64_t)p->P * H * H + (b ? H * 64 : 0);
+  cudaError_t e = launch_pdl(k_prep_w, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st,
+                             static_cast<const __nv_bfloat16*>(W), static_cast<float*>(Wk), p->P, H,
+                             bwd ? 0 : 1, b, b ? reinterpret_cast<uint16_t*>(b2T) : nullptr,
+                             p->max_deg > 256 ? 1 : 0, status);
   note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 // (The first n H bf16 elements are not used; the size is what callers have always been asked for,
@@ -1129,23 +1136,16 @@ cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* ou
                                 int batch, cudaStream_t st, int64_t ld_out) {
   dim3 grid((Cc + 31) / 32, (R + 31) / 32, batch);
   if (ld_out <= 0) ld_out = R;
+  const int64_t sb = (int64_t)R * Cc;
+  cudaError_t e;
   if (in_is_f32)
-    k_transpose_bf16<float><<<grid, dim3(32, 8), 0, st>>>(static_cast<const float*>(in), out, R, Cc,
-                                                          (int64_t)R * Cc, (int64_t)R * Cc, ld_out);
+    e = launch_pdl(k_transpose_bf16<float>, grid, dim3(32, 8), 0, st, static_cast<const float*>(in),
+                   out, R, Cc, sb, sb, ld_out);
   else
-    k_transpose_bf16<__nv_bfloat16><<<grid, dim3(32, 8), 0, st>>>(
-        static_cast<const __nv_bfloat16*>(in), out, R, Cc, (int64_t)R * Cc, (int64_t)R * Cc,
-        ld_out);
+    e = launch_pdl(k_transpose_bf16<__nv_bfloat16>, grid, dim3(32, 8), 0, st,
+                   static_cast<const __nv_bfloat16*>(in), out, R, Cc, sb, sb, ld_out);
   note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t prep_bias_split(const bg_plan* p, const float* b, __nv_bfloat16* b2T, int H,
-                            int* status, cudaStream_t st) {
-  k_bias_split<<<(H * 64 + 255) / 256, 256, 0, st>>>(b, reinterpret_cast<uint16_t*>(b2T), p->P, H,
-                                                     p->max_deg > 256 ? 1 : 0, status);
-  note_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, const float* b,
@@ -1158,8 +1158,7 @@ cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, c
   float* split = reinterpret_cast<float*>(ws + al256((size_t)n * H * 2) + band_tc_w_bytes(p, H) +
                                           al256((size_t)H * 64 * 2));
   // W_p [H_in][H_out] -> W_p^T in the kernel's operand type;  bias split
-  cudaError_t e = band_tc_prep_w(p, H, W, 0, WT, st);
-  if (e == cudaSuccess && b) e = prep_bias_split(p, b, b2T, H, status, st);
+  cudaError_t e = band_tc_prep_w(p, H, W, 0, WT, b, b2T, status, st);
   if (e != cudaSuccess) return e;
   ProfSpan span(BG_KID_BAND_FWD, st);
   return band_tc_fwd_core(p, H, static_cast<const __nv_bfloat16*>(E), WT, b ? b2T : nullptr, b, Y,
@@ -1185,7 +1184,7 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
   o += al256(sizeof(float) * part_floats);
   float* split = band_tc_split_floats(p, H) ? reinterpret_cast<float*>(ws + o) : nullptr;
   cudaError_t e = f32_to_bf16(dY, dYb, (int64_t)n * H, st);
-  if (e == cudaSuccess) e = band_tc_prep_w(p, H, W, 1, Wk, st);
+  if (e == cudaSuccess) e = band_tc_prep_w(p, H, W, 1, Wk, nullptr, nullptr, status, st);
   if (e == cudaSuccess) {
     ProfSpan span(BG_KID_BAND_BWD, st);
     e = band_tc_bwd_core(p, H, dYb, Wk, dE, accum, dM, split, status, st);
@@ -1228,7 +1227,6 @@ cudaError_t band_tc_preload_fwd(const bg_plan* p) {
   cudaError_t e = cudaSuccess;
   auto take = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   take(cudaFuncGetAttributes(&a, k_prep_w));
-  take(cudaFuncGetAttributes(&a, k_bias_split));
   take(cudaFuncGetAttributes(&a, k_band_split_fixup));
 #define BG_PRELOAD(HV, SV) take(cudaFuncGetAttributes(&a, k_band_tc<HV, SV, false>));
 #define BG_PRELOAD_S(SV) BG_PRELOAD(32, SV) BG_PRELOAD(64, SV) BG_PRELOAD(128, SV)

@@ -22,8 +22,11 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
 // The band kernel's second-product weights (band_tc_w_bytes): from W [P][H][H] bf16, the forward
 // operand W_p^T (bwd = 0) or the backward operand W_p (bwd = 1), fp32 (kind::tf32 product).
 size_t band_tc_w_bytes(const bg_plan* p, int H);
+// With b (forward): also the bias split b2T [H][64] 16-bit, columns p / 32+p the high part /
+// remainder of b[p][h], as bf16, or as fp16 for a plan whose in-degrees exceed 256 (the in-degree
+// table is fp16 then; a finite |b| above 65504 is recorded in `status`).
 cudaError_t band_tc_prep_w(const bg_plan* p, int H, const void* W, int bwd, void* Wk,
-                           cudaStream_t st);
+                           const float* b, __nv_bfloat16* b2T, int* status, cudaStream_t st);
 // Kernel-level entry points used by the fused GGNN steps (operands already in kernel layout):
 //   X: [n_pad][H] bf16 states; Wk: band_tc_prep_w(bwd = 0);
 //   b2T: [H][64] bf16 bias split or NULL.  Outputs (each optional): out fp32 [n][H],
@@ -49,11 +52,6 @@ cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, c
 // ld_out <= 0 means R; batches are R*Cc apart on both sides).
 cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* out, int R, int Cc,
                                 int batch, cudaStream_t st, int64_t ld_out = 0);
-// [H][64] 16-bit: columns p / 32+p hold the high part / remainder of b[p][h], as bf16, or as fp16
-// for a plan whose in-degrees exceed 256 (the in-degree table is fp16 then; a finite |b| above
-// 65504 is recorded in `status`).
-cudaError_t prep_bias_split(const bg_plan* p, const float* b, __nv_bfloat16* b2T, int H,
-                            int* status, cudaStream_t st);
 // Builds and uploads the tensor-core path's plan data (no-op where unsupported); 0 on success.
 int band_tc_upload(bg_plan* p, cudaStream_t st);
 // Host side of band_tc_upload (band_tiles.cpp): the bit-interleaved window chunks of every
