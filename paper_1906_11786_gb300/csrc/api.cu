@@ -336,9 +336,14 @@ extern "C" int bg_plan_upload(bg_plan* p, void* stream) {
   }
   // host vectors must outlive the async copies
   BG_CUDA(cudaStreamSynchronize(st));
-  if (bg::band_tc_upload(p, st) != 0 || bg::super_upload(p, st) != 0) {
+  bool up = false;
+  try {
+    up = bg::band_tc_upload(p, st) == 0 && bg::super_upload(p, st) == 0;
+  } catch (const std::bad_alloc&) {
+  }
+  if (!up) {
     free_device(p);
-    return bg_fail(BG_ENOMEM, "device allocation for the band tiles failed");
+    return bg_fail(BG_ENOMEM, "allocation for the band tiles failed");
   }
   // everything a device call may need to create on this device is created here, so that the
   // allocation-free entry point finds it: the status word, its static scratch, the kernels
@@ -681,13 +686,13 @@ extern "C" int bg_unpack_states(const bg_plan* p, bg_dtype dt, int32_t H, const 
 // ---------------------------------------------------------------------------------- propagate
 static int propagate_fwd_impl(const bg_plan* p, bg_dtype dt, int H, const void* E, const void* W,
                               const float* b, float* Y, char* ws, size_t ws_bytes,
-                              cudaStream_t st) {
+                              cudaStream_t st, bool lists) {
   const int bf = dt == BG_BF16;
   if (bg::band_tc_supported(p, (int)dt, H)) {
     int* status = nullptr;
     BG_TRY(status_word_ptr(&status));
     // the band kernel alone is timed inside (its operand preparation is not)
-    BG_CUDA(bg::band_tc_fwd(p, H, E, W, b, Y, ws, ws_bytes, status, st));
+    BG_CUDA(bg::band_tc_fwd(p, H, E, W, b, Y, ws, ws_bytes, status, st, lists));
     // the supernode rows and columns (Section 6), added to the band's sums
     BG_CUDA(bg::super_fwd(p, bf, H, E, W, b, Y, 0, st));
     return BG_OK;
@@ -728,21 +733,21 @@ extern "C" int bg_band_propagate_fwd(const bg_plan* p, bg_dtype dt, int32_t H, c
   BG_PTR(E, "E"); BG_PTR(W, "W"); BG_OPT_PTR(b, "b"); BG_PTR(Y, "Y"); BG_PTR(ws, "ws");
   if (ws_bytes < fwd_ws(p, dt, H).total) return bg_fail(BG_ECAPACITY, "workspace too small");
   return propagate_fwd_impl(p, dt, H, E, W, b, Y, static_cast<char*>(ws), ws_bytes,
-                            (cudaStream_t)stream);
+                            (cudaStream_t)stream, true);
 }
 
 static int propagate_bwd_band(const bg_plan* p, bg_dtype dt, int H, const void* E, const void* W,
                               const float* dY, float* dE, float* dW, float* db, int accum,
-                              char* ws, size_t ws_bytes, cudaStream_t st);
+                              char* ws, size_t ws_bytes, cudaStream_t st, bool lists);
 
 // dE/dW/db accumulate when accum != 0 (callers zero them first otherwise).
 static int propagate_bwd_impl(const bg_plan* p, bg_dtype dt, int H, const void* E, const void* W,
                               const float* dY, float* dE, float* dW, float* db, int accum,
-                              char* ws, size_t ws_bytes, cudaStream_t st) {
+                              char* ws, size_t ws_bytes, cudaStream_t st, bool lists) {
   const int bf = dt == BG_BF16;
   BwdWs w = bwd_ws(p, dt, H);
   if (ws_bytes < w.total) return bg_fail(BG_ECAPACITY, "workspace too small");
-  BG_TRY(propagate_bwd_band(p, dt, H, E, W, dY, dE, dW, db, accum, ws, ws_bytes, st));
+  BG_TRY(propagate_bwd_band(p, dt, H, E, W, dY, dE, dW, db, accum, ws, ws_bytes, st, lists));
   // the supernode rows and columns (Section 6), added to the band's gradients
   BG_CUDA(bg::super_bwd(p, bf, H, E, W, dY, nullptr, dE, dW, db, ws + w.super, st));
   return BG_OK;
@@ -751,14 +756,15 @@ static int propagate_bwd_impl(const bg_plan* p, bg_dtype dt, int H, const void* 
 // The band part of propagate_bwd_impl.
 static int propagate_bwd_band(const bg_plan* p, bg_dtype dt, int H, const void* E, const void* W,
                               const float* dY, float* dE, float* dW, float* db, int accum,
-                              char* ws, size_t ws_bytes, cudaStream_t st) {
+                              char* ws, size_t ws_bytes, cudaStream_t st, bool lists) {
   const int bf = dt == BG_BF16;
   const size_t n = (size_t)p->n_pad();
   if (bg::band_tc_supported(p, (int)dt, H)) {
     int* status = nullptr;
     BG_TRY(status_word_ptr(&status));
     // the band kernel and the weight-gradient GEMM are timed inside
-    BG_CUDA(bg::band_tc_bwd(p, H, E, W, dY, dE, dW, db, accum, ws, ws_bytes, status, st));
+    BG_CUDA(bg::band_tc_bwd(p, H, E, W, dY, dE, dW, db, accum, ws, ws_bytes, status, st,
+                            lists));
     return BG_OK;
   }
   BwdWs w = bwd_ws(p, dt, H);
@@ -827,7 +833,7 @@ extern "C" int bg_band_propagate_bwd(const bg_plan* p, bg_dtype dt, int32_t H, c
   BG_OPT_PTR(db, "db"); BG_PTR(ws, "ws");
   if (ws_bytes < bwd_ws(p, dt, H).total) return bg_fail(BG_ECAPACITY, "workspace too small");
   return propagate_bwd_impl(p, dt, H, E, W, dY, dE, dW, db, (flags & BG_ACCUM) ? 1 : 0,
-                            static_cast<char*>(ws), ws_bytes, (cudaStream_t)stream);
+                            static_cast<char*>(ws), ws_bytes, (cudaStream_t)stream, true);
 }
 
 // ---------------------------------------------------------------------------------- GGNN
@@ -974,7 +980,8 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
     const void* Et = sv + saved_E_off(p, dt, H, t);
     void* En = sv + saved_E_off(p, dt, H, t + 1);
     float* Yt = reinterpret_cast<float*>(sv + saved_Y_off(p, dt, H, T, t));
-    BG_TRY(propagate_fwd_impl(p, dt, H, Et, prm->W, prm->b, Yt, wsc + w.prop, w.total - w.prop, st));
+    BG_TRY(propagate_fwd_impl(p, dt, H, Et, prm->W, prm->b, Yt, wsc + w.prop, w.total - w.prop, st,
+                              false));
     KTimer tm(BG_KID_GRU_FWD, st);
     BG_TRY(gru_gates_in(p, bf, H, Yt, Et, prm, gi, gh, part, pf, st,
                         tc_gemm_path(dt, H) ? reinterpret_cast<__nv_bfloat16*>(wsc + w.Ybf)
@@ -1244,7 +1251,7 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
     }
     // g += A^T-band backward of the messages; parameter gradients accumulate
     BG_TRY(propagate_bwd_impl(p, dt, H, Et, prm->W, dX, g, gr->dW, gr->db, 1, wsc + w.prop,
-                              w.total - w.prop, st));
+                              w.total - w.prop, st, false));
     if (t > 0) {
       // next iteration reads gin while writing g: keep them distinct
       BG_CUDA(cudaMemcpyAsync(dX, g, sizeof(float) * (size_t)n * H, cudaMemcpyDeviceToDevice, st));

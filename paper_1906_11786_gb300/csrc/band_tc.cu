@@ -46,6 +46,7 @@
 
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -741,6 +742,595 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
   }
 }
 
+// ------------------------------------------------------------------------------ gathered band
+// The same products for a sparse band.  A 128-row tile of a program graph holds a few hundred
+// edges per type where the dense product multiplies 128 x 128 C1 entries, so pre_p is summed
+// from the edges instead: a warp takes 16 rows and the edges of one type 16 at a time,
+//     pre[16 x SW] += T [16 x 16] X[16 x SW],
+// where the B operand is the 16 source rows, named one by one in ldmatrix's addresses (a gather
+// from the row-major window in shared memory), and T holds a 1 where an edge ends in a row.  The
+// accumulator fragment is the register layout of tcgen05.st.16x256b, so pre_p goes to TMEM as the A
+// operand of the second product, which is issued exactly as in k_band_tc.  A sum of a few bf16 values
+// is nearly always exact in fp32, so the results agree with the dense kernel's but for the rare sum
+// that is not (1e-10 to 1e-6 of the norm).  A GGNN step rounds Y to bf16 and feeds it back, where even
+// that grows through the layers; its saved activations and gradients do not depend on how dense a
+// plan is, so the GGNN steps stay on the dense kernel.
+//
+// Bound: latency along each warp's chain (words, ldmatrix, products, TMEM store), with the shared-memory
+// and tensor pipes each about half busy at 16 warps of 80 registers.  A step (4 ldmatrix.x4, 8 mma.sync)
+// takes 26 cycles of the SM with conflict-free rows, 44 with random ones, which is why the plan deals
+// edges into sets of 8 whose rows differ mod 8.  S = 512, H = 64, 131k nodes, 52 edges per node: 97 us
+// against the dense kernel's 440; S = 256, H = 128, 20k nodes backward: 60 us against 86.
+//
+// Roles (24 warps, one CTA per SM, persistent over the same items as k_band_tc):
+//   warp 0       TMA producer: state windows, W tiles, deg, bias
+//   warp 1       TMEM allocator and issuer of the second product and the bias product
+//   warps 4-7    epilogue, Y from TMEM (two accumulators up to H = 128, so it overlaps)
+//   warps 8-23   gather: 8 warps of 16 rows for the even types, 8 for the odd ones
+template <int H, bool BWD>
+struct GaCfg {
+  static constexpr int SW = H < 64 ? 32 : 64;
+  static constexpr int NH = H / SW;
+  static constexpr int NT = SW / 8;                     // accumulator n-tiles
+  static constexpr int YC = H < 64 ? 64 : H;            // TMEM columns of one Y
+  static constexpr int NY = H <= 128 ? 2 : 1;
+  static constexpr int UC = 64;                         // columns of one pre_p unit
+  static constexpr int UCOL = NY * YC;
+  static constexpr int NU0 = (512 - UCOL) / UC;
+  static constexpr int NU = NU0 > 6 ? 6 : NU0;
+  // W stages as in k_band_tc: fp32 K-columns of W_p^T in 32-column atoms of H rows
+  static constexpr int WK = H <= 128 ? SW : 32;
+  static constexpr int WJ = SW / WK;
+  static constexpr int WSTAGE = (WK / 32) * H * 128;
+  static constexpr bool BIAS = !BWD;                    // bias as a product
+  static constexpr int DEG = BIAS ? kTile * 128 : 0;
+  static constexpr int B2 = BIAS ? H * 128 : 0;
+  static constexpr int DM = BWD ? 16 * 16 * SW * 2 : 0; // a 16-row staging tile per gather warp
+  static constexpr int FIXED = DEG + B2 + DM + 1024 + 1024;
+  static constexpr int THREADS = 32 * 24;
+  static_assert(NU >= 2, "pre_p units");
+};
+
+struct GaBars {
+  uint64_t x_full[2], x_empty[2];
+  uint64_t w_full[4], w_empty[4];
+  uint64_t deg_full, deg_empty;
+  uint64_t b2_full;
+  uint64_t u_full[6], u_empty[6];
+  uint64_t y_full[2], y_empty[2];
+  uint64_t drain;
+  uint32_t tmem_base;
+  int abort;
+};
+static_assert(sizeof(GaBars) <= 1024, "barriers");
+
+// Shared-memory split of one launch: window rows (and boxes to load them in), buffers of each ring.
+struct GaLayout {
+  int lo, rows, box_rows, nxb, nw;
+};
+
+// Windows and W stages that fit, or nxb = 0.
+template <int H, bool BWD>
+GaLayout ga_layout(int lo, int rows) {
+  using C = GaCfg<H, BWD>;
+  GaLayout g{};
+  g.lo = lo;
+  g.rows = rows;
+  g.box_rows = rows / ((rows + 255) / 256);  // the plan made them equal
+  const int win = (rows + 8) * 128;
+  // A W stage takes about 1.5 us from release to refill (L2), so the ring's depth over that time caps
+  // the jobs (at two 16 KB stages 70 us a launch at packed64); a second window hides one window load
+  // per tile.
+  constexpr int kTry[8][2] = {{2, 4}, {2, 3}, {1, 4}, {1, 3}, {2, 2}, {1, 2}, {2, 1}, {1, 1}};
+  for (auto& t : kTry)
+    if (t[0] * win + t[1] * C::WSTAGE + C::FIXED <= 232448) {
+      g.nxb = t[0];
+      g.nw = t[1];
+      break;
+    }
+  return g;
+}
+
+__device__ __forceinline__ void ldsm4t(uint32_t* r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void stsm4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a),
+               "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
+__device__ __forceinline__ void mma16816(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma16816_first(float* c, const uint32_t* a, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+// accumulator fragments of 16 rows to 64 / 32 fp32 columns of TMEM
+__device__ __forceinline__ void st_16x256b(uint32_t t, const float (&r)[32]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(t),
+      "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]),
+      "f"(r[8]), "f"(r[9]), "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15]),
+      "f"(r[16]), "f"(r[17]), "f"(r[18]), "f"(r[19]), "f"(r[20]), "f"(r[21]), "f"(r[22]),
+      "f"(r[23]), "f"(r[24]), "f"(r[25]), "f"(r[26]), "f"(r[27]), "f"(r[28]), "f"(r[29]),
+      "f"(r[30]), "f"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ void st_16x256b(uint32_t t, const float (&r)[16]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16};" ::"r"(t),
+      "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]),
+      "f"(r[8]), "f"(r[9]), "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
+      : "memory");
+}
+// One gather warp's blocks of four steps in the order of their use: the passes of the CTA's items, one
+// per slice of the state.  Lane l holds the block range of pass `held` + l, so that moving on to the
+// next pass touches no memory.
+struct StepBlocks {
+  const uint4* words;  // this lane's words of block 0
+  uint32_t at, end;    // next block to request, end of its pass
+  int pass, passes;    // pass of `at`, passes in all
+  int held;
+  uint32_t sb, se;
+  __device__ __forceinline__ void fill(const Sched& sc, const uint32_t* off, int P, int jobs, int g,
+                                       int b, int first, int lane) {
+    int skip = first + lane, n = 0;
+    held = first;
+    sb = se = 0;
+    for (int w = blockIdx.x; w < sc.n_items; w += gridDim.x) {
+      int tile, j0, j1, part;
+      item_of(sc, w, jobs, tile, j0, j1, part);
+      const int h0 = j0 / P, cnt = (j1 - 1) / P - h0 + 1;
+      if (skip >= 0 && skip < cnt) {
+        const int jh = (h0 + skip) * P, pa = max(j0 - jh, 0), pb = min(j1 - jh, P);
+        const int p0 = pa + ((pa ^ g) & 1);
+        if (p0 < pb) {
+          const uint32_t* o = off + ((size_t)tile * 8 + b) * (P + 1) + (g ? (P + 1) / 2 : 0) + (p0 >> 1);
+          sb = o[0];
+          se = o[(pb - p0 + 1) >> 1];
+        }
+      }
+      skip -= cnt;
+      n += cnt;
+    }
+    passes = n;
+  }
+  __device__ __forceinline__ uint4 request(const Sched& sc, const uint32_t* off, int P, int jobs, int g,
+                                           int b, int lane) {
+    while (at == end) {
+      if (++pass >= passes) {
+        pass = passes;
+        return make_uint4(0u, 0u, 0u, 0u);  // past the end: never used
+      }
+      if (pass - held == 32) fill(sc, off, P, jobs, g, b, pass, lane);
+      __syncwarp();
+      at = __shfl_sync(0xffffffffu, sb, pass - held);
+      end = __shfl_sync(0xffffffffu, se, pass - held);
+    }
+    return __ldg(words + (size_t)(at++) * 32);
+  }
+};
+
+template <int H, bool BWD>
+__global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
+    k_band_gather(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
+                  const __grid_constant__ CUtensorMap tm_deg,
+                  const __grid_constant__ CUtensorMap tm_b2, const uint32_t* __restrict__ words,
+                  const uint32_t* __restrict__ off, float* __restrict__ out,
+                  __nv_bfloat16* __restrict__ outb, __nv_bfloat16* __restrict__ outT,
+                  int64_t ld_outT, __nv_bfloat16* __restrict__ dM, const Sched sc, const GaLayout lay, int n, int P, int has_bias,
+                  int bias_f16, int accumulate, int* status) {
+  using C = GaCfg<H, BWD>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~uintptr_t(1023));
+  const int xbytes = (lay.rows + 8) * 128;
+  uint8_t* xwin = smem;
+  uint8_t* wring = xwin + lay.nxb * xbytes;
+  uint8_t* degs = wring + lay.nw * C::WSTAGE;
+  uint8_t* b2s = degs + C::DEG;
+  uint8_t* dms = b2s + C::B2;
+  GaBars* bars = reinterpret_cast<GaBars*>(dms + C::DM);
+  volatile int* abort = &bars->abort;
+  const int jobs = C::NH * P;
+  const bool bias_mma = C::BIAS && has_bias;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->x_full[i], 1); mbar_init(&bars->x_empty[i], 16);
+      mbar_init(&bars->y_full[i], 1); mbar_init(&bars->y_empty[i], 4);
+    }
+    for (int i = 0; i < 4; ++i) { mbar_init(&bars->w_full[i], 1); mbar_init(&bars->w_empty[i], 1); }
+    for (int i = 0; i < 6; ++i) { mbar_init(&bars->u_full[i], 8); mbar_init(&bars->u_empty[i], 1); }
+    mbar_init(&bars->b2_full, 1);
+    mbar_init(&bars->deg_full, 1);
+    mbar_init(&bars->deg_empty, 1);
+    mbar_init(&bars->drain, 1);
+    bars->abort = 0;
+    fence_mbar_init();
+  }
+  // the zero rows after each window, which padding entries name
+  for (int i = threadIdx.x; i < lay.nxb * 64; i += C::THREADS)
+    *reinterpret_cast<uint4*>(xwin + (i >> 6) * xbytes + lay.rows * 128 + (i & 63) * 16) =
+        make_uint4(0u, 0u, 0u, 0u);
+  if (warp == 1) {
+    tmem_alloc(&bars->tmem_base, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  // TMEM is held: the next kernel in the stream may be scheduled on SMs as they free up
+  grid_dep_launch();
+  const uint32_t tmem = bars->tmem_base;
+
+  // let this CTA's own copies land before shared memory is released (bounded)
+  auto settle = [](uint64_t* bar, uint32_t uses) {
+    if (!uses) return;
+    for (uint32_t t = 0; t < (1u << 22) && !mbar_try(bar, (uses - 1) & 1); ++t) {
+    }
+  };
+  if (warp == 0 && lane == 0) {
+    // ------------------------------------------------------------------ W producer
+    tma_prefetch_desc(&tm_w);
+    grid_dep_wait();  // W may be the previous kernel's output
+    uint32_t wi = 0, wph = 0, n_w[4] = {0, 0, 0, 0};
+    bool ok = true;
+    for (int w = blockIdx.x; w < sc.n_items && ok && !*abort; w += gridDim.x) {
+      int k, j0, j1, part;
+      item_of(sc, w, jobs, k, j0, j1, part);
+      int hh = j0 / P, p = j0 - hh * P;
+      for (int jb = j0; jb < j1 && ok; ++jb, p = p + 1 == P ? (++hh, 0) : p + 1) {
+        for (int wj = 0; wj < C::WJ; ++wj) {
+          if (!mbar_wait(&bars->w_empty[wi], (wph & 1) ^ 1, status, 153, abort)) {
+            ok = false;
+            break;
+          }
+          ++n_w[wi];
+          mbar_expect_tx(&bars->w_full[wi], C::WSTAGE);
+          for (int a = 0; a < C::WK / 32; ++a)
+            tma_load_2d(wring + wi * C::WSTAGE + a * H * 128, &tm_w, &bars->w_full[wi],
+                        C::SW * hh + C::WK * wj + 32 * a, p * H);
+          if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
+        }
+      }
+    }
+    if (*abort)
+      for (int q = 0; q < 4; ++q) settle(&bars->w_full[q], n_w[q]);
+  } else if (warp == 2 && lane == 0) {
+    // ------------------------------------------------------------------ window producer
+    // (its own thread: behind the W ring a window was requested only four jobs before its first use,
+    // and the gather warps run six jobs ahead of the issuer)
+    tma_prefetch_desc(&tm_x);
+    // states and the bias split may be the previous kernel's output (in-degrees are plan data)
+    grid_dep_wait();
+    if (bias_mma) {
+      mbar_expect_tx(&bars->b2_full, C::B2);
+      tma_load_2d(b2s, &tm_b2, &bars->b2_full, 0, 0);
+    }
+    uint32_t xi = 0, di = 0;  // windows and deg tiles so far
+    uint32_t n_x[2] = {0, 0}, n_deg = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < sc.n_items && ok && !*abort; w += gridDim.x) {
+      int k, j0, j1, part;
+      item_of(sc, w, jobs, k, j0, j1, part);
+      const int row0 = k * kTile;
+      for (int jb = j0; jb < j1; jb = (jb / P + 1) * P, ++xi) {
+        const int xb = lay.nxb == 2 ? (xi & 1) : 0, xn = lay.nxb == 2 ? (xi >> 1) : xi;
+        if (!mbar_wait(&bars->x_empty[xb], (xn & 1) ^ 1, status, 151, abort, 32)) {
+          ok = false;
+          break;
+        }
+        ++n_x[xb];
+        mbar_expect_tx(&bars->x_full[xb], lay.rows * 128);
+        for (int r = 0; r < lay.rows; r += lay.box_rows)
+          tma_load_2d(xwin + xb * xbytes + r * 128, &tm_x, &bars->x_full[xb], C::SW * (jb / P),
+                      row0 - lay.lo + r);
+      }
+      if (ok && bias_mma && part <= 0) {
+        if (!mbar_wait(&bars->deg_empty, (di & 1) ^ 1, status, 152, abort, 32)) break;
+        ++n_deg;
+        ++di;
+        mbar_expect_tx(&bars->deg_full, C::DEG);
+        tma_load_2d(degs, &tm_deg, &bars->deg_full, 0, row0);
+      }
+    }
+    if (*abort) {
+      for (int q = 0; q < 2; ++q) settle(&bars->x_full[q], n_x[q]);
+      settle(&bars->deg_full, n_deg);
+      if (bias_mma) settle(&bars->b2_full, 1);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ issuer
+    // Y (+)= pre_p W_p over the jobs (K = the SW rows of W_p of the job's slice), then the bias
+    const bool leader = elect_one_sync();
+    const uint32_t idescb = bias_f16 ? idesc_f16_f32(kTile, H) : idesc_bf16_f32(kTile, H);
+    constexpr uint32_t idesc = idesc_tf32_f32(kTile, H);
+    uint32_t u = 0, uph = 0, wi = 0, wph = 0, di = 0;
+    bool ok = true;
+    int i = 0;
+    for (int w = blockIdx.x; w < sc.n_items && ok; w += gridDim.x, ++i) {
+      int k, j0, j1, part;
+      item_of(sc, w, jobs, k, j0, j1, part);
+      const int yb = i % C::NY;
+      const uint32_t ycol = tmem + yb * C::YC;
+      for (int jb = j0; jb < j1 && ok; ++jb) {
+        if (!mbar_wait(&bars->u_full[u], uph & 1, status, 258, abort) ||
+            (jb == j0 && !mbar_wait(&bars->y_empty[yb], ((i / C::NY) & 1) ^ 1, status, 253, abort))) {
+          ok = false;
+          break;
+        }
+        const uint32_t ucol = tmem + C::UCOL + u * C::UC;
+        for (int wj = 0; wj < C::WJ; ++wj) {
+          if (!mbar_wait(&bars->w_full[wi], wph & 1, status, 252, abort)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t wbase = smem_u32(wring + wi * C::WSTAGE);
+          const bool first = jb == j0 && wj == 0;
+#pragma unroll
+          for (int kk = 0; kk < C::WK / 8; ++kk)
+            if (leader)
+              mma_ts_tf32(ycol, ucol + C::WK * wj + kk * 8,
+                          desc_sw128_kmajor(wbase + (kk / 4) * H * 128 + (kk % 4) * 32), idesc,
+                          (first && kk == 0) ? 0u : 1u);
+          if (leader) tc_commit(&bars->w_empty[wi]);
+          if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
+        }
+        if (!ok) break;
+        if (leader) tc_commit(&bars->u_empty[u]);
+        if (++u == (uint32_t)C::NU) u = 0, ++uph;
+      }
+      if (!ok) break;
+      if (bias_mma && part <= 0) {
+        if (!mbar_wait(&bars->deg_full, di & 1, status, 256, abort)) break;
+        if (di == 0 && !mbar_wait(&bars->b2_full, 0, status, 257, abort)) break;
+        ++di;
+        tc_fence_after();
+        const uint32_t dbase = smem_u32(degs), bbase = smem_u32(b2s);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          if (leader)
+            mma_ss(ycol, desc_sw128_kmajor(dbase + kk * 32), desc_sw128_kmajor(bbase + kk * 32),
+                   idescb, 1u);
+        if (leader) tc_commit(&bars->deg_empty);
+      }
+      if (leader) tc_commit(&bars->y_full[yb]);
+    }
+    // a CTA whose items were all later slices of split tiles never used the bias rows it loaded:
+    // let that copy land before the CTA's shared memory is released
+    if (bias_mma && di == 0) mbar_wait(&bars->b2_full, 0, status, 259, abort);
+    drain_mmas(leader, &bars->drain);
+  } else if (warp >= 4 && warp < 8) {
+    // ------------------------------------------------------------------ epilogue
+    grid_dep_wait();  // outputs (and the accumulated dE) may still be in use by the previous kernel
+    const int r = (warp & 3) * 32 + lane;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    int i = 0;
+    for (int w = blockIdx.x; w < sc.n_items && !*abort; w += gridDim.x, ++i) {
+      int k, j0, j1, part;
+      item_of(sc, w, jobs, k, j0, j1, part);
+      const int row = k * kTile + r, yb = i % C::NY;
+      const bool live = row < n;
+      const int asl = (!BWD && sc.addend && part < 0 && live) ? sc.slot[row] : -1;
+      if (!mbar_wait(&bars->y_full[yb], (i / C::NY) & 1, status, 452, abort, 64)) break;
+      tc_fence_after();
+#pragma unroll 1
+      for (int h0 = 0; h0 < H; h0 += 32) {
+        __syncwarp();
+        uint32_t v[32];
+        tmem_ld32(tmem + lane_base + yb * C::YC + h0, v);
+        tmem_wait_ld();
+        if (h0 + 32 >= H) {
+          tc_fence_before();
+          warp_arrive(&bars->y_empty[yb]);
+        }
+        if (!live) continue;
+        if (asl >= 0) {
+          const float* ad = sc.addend + (size_t)asl * H + h0;
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ad[j]);
+        }
+        if (part >= 0) {
+          // a slice of a split tile: its partial Y, summed with the other slices' by the fix-up
+          float4* o = reinterpret_cast<float4*>(
+              sc.part + ((size_t)part * sc.part_rows + (size_t)(k - sc.n_full) * kTile + r) * H + h0);
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            o[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                               __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+          continue;
+        }
+        if (out) {
+          float4* o = reinterpret_cast<float4*>(out + (size_t)row * H + h0);
+#pragma unroll
+          for (int jh = 0; jh < 8; jh += 4) {
+            float4 prev[4];
+            if (accumulate) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) prev[j] = o[jh + j];
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t* vj = v + 4 * (jh + j);
+              float4 a = make_float4(__uint_as_float(vj[0]), __uint_as_float(vj[1]),
+                                     __uint_as_float(vj[2]), __uint_as_float(vj[3]));
+              if (accumulate) {
+                a.x += prev[j].x; a.y += prev[j].y; a.z += prev[j].z; a.w += prev[j].w;
+              }
+              o[jh + j] = a;
+            }
+          }
+        }
+        if (outb || outT) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            pk[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+          if (outb) {
+            uint4* ob = reinterpret_cast<uint4*>(outb + (size_t)row * H + h0);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              ob[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+          }
+          if (outT) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              __nv_bfloat16* d = outT + (size_t)(h0 + 2 * j) * ld_outT + row;
+              d[0] = __ushort_as_bfloat16((unsigned short)(pk[j] & 0xFFFFu));
+              d[ld_outT] = __ushort_as_bfloat16((unsigned short)(pk[j] >> 16));
+            }
+          }
+        }
+      }
+    }
+  } else if (warp >= 8) {
+    // ------------------------------------------------------------------ gather
+    const int gw = warp - 8, g = gw >> 3;            // types of parity g
+    const int b = 2 * (warp & 3) + ((gw >> 2) & 1);  // 16-row group within the tile
+    const uint32_t tlane = (uint32_t)(16 * b) << 16;
+    // staging tile of 16 dM_p rows, and this lane's row and chunk parity in stmatrix's x4 form
+    const uint32_t dmw = smem_u32(dms) + gw * 16 * C::SW * 2;
+    const int srow = (lane & 7) + (lane & 8), shi = lane >> 4;
+    auto swz = [](int row, int ch) { return C::SW == 64 ? (ch ^ (row & 7)) : (ch ^ ((row >> 1) & 3)); };
+    StepBlocks sb{reinterpret_cast<const uint4*>(words) + lane, 0, 0, -1, 0, 0, 0, 0};
+    sb.fill(sc, off, P, jobs, g, b, 0, lane);
+    uint4 nx = sb.request(sc, off, P, jobs, g, b, lane);
+    uint4 nx2 = sb.request(sc, off, P, jobs, g, b, lane);
+    // the unit of the last job, until its store to TMEM is known to be done: the wait is put off
+    // until the next job's first products are under way
+    int pending = -1;
+    auto flush = [&]() {
+      if (pending >= 0) {
+        tmem_wait_st();
+        tc_fence_before();
+        warp_arrive(&bars->u_full[pending]);
+        pending = -1;
+      }
+    };
+    uint32_t u = 0, uph = 0, xi = 0;  // the next job's pre_p unit and its phase, windows so far
+    auto unit_add = [&](int d) {      // d <= 2 <= NU
+      u += d;
+      if (u >= (uint32_t)C::NU) u -= C::NU, uph ^= 1;
+    };
+    bool ok = true;
+    for (int w = blockIdx.x; w < sc.n_items && ok && !*abort; w += gridDim.x) {
+      int k, j0, j1, part;
+      item_of(sc, w, jobs, k, j0, j1, part);
+      int hh = j0 / P;
+      for (int jb = j0; jb < j1 && ok; ++xi, ++hh) {
+        const int pa = jb - hh * P, pb = min(j1 - hh * P, P);
+        const int xb = lay.nxb == 2 ? (xi & 1) : 0, xn = lay.nxb == 2 ? (xi >> 1) : xi;
+        if (!mbar_wait(&bars->x_full[xb], xn & 1, status, 351, abort, 32)) { ok = false; break; }
+        __syncwarp();
+        const uint32_t xaddr = smem_u32(xwin + xb * xbytes);
+        int p = pa + ((pa ^ g) & 1);
+        unit_add(p - pa);
+        bool begun = false;
+        float acc[4 * C::NT];
+        while (p < pb) {
+          // up to four steps of 16 edges
+          const uint4 cur = nx;
+          nx = nx2;
+          nx2 = sb.request(sc, off, P, jobs, g, b, lane);
+          auto step = [&](uint32_t word, auto first) {
+            const uint32_t ad = xaddr + (word & 0x3FFFFu), bits = (word >> 24) * 4097u;
+            uint32_t bq[2 * C::NT], a[4];
+#pragma unroll
+            for (int j = 0; j < C::NT / 2; ++j) ldsm4t(bq + 4 * j, ad ^ (j << 5));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) a[j] = expand_pair(bits, j);
+#pragma unroll
+            for (int j = 0; j < C::NT; ++j) {
+              if constexpr (decltype(first)::value)
+                mma16816_first(acc + 4 * j, a, bq[2 * j], bq[2 * j + 1]);
+              else
+                mma16816(acc + 4 * j, a, bq[2 * j], bq[2 * j + 1]);
+            }
+          };
+          if (begun) {
+            step(cur.x, std::false_type{});
+          } else {
+            step(cur.x, std::true_type{});
+            flush();
+          }
+          const uint32_t more = (cur.x / kGatherMore) & 3u;
+          if (more > 0) {
+            step(cur.y, std::false_type{});
+            if (more > 1) {
+              step(cur.z, std::false_type{});
+              if (more > 2) step(cur.w, std::false_type{});
+            }
+          }
+          begun = true;
+          if (!(cur.x & kGatherLast)) continue;
+          // the type's sums of these 16 rows are complete
+          begun = false;
+          if constexpr (BWD) {
+            // dM_p (bf16) through the warp's staging tile, so that rows leave as whole lines.  (As a
+            // bulk store, the proxy fence before it waited for the words on their way.)
+#pragma unroll
+            for (int j = 0; j < C::NT; j += 2)
+              stsm4(dmw + srow * C::SW * 2 + swz(srow, j + shi) * 16, pack_bf16(acc[4 * j], acc[4 * j + 1]),
+                    pack_bf16(acc[4 * j + 2], acc[4 * j + 3]), pack_bf16(acc[4 * j + 4], acc[4 * j + 5]),
+                    pack_bf16(acc[4 * j + 6], acc[4 * j + 7]));
+          }
+          if (!mbar_wait(&bars->u_empty[u], uph ^ 1, status, 352, abort, 32)) {
+            ok = false;
+            break;
+          }
+          __syncwarp();
+          tc_fence_after();
+          st_16x256b(tmem + tlane + C::UCOL + u * C::UC, acc);
+          pending = (int)u;
+          if constexpr (BWD) {
+            constexpr int CH = C::SW / 8;  // 16-byte chunks per row
+            uint4* d = reinterpret_cast<uint4*>(dM + ((size_t)(k * kTile + 16 * b) * P + p) * H + C::SW * hh);
+#pragma unroll
+            for (int q = 0; q < C::SW / 16; ++q) {
+              const int row = (q * 32 + lane) / CH, ch = lane % CH;
+              uint4 v;
+              asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];"
+                           : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                           : "r"(dmw + row * C::SW * 2 + swz(row, ch) * 16)
+                           : "memory");
+              d[(size_t)row * (P * H / 8) + ch] = v;
+            }
+            __syncwarp();  // the tile is free for the next 16 rows
+          }
+          unit_add(min(2, pb - p));
+          p += 2;
+        }
+        if (!ok) break;
+        flush();
+        warp_arrive(&bars->x_empty[xb]);
+        jb += pb - pa;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
 // ------------------------------------------------------------------------------------ prep
 // out[c][r] = bf16(in[r][c]) for an R x Cc row-major input (batched over blockIdx.z)
 template <typename T>
@@ -978,6 +1568,104 @@ cudaError_t launch(const bg_plan* p, const CUtensorMap& tx, const CUtensorMap& t
 #undef BG_BAND_S
 }
 
+// Operands of a launch of the gathered kernel (band_tc.h gives their meanings).
+struct GaOps {
+  const __nv_bfloat16* X;
+  const void* Wk;
+  const __nv_bfloat16* b2T;
+  float* out;
+  __nv_bfloat16 *outb, *outT;
+  int64_t ld_outT;
+  __nv_bfloat16* dM;
+  int accumulate;
+  float* split;
+  const float* addend;
+};
+
+template <int H, bool BWD>
+cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStream_t st) {
+  using C = GaCfg<H, BWD>;
+  const int n = p->n_pad(), P = p->P;
+  const GaLayout lay = ga_layout<H, BWD>(p->g_lo[BWD], p->g_rows[BWD]);
+  if (!lay.nxb) return cudaErrorInvalidValue;
+  CUtensorMap tx, tw, tdeg, tb2;
+  if (!make_map_ld(&tx, o.X, n, H, H, lay.box_rows) ||
+      !make_map_w(&tw, o.Wk, P, H))
+    return cudaErrorInvalidValue;
+  const bool bias_mma = C::BIAS && o.b2T != nullptr;
+  tdeg = tb2 = tx;
+  if (bias_mma && (!make_map(&tdeg, p->d_deg2, n, 64, kTile) || !make_map(&tb2, o.b2T, H, 64, H)))
+    return cudaErrorInvalidValue;
+  const int smem = lay.nxb * (lay.rows + 8) * 128 + lay.nw * C::WSTAGE + C::FIXED;
+  cudaError_t e = cudaFuncSetAttribute(k_band_gather<H, BWD>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int n_tiles = (n + kTile - 1) / kTile, sms = num_sms();
+  Sched sc = make_sched(n_tiles, C::NH * P, sms, o.split != nullptr && n % kTile == 0);
+  sc.part = o.split;
+  sc.addend = BWD ? nullptr : o.addend;
+  sc.slot = p->d_sin_slot;
+  e = launch_pdl(k_band_gather<H, BWD>, dim3(std::min(sc.n_items, sms)), dim3(C::THREADS),
+                 smem, st, tx, tw, tdeg, tb2, (const uint32_t*)p->d_glist[BWD],
+                 (const uint32_t*)p->d_goff[BWD], o.out, o.outb, o.outT, o.ld_outT, o.dM, sc, lay, n, P,
+                 bias_mma ? 1 : 0, p->max_deg > 256 ? 1 : 0, o.accumulate, status);
+  note_launch();
+  if (e != cudaSuccess || sc.ksplit == 1) return e;
+  const int64_t n4 = (int64_t)sc.part_rows * H / 4;
+  e = launch_pdl(k_band_split_fixup, dim3((unsigned)std::min<int64_t>((n4 + 255) / 256, 2048)),
+                 dim3(256), 0, st, (const float*)o.split, sc.ksplit, sc.part_rows,
+                 sc.n_full * kTile, H, o.out, o.outb, o.outT, o.ld_outT, o.accumulate, sc.addend,
+                 sc.slot);
+  note_launch();
+  return e;
+}
+
+template <bool BWD>
+cudaError_t launch_gather_h(const bg_plan* p, int H, const GaOps& o, int* status, cudaStream_t st) {
+  switch (H) {
+    case 32: return launch_gather<32, BWD>(p, o, status, st);
+    case 64: return launch_gather<64, BWD>(p, o, status, st);
+    case 128: return launch_gather<128, BWD>(p, o, status, st);
+    default: return launch_gather<256, BWD>(p, o, status, st);
+  }
+}
+
+template <bool BWD>
+bool gather_fits(int lo, int rows, int H) {
+  switch (H) {
+    case 32: return ga_layout<32, BWD>(lo, rows).nxb > 0;
+    case 64: return ga_layout<64, BWD>(lo, rows).nxb > 0;
+    case 128: return ga_layout<128, BWD>(lo, rows).nxb > 0;
+    case 256: return ga_layout<256, BWD>(lo, rows).nxb > 0;
+    default: return false;
+  }
+}
+
+// The average number of gather steps per (tile, type) up to which the edge lists are used (0: never).
+// The gathered kernel's time follows the steps and hardly the block size, the dense one's follows the
+// window's chunks and not the edges.  Measured on 48 graphs, 61.7k nodes, 20 types, at 20 and 160
+// edges per node, lists against chunks in us a launch: S = 256 forward 34 and 68 against 93 (H = 32),
+// 49 and 104 against 101 (64), 94 and 211 against 225 (128), backward 47 and 76 against 95, 65 and 115
+// against 103, 125 and 238 against 222; S = 512 forward 37 and 74 against 183, 50 and 107 against 225,
+// 100 and 214 against 495, backward 50 and 82 against 186, 68 and 120 against 187, 146 and 241 against
+// 560.  The entries lie where the measured lines cross, or at S = 512 at half the distance beyond the
+// last measured point (about 80 steps).  At S = 128 the two are within 7% of one another at H = 64 and
+// 52 edges per node, and the lists are not built there.
+int gather_max_steps(int S, int H, bool bwd) {
+  if (S != 256 && S != 512) return 0;
+  const int h = H == 32 ? 0 : H == 64 ? 1 : H == 128 ? 2 : 3;
+  static constexpr int kMax[2][2][4] = {{{100, 70, 80, 0}, {80, 60, 68, 0}},      // S = 256
+                                        {{200, 160, 200, 0}, {200, 110, 200, 0}}};  // S = 512
+  return kMax[S == 512][bwd][h];
+}
+
+// Shapes whose propagation runs on the fused tensor-core kernels (and rounds where they round).
+bool tc_shape_ok(int S, int H) {
+  return ((H == 32 || H == 64 || H == 128) &&
+          (S == 32 || S == 64 || S == 128 || S == 256 || S == 512)) ||
+         (H == 256 && (S == 32 || S == 64 || S == 128));
+}
+
 }  // namespace
 
 // Row-major fp32 [rows][cols], boxes of 32 columns (one 128-byte swizzle row) x box_rows.
@@ -1041,13 +1729,13 @@ bool make_map_3d(CUtensorMap* m, const void* base, uint64_t batch, uint64_t rows
 }
 
 bool band_tc_supported(const bg_plan* p, int dtype, int H) {
-  if (!p || dtype != 1 || p->P > 32 || p->n_pad() % kTile) return false;
-  const bool shape = ((H == 32 || H == 64 || H == 128) &&
-                      (p->S == 32 || p->S == 64 || p->S == 128 || p->S == 256 || p->S == 512)) ||
-                     (H == 256 && (p->S == 32 || p->S == 64 || p->S == 128));
-  return shape && p->d_maskI && p->d_maskTI && p->d_deg2 && p->max_deg < 2048 &&
-         encode_fn() != nullptr;
+  if (!p || dtype != 1 || p->P > 32 || p->n_pad() % kTile || !tc_shape_ok(p->S, H)) return false;
+  return p->d_maskI && p->d_maskTI && p->d_deg2 && p->max_deg < 2048 && encode_fn() != nullptr;
 }
+
+namespace {
+bool use_lists(const bg_plan* p, int H, bool bwd) { return p->list_h[bwd] >> (H / 32) & 1; }
+}  // namespace
 
 size_t band_tc_w_bytes(const bg_plan* p, int H) {
   return al256((size_t)p->P * H * H * 4);
@@ -1090,9 +1778,12 @@ size_t band_tc_split_floats(const bg_plan* p, int H) {
 cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, const void* Wk,
                              const __nv_bfloat16* b2T, const float* b32, float* out,
                              __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
-                             float* split, const float* addend, int* status,
-                             cudaStream_t st) {
+                             float* split, const float* addend, int* status, cudaStream_t st,
+                             bool lists) {
   const int n = p->n_pad(), P = p->P;
+  if (lists && use_lists(p, H, false))
+    return launch_gather_h<false>(
+        p, H, GaOps{X, Wk, b2T, out, outb, outT, ld_outT, nullptr, 0, split, addend}, status, st);
   CUtensorMap tx, tw, tdeg, tb2;
   if (!make_map_box(&tx, X, n, H, H, H < 64 ? 32 : 64, kTile) ||
       !make_map_w(&tw, Wk, P, H) || !make_map(&tdeg, p->d_deg2, n, 64, kTile) ||
@@ -1113,8 +1804,12 @@ cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, co
 
 cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, const void* Wk,
                              float* dE, int accumulate, __nv_bfloat16* dM, float* split,
-                             int* status, cudaStream_t st) {
+                             int* status, cudaStream_t st, bool lists) {
   const int n = p->n_pad(), P = p->P;
+  if (lists && use_lists(p, H, true))
+    return launch_gather_h<true>(
+        p, H, GaOps{dY, Wk, nullptr, dE, nullptr, nullptr, 0, dM, accumulate, split, nullptr},
+        status, st);
   CUtensorMap tx, tw, tdm;
   const int sw = H < 64 ? 32 : 64;
   if (!make_map_box(&tx, dY, n, H, H, sw, kTile) || !make_map_w(&tw, Wk, P, H) ||
@@ -1149,7 +1844,8 @@ cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* ou
 }
 
 cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, const float* b,
-                        float* Y, char* ws, size_t ws_bytes, int* status, cudaStream_t st) {
+                        float* Y, char* ws, size_t ws_bytes, int* status, cudaStream_t st,
+                        bool lists) {
   if (ws_bytes < band_tc_fwd_ws_bytes(p, 1, H)) return cudaErrorInvalidValue;
   const int n = p->n_pad();
   void* WT = ws + al256((size_t)n * H * 2);
@@ -1162,12 +1858,13 @@ cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, c
   if (e != cudaSuccess) return e;
   ProfSpan span(BG_KID_BAND_FWD, st);
   return band_tc_fwd_core(p, H, static_cast<const __nv_bfloat16*>(E), WT, b ? b2T : nullptr, b, Y,
-                          nullptr, nullptr, 0, band_tc_split_floats(p, H) ? split : nullptr, nullptr, status, st);
+                          nullptr, nullptr, 0, band_tc_split_floats(p, H) ? split : nullptr, nullptr, status, st,
+                          lists);
 }
 
 cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, const float* dY,
                         float* dE, float* dW, float* db, int accum, char* ws, size_t ws_bytes,
-                        int* status, cudaStream_t st) {
+                        int* status, cudaStream_t st, bool lists) {
   if (ws_bytes < band_tc_bwd_ws_bytes(p, 1, H)) return cudaErrorInvalidValue;
   const int n = p->n_pad(), P = p->P;
   size_t o = 0;
@@ -1187,7 +1884,7 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
   if (e == cudaSuccess) e = band_tc_prep_w(p, H, W, 1, Wk, nullptr, nullptr, status, st);
   if (e == cudaSuccess) {
     ProfSpan span(BG_KID_BAND_BWD, st);
-    e = band_tc_bwd_core(p, H, dYb, Wk, dE, accum, dM, split, status, st);
+    e = band_tc_bwd_core(p, H, dYb, Wk, dE, accum, dM, split, status, st, lists);
   }
   if (e != cudaSuccess) return e;
   // E^T; the weight-gradient product appends its ones row, which turns the bias gradient into
@@ -1200,23 +1897,54 @@ cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, c
                  status, st);
 }
 
+namespace {
+template <typename T>
+bool upload_to(const std::vector<T>& v, T** d, cudaStream_t st) {
+  const size_t bytes = v.size() * sizeof(T);
+  return cudaMalloc(d, std::max<size_t>(bytes, 16)) == cudaSuccess &&
+         (bytes == 0 || cudaMemcpyAsync(*d, v.data(), bytes, cudaMemcpyHostToDevice, st) == cudaSuccess);
+}
+}  // namespace
+
 int band_tc_upload(bg_plan* p, cudaStream_t st) {
   const int S = p->S;
   if (p->P > 32 || (S != 32 && S != 64 && S != 128 && S != 256 && S != 512)) return 0;
   const size_t n = (size_t)p->K * S;
   if (n % kTile) return 0;
-  std::vector<uint32_t> mi, mti;
   std::vector<uint16_t> deg;
-  const int max_deg = band_tc_host_tiles(p, band_chunks(S), mi, mti, deg);
-  p->max_deg = max_deg;
-  if (cudaMalloc(&p->d_maskI, mi.size() * 4) != cudaSuccess ||
-      cudaMalloc(&p->d_maskTI, mti.size() * 4) != cudaSuccess ||
-      cudaMalloc(&p->d_deg2, deg.size() * 2) != cudaSuccess)
-    return -1;
-  if (cudaMemcpyAsync(p->d_maskI, mi.data(), mi.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(p->d_maskTI, mti.data(), mti.size() * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-      cudaMemcpyAsync(p->d_deg2, deg.data(), deg.size() * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return -1;
+  p->max_deg = band_tc_host_degrees(p, deg);
+  if (!upload_to(deg, &p->d_deg2, st)) return -1;
+  const size_t words = n / kTile * p->P * band_chunks(S) * kTile * 4;
+  for (int d = 0; d < 2; ++d) {
+    std::unique_ptr<uint32_t[]> m(new uint32_t[words]);
+    band_tc_host_chunks(p, band_chunks(S), d, m.get());
+    uint32_t** dst = d ? &p->d_maskTI : &p->d_maskI;
+    if (cudaMalloc(dst, std::max<size_t>(words * 4, 16)) != cudaSuccess ||
+        cudaMemcpyAsync(*dst, m.get(), words * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      return -1;
+  }
+  GatherLists lists[2];
+  for (int d = 0; d < 2; ++d) {
+    // each orientation: lists for the state sizes that are faster on them and fit
+    if (gather_max_steps(S, 64, d) == 0) break;
+    const double per = (double)band_tc_list_steps(p, d) / ((double)(n / kTile) * p->P);
+    uint32_t want = 0;
+    for (int H : {32, 64, 128, 256})
+      if (per <= gather_max_steps(S, H, d)) want |= 1u << (H / 32);
+    if (!want) continue;
+    GatherLists& l = lists[d];
+    band_tc_host_lists(p, d, l);
+    for (int H : {32, 64, 128, 256})
+      if ((l.blocks >> 31) ||
+          !(d ? gather_fits<true>(l.lo, l.rows, H) : gather_fits<false>(l.lo, l.rows, H)))
+        want &= ~(1u << (H / 32));
+    if (!want) continue;
+    p->g_lo[d] = l.lo;
+    p->g_rows[d] = l.rows;
+    if (!upload_to(l.words, &p->d_glist[d], st) || !upload_to(l.off, &p->d_goff[d], st)) return -1;
+    p->list_h[d] = want;
+  }
   if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
   return 0;
 }
@@ -1240,6 +1968,10 @@ cudaError_t band_tc_preload_fwd(const bg_plan* p) {
   }
 #undef BG_PRELOAD_S
 #undef BG_PRELOAD
+  take(cudaFuncGetAttributes(&a, k_band_gather<32, false>));
+  take(cudaFuncGetAttributes(&a, k_band_gather<64, false>));
+  take(cudaFuncGetAttributes(&a, k_band_gather<128, false>));
+  take(cudaFuncGetAttributes(&a, k_band_gather<256, false>));
   return e;
 }
 
@@ -1247,6 +1979,12 @@ void band_tc_release(bg_plan* p) {
   cudaFree(p->d_maskI);
   cudaFree(p->d_maskTI);
   cudaFree(p->d_deg2);
+  for (int d = 0; d < 2; ++d) {
+    cudaFree(p->d_glist[d]);
+    cudaFree(p->d_goff[d]);
+    p->d_glist[d] = p->d_goff[d] = nullptr;
+  }
+  p->list_h[0] = p->list_h[1] = 0;
   p->d_maskI = p->d_maskTI = nullptr;
   p->d_deg2 = nullptr;
 }

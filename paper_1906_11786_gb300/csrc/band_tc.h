@@ -12,13 +12,15 @@ namespace bg {
 bool band_tc_supported(const bg_plan* p, int dtype, int H);
 size_t band_tc_fwd_ws_bytes(const bg_plan* p, int dtype, int H);
 size_t band_tc_bwd_ws_bytes(const bg_plan* p, int dtype, int H);
-// Y = sum_p A_p (E W_p + b_p), bf16 operands, fp32 accumulation and output.
+// Y = sum_p A_p (E W_p + b_p), bf16 operands, fp32 accumulation and output.  `lists` allows the
+// gathered kernel where the plan has edge lists (single propagations; GGNN steps pass false).
 cudaError_t band_tc_fwd(const bg_plan* p, int H, const void* E, const void* W, const float* b,
-                        float* Y, char* ws, size_t ws_bytes, int* status, cudaStream_t st);
+                        float* Y, char* ws, size_t ws_bytes, int* status, cudaStream_t st,
+                        bool lists);
 // dE (+)= sum_p (A_p^T dY) W_p^T, dW_p (+)= E^T A_p^T dY, db_p (+)= colsum(A_p^T dY).
 cudaError_t band_tc_bwd(const bg_plan* p, int H, const void* E, const void* W, const float* dY,
                         float* dE, float* dW, float* db, int accum, char* ws, size_t ws_bytes,
-                        int* status, cudaStream_t st);
+                        int* status, cudaStream_t st, bool lists);
 // The band kernel's second-product weights (band_tc_w_bytes): from W [P][H][H] bf16, the forward
 // operand W_p^T (bwd = 0) or the backward operand W_p (bwd = 1), fp32 (kind::tf32 product).
 size_t band_tc_w_bytes(const bg_plan* p, int H);
@@ -41,13 +43,13 @@ size_t band_tc_split_floats(const bg_plan* p, int H);
 cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, const void* Wk,
                              const __nv_bfloat16* b2T, const float* b32, float* out,
                              __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
-                             float* split, const float* addend, int* status,
-                             cudaStream_t st);
+                             float* split, const float* addend, int* status, cudaStream_t st,
+                             bool lists = false);
 //   dY: [n_pad][H] bf16; Wk: band_tc_prep_w(bwd = 1); dE fp32 (+)=; dM: [n_pad][P*H] bf16, 16-byte
 //   aligned.
 cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, const void* Wk,
                              float* dE, int accumulate, __nv_bfloat16* dM, float* split,
-                             int* status, cudaStream_t st);
+                             int* status, cudaStream_t st, bool lists = false);
 // out[c * ld_out + r] = bf16(in[r][c]) for `batch` consecutive R x Cc matrices (in fp32 or bf16;
 // ld_out <= 0 means R; batches are R*Cc apart on both sides).
 cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* out, int R, int Cc,
@@ -59,6 +61,27 @@ int band_tc_upload(bg_plan* p, cudaStream_t st);
 // orientations, and the per-row in-degrees [n_pad][64] as bf16; returns the largest in-degree.
 int band_tc_host_tiles(const bg_plan* p, int C1, std::vector<uint32_t>& mi,
                        std::vector<uint32_t>& mti, std::vector<uint16_t>& deg);
+int band_tc_host_degrees(const bg_plan* p, std::vector<uint16_t>& deg);
+void band_tc_host_chunks(const bg_plan* p, int C1, bool transposed, uint32_t* out);
+// Edge lists of the gathered band kernel, one orientation.  Per 128-row tile, 16-row group and edge
+// type: steps of 16 edges (at least one) in blocks of kGatherBlock, each step 32 words, one per lane of
+// the warp that multiplies it (band_tc.cu): bits 0-17 the byte offset, within the tile's window of
+// 128-byte state rows, of the 16 bytes this lane names to ldmatrix (edge lane % 16, column chunk
+// lane / 16, 128-byte swizzle applied); bit 18 set in the type's last block; bits 19-20 the block's
+// steps less one; bits 24-31 this lane's entries of the 16 x 16 0/1 matrix (row of the group, edge)
+// in mma fragment order.  The window holds rows row0 - lo .. row0 - lo + rows of the state and 8 zero
+// rows after them, which padding entries name.
+constexpr uint32_t kGatherLast = 1u << 18, kGatherMore = 1u << 19;
+constexpr int kGatherBlock = 4;
+struct GatherLists {
+  std::vector<uint32_t> words;  // [blocks][32][kGatherBlock]
+  std::vector<uint32_t> off;    // [n_tiles][8][P + 1] first block, even types first, then odd
+  int lo = 0, rows = 0;
+  int64_t steps = 0, blocks = 0;
+};
+// Steps the lists of one orientation would have.
+int64_t band_tc_list_steps(const bg_plan* p, bool transposed);
+void band_tc_host_lists(const bg_plan* p, bool transposed, GatherLists& out);
 // Loads (CUDA lazy loading) every kernel band_tc_fwd can launch for this plan's block size, at
 // any H, on the current device.
 cudaError_t band_tc_preload_fwd(const bg_plan* p);

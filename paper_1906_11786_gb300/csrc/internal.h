@@ -63,6 +63,12 @@ struct bg_plan {
   uint32_t* d_maskTI = nullptr;
   uint16_t* d_deg2 = nullptr;
   int32_t max_deg = 0;
+  // gathered band kernel: edge lists of both orientations (band_tc.h, GatherLists), and the state
+  // sizes (bit H / 32) that run on them instead of the chunks above
+  uint32_t list_h[2] = {0, 0};
+  uint32_t* d_glist[2] = {nullptr, nullptr};
+  uint32_t* d_goff[2] = {nullptr, nullptr};
+  int32_t g_lo[2] = {0, 0}, g_rows[2] = {0, 0};
   int32_t n_pad() const { return K * S; }
 };
 

@@ -68,7 +68,7 @@ int bg_noalloc_prepare(const bg_plan* p) {
   int rc = resolve_scratch(dev, &s);
   if (rc != BG_OK) return rc;
   e = bg::preload_fwd_simt();
-  if (e == cudaSuccess && p->d_maskI) e = bg::band_tc_preload_fwd(p);
+  if (e == cudaSuccess && p->d_deg2) e = bg::band_tc_preload_fwd(p);
   if (e == cudaSuccess) e = bg::super_preload_fwd();
   if (e != cudaSuccess) return bg_fail(BG_ECUDA, std::string("kernel load: ") + cudaGetErrorString(e));
   return BG_OK;
@@ -108,7 +108,7 @@ extern "C" int bg_band_propagate_fwd_noalloc(const bg_plan* p, bg_dtype dt, int3
   cudaError_t e;
   if (bg::band_tc_supported(p, (int)dt, H)) {
     // every byte of scratch the tensor-core path reads is written first in the same call
-    e = bg::band_tc_fwd(p, H, E, W, b, Y, scratch, kNoAllocScratchBytes, status, st);
+    e = bg::band_tc_fwd(p, H, E, W, b, Y, scratch, kNoAllocScratchBytes, status, st, true);
   } else {
     // SIMT path: messages M_p = E W_p + b_p into the scratch, then the band sum over the tiles
     const size_t n = (size_t)p->n_pad();

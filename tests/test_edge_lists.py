@@ -1,0 +1,131 @@
+"""The edge lists of the gathered band kernel (wide bands, S >= 256): on the CPU, the lists of random
+plans decoded back to exactly the bit tiles' edges; on the GPU, propagation on plans that use them
+against the oracle, at the edges of their ranges."""
+import os
+import struct
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1906_11786_gb300 import build as B
+from paper_1906_11786_gb300 import synth
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+LAST, MORE = 1 << 18, 1 << 19
+
+
+@pytest.fixture(scope="session")
+def probe(tmp_path_factory):
+    B.build()
+    exe = str(tmp_path_factory.mktemp("lists") / "lists_probe")
+    pkg = os.path.join(ROOT, "paper_1906_11786_gb300")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", os.path.join(pkg, "csrc"), "-I",
+                    os.path.join(ROOT, "include"), "-I", "/usr/local/cuda/include",
+                    os.path.join(ROOT, "tests", "lists_probe.cpp"), "-o", exe, "-L", pkg,
+                    "-l:libbandggnn.so", f"-Wl,-rpath,{pkg}"], check=True)
+    return exe
+
+
+def _run(probe, tmp_path, graphs, P, S, transposed):
+    src, dst = str(tmp_path / "in.bin"), str(tmp_path / "out.bin")
+    with open(src, "wb") as f:
+        f.write(struct.pack("=i", len(graphs)))
+        for g in graphs:
+            f.write(struct.pack("=iq", g.n_nodes, g.n_edges))
+            for x in (g.src, g.dst, g.etype):
+                f.write(np.ascontiguousarray(x, np.int32).tobytes())
+    subprocess.run([probe, src, dst, str(P), str(S), str(transposed)], check=True)
+    raw = open(dst, "rb").read()
+    K, lo, rows = struct.unpack_from("=3i", raw, 0)
+    steps, blocks, ahead, nm, nw, no = struct.unpack_from("=6q", raw, 12)
+    a = np.frombuffer(raw, np.uint32, nm + nw + no, 60)
+    return K, lo, rows, steps, blocks, ahead, a[:nm], a[nm:nm + nw], a[nm + nw:]
+
+
+def _tile_edges(masks, K, P, S):
+    bits = np.unpackbits(masks.view(np.uint8), bitorder="little").reshape(K, 3, P, S, S)
+    k, d, p, r, c = np.nonzero(bits)
+    kc = k + d - 1
+    ok = (kc >= 0) & (kc < K)
+    return set(zip((k * S + r)[ok].tolist(), (kc * S + c)[ok].tolist(), p[ok].tolist()))
+
+
+@pytest.mark.parametrize("S,P,F,lam,sizes", [(256, 20, 10, 3.0, [700, 301]), (512, 1, 1, 0.0, [1025]),
+                                             (512, 3, 3, 9.0, [600]), (128, 7, 7, 0.2, [129, 1]),
+                                             (32, 4, 4, 5.0, [95])])
+@pytest.mark.parametrize("transposed", [0, 1])
+def test_lists_hold_exactly_the_tiles_edges(probe, tmp_path, S, P, F, lam, sizes, transposed):
+    graphs = [synth.gen_graph(n, F, P == 2 * F, S // 3, S // 3, lam, 31 * i + S) for i, n in
+              enumerate(sizes)]
+    graphs.append(synth.hub_graph(90, max(P, 2), 5, 0.0) if P > 1 else graphs[0])
+    K, lo, rows, steps, blocks, ahead, masks, words, off = _run(probe, tmp_path, graphs, P, S, transposed)
+    n_tiles = (K * S + 127) // 128
+    w = words.reshape(blocks, 32, 4)
+    off = off.reshape(n_tiles, 8, P + 1)
+    order = list(range(0, P, 2)) + list(range(1, P, 2))
+    lane = np.arange(32)
+    got, at, count = set(), 0, 0
+    assert rows % 8 == 0 and lo % 8 == 0
+    for t in range(n_tiles):
+        for b in range(8):
+            for i, ty in enumerate(order):
+                assert off[t, b, i] == at
+                last = False
+                while not last:
+                    head = int(w[at, 0, 0])
+                    last, m = bool(head & LAST), ((head >> 19) & 3) + 1
+                    for s in range(m):
+                        x = w[at, :, s].astype(np.int64)
+                        assert ((x & (7 << 18)) == (head & (7 << 18))).all()
+                        row = (x & 0x3FFFF) >> 7
+                        assert (row < rows + 8).all() and (row[:16] == row[16:]).all()
+                        assert (((x >> 4) & 7) == ((lane >> 4) ^ (row & 7))).all()
+                        for l in range(32):
+                            for j in range(8):
+                                if x[l] >> (24 + j) & 1:
+                                    r = l // 4 + 8 * (j & 1)
+                                    k = 2 * (l % 4) + (j >> 2) + 8 * (j >> 1 & 1)
+                                    assert row[k] < rows  # a padding entry names a zero row
+                                    e = (128 * t + 16 * b + r, int(row[k]) + 128 * t - lo, ty)
+                                    assert e not in got
+                                    got.add(e)
+                        count += 1
+                    at += 1
+            assert off[t, b, P] == at
+    assert at == blocks and count == steps == ahead
+    assert got == _tile_edges(masks, K, P, S)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("S,H,P,F,lam,sizes", [
+    (256, 64, 20, 10, 3.0, [1500, 900]), (256, 128, 20, 10, 3.0, [2000]), (256, 32, 5, 5, 1.0, [257]),
+    (512, 64, 20, 10, 3.0, [1800, 700]), (512, 128, 4, 4, 2.0, [1300]), (512, 32, 1, 1, 0.0, [40]),
+    (256, 64, 3, 3, 40.0, [1100]),    # 120 edges per 16 rows and type: several blocks each
+    (256, 64, 3, 3, 70.0, [1100])])   # and beyond the lists' range: the dense kernel
+def test_propagation_on_lists_matches_the_oracle(S, H, P, F, lam, sizes):
+    import oracle
+    import torch
+    from gpu_common import Case, L, TOL, assert_close, ensure_built, f32_dev
+    ensure_built()
+    graphs = [synth.gen_graph(n, F, P == 2 * F, 3 * S // 8, 3 * S // 8, lam, 100 + i)
+              for i, n in enumerate(sizes)]
+    c = Case(graphs, P, S, H, "bf16", seed=S + H)
+    Y = torch.empty((c.N, H), device="cuda")
+    L.band_propagate_fwd(c.plan, "bf16", H, c.E_band_dev, c.dprm["W"], c.dprm["b"], Y,
+                         c.ws(L.BG_OP_PROPAGATE_FWD))
+    dY = np.zeros((c.N, H))
+    dY[: c.n_real] = np.random.default_rng(7).standard_normal((c.n_real, H)).astype(np.float32)
+    dE, dW = torch.empty((c.N, H), device="cuda"), torch.empty((P, H, H), device="cuda")
+    db = torch.empty((P, H), device="cuda")
+    L.band_propagate_bwd(c.plan, "bf16", H, c.E_band_dev, c.dprm["W"], f32_dev(dY), dE, dW, db,
+                         c.ws(L.BG_OP_PROPAGATE_BWD))
+    torch.cuda.synchronize()
+    L.check_device()
+    args = (c.N, P, H, *c.edges, c.E_band, c.prm["W"])
+    # the repository's bf16 tolerance; rounding pre_p to tf32 alone gives about 2e-4
+    assert_close(Y.cpu().numpy(), oracle.propagate_fwd(*args, c.prm["b"]), TOL["bf16"], "Y")
+    rE, rW, rb = oracle.propagate_bwd(*args, dY)
+    for got, ref, what in ((dE, rE, "dE"), (dW, rW, "dW"), (db, rb, "db")):
+        assert_close(got.cpu().numpy(), ref, TOL["bf16"], what)
+    assert float(Y[c.n_real:].abs().max() if c.N > c.n_real else 0.0) == 0.0
