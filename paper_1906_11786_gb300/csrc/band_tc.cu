@@ -759,8 +759,8 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 // Bound: latency along each warp's chain (words, ldmatrix, products, TMEM store), with the shared-memory
 // and tensor pipes each about half busy at 16 warps of 80 registers.  A step (4 ldmatrix.x4, 8 mma.sync)
 // takes 26 cycles of the SM with conflict-free rows, 44 with random ones, which is why the plan deals
-// edges into sets of 8 whose rows differ mod 8.  S = 512, H = 64, 131k nodes, 52 edges per node: 97 us
-// against the dense kernel's 440; S = 256, H = 128, 20k nodes backward: 60 us against 86.
+// edges into sets of 8 whose rows differ mod 8.  S = 512, H = 64, 131k nodes, 52 edges per node: 112 us
+// against the dense kernel's 457; S = 256, H = 128, 20k nodes backward: 61 us against 89 (ncu).
 //
 // Roles (24 warps, one CTA per SM, persistent over the same items as k_band_tc):
 //   warp 0       TMA producer: state windows, W tiles, deg, bias
@@ -818,9 +818,8 @@ GaLayout ga_layout(int lo, int rows) {
   g.rows = rows;
   g.box_rows = rows / ((rows + 255) / 256);  // the plan made them equal
   const int win = (rows + 8) * 128;
-  // A W stage takes about 1.5 us from release to refill (L2), so the ring's depth over that time caps
-  // the jobs (at two 16 KB stages 70 us a launch at packed64); a second window hides one window load
-  // per tile.
+  // Two windows (the second hides one load per pass) with four or three W stages (their refills come
+  // from L2); where that does not fit, the stages before the second window.
   constexpr int kTry[8][2] = {{2, 4}, {2, 3}, {1, 4}, {1, 3}, {2, 2}, {1, 2}, {2, 1}, {1, 1}};
   for (auto& t : kTry)
     if (t[0] * win + t[1] * C::WSTAGE + C::FIXED <= 232448) {

@@ -33,51 +33,78 @@ inline int grid_for(int64_t n, int threads) {
 }
 
 // ------------------------------------------------------------------------------------ GEMM
-constexpr int GT = 64;   // output tile edge
 constexpr int GK = 16;   // k step
 
-// 64 x 64 tile, 4 x 4 outputs per thread.  The next K step's operands are on their way in registers
-// while the current one is multiplied from shared memory (two buffers, one barrier a step): with the
-// loads in front of each step the loop was latency-bound (four 512 x 64 x 64 products 15.4 us
-// against 8.2; six products of 3,008 rows at H = 96 198 us against 134, ncu).
-template <typename TA, typename TB>
+// 16 TM x 16 TN tile, TM x TN outputs per thread.  The next K step's operands are on their way in
+// registers while the current one is multiplied from shared memory (two buffers, one barrier a step):
+// with the loads in front of each step the loop was latency-bound (four 512 x 64 x 64 products 15.4 us
+// against 8.2, ncu).  Eight rows a thread do 32 or 48 FMAs per 3 or 3.5 16-byte shared loads instead of
+// 16 per 2; six columns fit a width of 96 without an idle quarter (a two-step fp32 batch of 3,001 nodes
+// at H = 96, mostly these products: 157 us a pass with 4 x 4, 137 so).
+template <int N>
+__device__ __forceinline__ void lds_vec(float (&v)[N], const float* p) {
+  if constexpr (N % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + i);
+      v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+      const float2 x = *reinterpret_cast<const float2*>(p + i);
+      v[i] = x.x; v[i + 1] = x.y;
+    }
+  }
+}
+
+template <int TM, int TN, typename TA, typename TB>
 __global__ void __launch_bounds__(256) k_gemm(Gemm g, int splits, int kchunk, float* part) {
-  __shared__ __align__(16) float As[2][GK][GT + 4];
-  __shared__ __align__(16) float Bs[2][GK][GT + 4];
+  constexpr int BM = 16 * TM, BN = 16 * TN;
+  __shared__ __align__(16) float As[2][GK][BM + 4];
+  __shared__ __align__(16) float Bs[2][GK][BN + 4];
   grid_dep_wait();
   const TA* A = static_cast<const TA*>(g.A);
   const TB* B = static_cast<const TB*>(g.B);
   const int b = blockIdx.z / splits, s = blockIdx.z % splits;
-  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int kbeg = s * kchunk;
   const int kend = min(g.K, kbeg + kchunk);
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   const bool a_k_fast = (g.sAk == 1);
   const bool b_n_fast = (g.sBn == 1);
-  float acc[4][4];
+  float acc[TM][TN];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < TM; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  float ra[4], rb[4];
+    for (int c = 0; c < TN; ++c) acc[r][c] = 0.f;
+  float ra[TM], rb[TN];
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < TM; ++q) {
       const int idx = tid + 256 * q;
-      const int am = a_k_fast ? idx / GK : idx % GT, ak = a_k_fast ? idx % GK : idx / GT;
+      const int am = a_k_fast ? idx / GK : idx % BM, ak = a_k_fast ? idx % GK : idx / BM;
       const int m = m0 + am, k = k0 + ak;
       ra[q] = (m < g.M && k < kend) ? ld(A, b * g.sAb + m * g.sAm + k * g.sAk) : 0.f;
-      const int bn = b_n_fast ? idx % GT : idx / GK, bk = b_n_fast ? idx / GT : idx % GK;
-      const int n = n0 + bn, kb = k0 + bk;
-      rb[q] = (n < g.N && kb < kend) ? ld(B, b * g.sBb + kb * g.sBk + n * g.sBn) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < TN; ++q) {
+      const int idx = tid + 256 * q;
+      const int bn = b_n_fast ? idx % BN : idx / GK, bk = b_n_fast ? idx / BN : idx % GK;
+      const int n = n0 + bn, k = k0 + bk;
+      rb[q] = (n < g.N && k < kend) ? ld(B, b * g.sBb + k * g.sBk + n * g.sBn) : 0.f;
     }
   };
   auto stage = [&](int buf) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < TM; ++q) {
       const int idx = tid + 256 * q;
-      As[buf][a_k_fast ? idx % GK : idx / GT][a_k_fast ? idx / GK : idx % GT] = ra[q];
-      Bs[buf][b_n_fast ? idx / GT : idx % GK][b_n_fast ? idx % GT : idx / GK] = rb[q];
+      As[buf][a_k_fast ? idx % GK : idx / BM][a_k_fast ? idx / GK : idx % BM] = ra[q];
+    }
+#pragma unroll
+    for (int q = 0; q < TN; ++q) {
+      const int idx = tid + 256 * q;
+      Bs[buf][b_n_fast ? idx / BN : idx % GK][b_n_fast ? idx % BN : idx / GK] = rb[q];
     }
   };
   if (kbeg < kend) {
@@ -90,24 +117,24 @@ __global__ void __launch_bounds__(256) k_gemm(Gemm g, int splits, int kchunk, fl
     if (more) fetch(k0 + GK);
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[buf][kk][ty * 4]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * 4]);
-      const float a[4] = {av.x, av.y, av.z, av.w}, bb[4] = {bv.x, bv.y, bv.z, bv.w};
+      float a[TM], bb[TN];
+      lds_vec(a, &As[buf][kk][ty * TM]);
+      lds_vec(bb, &Bs[buf][kk][tx * TN]);
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < TM; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] += a[r] * bb[c];
+        for (int c = 0; c < TN; ++c) acc[r][c] += a[r] * bb[c];
     }
     if (more) stage(buf ^ 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    int m = m0 + ty * 4 + r;
+  for (int r = 0; r < TM; ++r) {
+    int m = m0 + ty * TM + r;
     if (m >= g.M) continue;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      int n = n0 + tx * 4 + c;
+    for (int c = 0; c < TN; ++c) {
+      int n = n0 + tx * TN + c;
       if (n >= g.N) continue;
       if (splits == 1) {
         int64_t o = b * g.sCb + (int64_t)m * g.ldc + n;
@@ -553,13 +580,31 @@ __global__ void k_add(float* d, const float* s, int64_t n) {
 
 // ====================================================================================== hosts
 
+namespace {
+using GemmFn = void (*)(Gemm, int, int, float*);
+template <int TM, int TN>
+GemmFn gemm_types(const Gemm& g) {
+  if (g.a_bf16) return g.b_bf16 ? k_gemm<TM, TN, __nv_bfloat16, __nv_bfloat16> : k_gemm<TM, TN, __nv_bfloat16, float>;
+  return g.b_bf16 ? k_gemm<TM, TN, float, __nv_bfloat16> : k_gemm<TM, TN, float, float>;
+}
+GemmFn gemm_fn(const Gemm& g, int TM, int TN) {
+  return TM == 8 ? (TN == 6 ? gemm_types<8, 6>(g) : gemm_types<8, 4>(g))
+                 : (TN == 6 ? gemm_types<4, 6>(g) : gemm_types<4, 4>(g));
+}
+}  // namespace
+
 cudaError_t gemm(const Gemm& g, float* part, size_t part_floats, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
-  int tiles = ((g.N + GT - 1) / GT) * ((g.M + GT - 1) / GT) * g.batch;
+  // six columns a thread where the width is a multiple of 96 and not of 64; eight rows where tiles of
+  // 128 rows still give every SM one
+  const int TN = (g.N % 96 == 0 && g.N % 64 != 0) ? 6 : 4, BN = 16 * TN;
+  const int nt = (g.N + BN - 1) / BN;
+  const int TM = (int64_t)nt * ((g.M + 127) / 128) * g.batch >= 152 ? 8 : 4, BM = 16 * TM;
+  const int tiles = nt * ((g.M + BM - 1) / BM) * g.batch;
   // Few tiles: K split over more blocks, at least 64 of it each (four steps of the loop).  The second
   // launch costs about 3.5 us, so K below 256 is not split.  The two products of the 512-node fp32
-  // backward (512 x 64 x 256, and 64 x 64 x 512 for four types) take 15.4 us and 7.2 for their
-  // reductions; with the split from K > 512 on and the old loop 161.7 us (ncu).
+  // backward (512 x 64 x 256, and 64 x 64 x 512 for four types) take 15.3 us and 7.2 for their
+  // reductions; with the split from K > 512 on and the old loop 165 us (ncu).
   int splits = 1;
   if (g.K >= 256 && tiles < 304 && part) {
     splits = (304 + tiles - 1) / tiles;
@@ -572,16 +617,8 @@ cudaError_t gemm(const Gemm& g, float* part, size_t part_floats, cudaStream_t st
   kchunk = ((kchunk + GK - 1) / GK) * GK;
   splits = (g.K + kchunk - 1) / kchunk;
   if (splits < 1) splits = 1;
-  dim3 grid((g.N + GT - 1) / GT, (g.M + GT - 1) / GT, g.batch * splits);
-  cudaError_t e;
-  if (g.a_bf16 && g.b_bf16)
-    e = launch_pdl(k_gemm<__nv_bfloat16, __nv_bfloat16>, grid, dim3(256), 0, st, g, splits, kchunk, part);
-  else if (g.a_bf16)
-    e = launch_pdl(k_gemm<__nv_bfloat16, float>, grid, dim3(256), 0, st, g, splits, kchunk, part);
-  else if (g.b_bf16)
-    e = launch_pdl(k_gemm<float, __nv_bfloat16>, grid, dim3(256), 0, st, g, splits, kchunk, part);
-  else
-    e = launch_pdl(k_gemm<float, float>, grid, dim3(256), 0, st, g, splits, kchunk, part);
+  dim3 grid(nt, (g.M + BM - 1) / BM, g.batch * splits);
+  cudaError_t e = launch_pdl(gemm_fn(g, TM, TN), grid, dim3(256), 0, st, g, splits, kchunk, part);
   note_launch();
   if (e == cudaSuccess && splits > 1) {
     int64_t total = (int64_t)g.batch * g.M * g.N;
@@ -669,10 +706,12 @@ cudaError_t preload_fwd_simt() {
   cudaFuncAttributes a;
   cudaError_t e = cudaSuccess;
   auto take = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-  take(cudaFuncGetAttributes(&a, k_gemm<__nv_bfloat16, __nv_bfloat16>));
-  take(cudaFuncGetAttributes(&a, k_gemm<__nv_bfloat16, float>));
-  take(cudaFuncGetAttributes(&a, k_gemm<float, __nv_bfloat16>));
-  take(cudaFuncGetAttributes(&a, k_gemm<float, float>));
+  for (int v = 0; v < 16; ++v) {
+    Gemm g;
+    g.a_bf16 = v & 1;
+    g.b_bf16 = v >> 1 & 1;
+    take(cudaFuncGetAttributes(&a, reinterpret_cast<const void*>(gemm_fn(g, v & 4 ? 8 : 4, v & 8 ? 6 : 4))));
+  }
   take(cudaFuncGetAttributes(&a, k_gemm_reduce));
   for (int H = 32; H <= 256; H += 32)
     take(with_hq(H, [&](auto hq) {
