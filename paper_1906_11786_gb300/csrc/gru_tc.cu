@@ -153,6 +153,21 @@ __device__ __forceinline__ void store_T4(__nv_bfloat16* dst, int64_t ld, int row
   store_T_pairs<4>(dst, ld, row, h0, pk);
 }
 
+// 16 bf16 (8 packed pairs) of each lane's row, rows consecutive over the warp (row parity = lane
+// parity); dst: the lane pair's first row, ld its stride.  The pair swaps halves with four shuffles, so
+// that each 16-byte store instruction fills whole 32-byte sectors (a lane's own two halves in two
+// instructions leave every sector written half at a time).  Every lane of the warp calls it.
+__device__ __forceinline__ void store_rows16(__nv_bfloat16* dst, int64_t ld, const uint32_t* px) {
+  const bool odd = threadIdx.x & 1;
+  uint32_t o[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) o[j] = __shfl_xor_sync(0xffffffffu, odd ? px[j] : px[4 + j], 1);
+  const uint4 first = odd ? make_uint4(o[0], o[1], o[2], o[3]) : make_uint4(px[0], px[1], px[2], px[3]);
+  const uint4 second = odd ? make_uint4(px[4], px[5], px[6], px[7]) : make_uint4(o[0], o[1], o[2], o[3]);
+  *reinterpret_cast<uint4*>(dst + 8 * odd) = first;         // the even lane's row
+  *reinterpret_cast<uint4*>(dst + ld + 8 * odd) = second;   // the odd lane's row
+}
+
 template <int KH>
 struct GruSmem {
   static constexpr int TILE = 128 * 128;  // 128 rows x 64 bf16 (columns >= KH zero)
@@ -554,9 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t px[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) px[j] = pk2(__uint_as_float(vx[2 * j]), __uint_as_float(vx[2 * j + 1]));
-      uint4* dx = reinterpret_cast<uint4*>(dX + (size_t)row * KH + h0);
-      dx[0] = make_uint4(px[0], px[1], px[2], px[3]);
-      dx[1] = make_uint4(px[4], px[5], px[6], px[7]);
+      store_rows16(dX + (size_t)(row & ~1) * KH + h0, KH, px);
       float4* go = reinterpret_cast<float4*>(gout + (size_t)row * KH + h0);
 #pragma unroll
       for (int q = 0; q < 4; ++q)
@@ -1260,9 +1273,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t px[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) px[j] = pk2(__uint_as_float(vx[2 * j]), __uint_as_float(vx[2 * j + 1]));
-        uint4* dx = reinterpret_cast<uint4*>(dX + (size_t)row * H + h0);
-        dx[0] = make_uint4(px[0], px[1], px[2], px[3]);
-        dx[1] = make_uint4(px[4], px[5], px[6], px[7]);
+        store_rows16(dX + (size_t)(row & ~1) * H + h0, H, px);
         // this thread stored the direct term of these columns above
         float4* go = reinterpret_cast<float4*>(gout + (size_t)row * H + h0);
 #pragma unroll
