@@ -549,11 +549,27 @@ def run_op(args, st, c):
     torch.cuda.synchronize()
     L.check_device()
     ms = e0.elapsed_time(e1) / args.steps
-    f = st.plan.flops(H, L.BG_FLOPS_BAND) + st.plan.flops(H, L.BG_FLOPS_XFORM)
+    f, counted, kernel = _band_flops(L, st.plan, st.dt, H, args.op, False)
     print(json.dumps({"op": args.op, "ms_per_call": ms, "tflops": f / (ms / 1e3) / 1e12,
+                      "flops_counted": counted, "kernel": kernel,
                       "band_kernels": "tcgen05" if L.band_uses_tensor_cores(st.plan, st.dt, H)
                       else "simt"}))
     return 0
+
+
+def _band_flops(L, plan, dtype, H, op, in_step):
+    """Operations one launch of the band kernel executes (op band_fwd or band_bwd; in_step: inside a
+    GGNN step), what they count, and the kernel.  A single propagation on a plan with edge lists does
+    one multiply-add per edge and column, every other launch the band-dense count."""
+    if not L.band_uses_tensor_cores(plan, dtype, H):
+        gathered, kernel = False, "simt"
+    else:
+        gathered = not in_step and L.band_uses_lists(
+            plan, dtype, H, L.BG_OP_PROPAGATE_FWD if op == "band_fwd" else L.BG_OP_PROPAGATE_BWD)
+        kernel = "k_band_gather" if gathered else "k_band_tc"
+    flops = (plan.flops(H, L.BG_FLOPS_NNZ if gathered else L.BG_FLOPS_BAND) +
+             plan.flops(H, L.BG_FLOPS_XFORM))
+    return flops, "edges and transforms" if gathered else "band-dense and transforms", kernel
 
 
 KNAMES = ["band_fwd", "band_bwd", "gru_fwd", "gru_bwd", "dW"]
@@ -572,11 +588,7 @@ def roofline(L, st, c, kt, pk, workload_name):
     kern = "band_fwd" if fwd_ms >= bwd_ms else "band_bwd"
     avg_ms = (fwd_ms / max(fwd_n, 1)) if kern == "band_fwd" else (bwd_ms / max(bwd_n, 1))
     tc = L.band_uses_tensor_cores(st.plan, c["dtype"], H)
-    # single bf16 propagations at S >= 256 sum the workloads' sparse bands from edge lists: the
-    # operations executed are one multiply-add per edge and column, not the band-dense count
-    gathered = tc and not c["gru"] and st.plan.info()["S"] >= 256
-    flops = (st.plan.flops(H, L.BG_FLOPS_NNZ if gathered else L.BG_FLOPS_BAND) +
-             st.plan.flops(H, L.BG_FLOPS_XFORM))
+    flops, counted, _ = _band_flops(L, st.plan, c["dtype"], H, kern, c["gru"])
     achieved = flops / (avg_ms / 1e3) / 1e12 if avg_ms > 0 else 0.0
     if tc:
         bound, peak = "tensor", pk["bf16"]
@@ -591,7 +603,7 @@ def roofline(L, st, c, kt, pk, workload_name):
             "traffic_src": "profiles/ ncu capture (dram read+write bytes per launch)"
             if traffic else None, "peak_src": peak_src,
             "kernel_ms": {k: (kt[i][0] / max(kt[i][1], 1)) for i, k in enumerate(KNAMES)},
-            "flops_counted": "edges and transforms" if gathered else "band-dense and transforms",
+            "flops_counted": counted,
             "nnz_tflops": st.plan.flops(H, L.BG_FLOPS_NNZ) / (avg_ms / 1e3) / 1e12
             if avg_ms > 0 else 0.0}
     if tc:

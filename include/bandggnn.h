@@ -341,6 +341,11 @@ int64_t bg_launch_count(void);
  * H not in {32, 64, 128, 256}, H = 256 at S >= 256, P > 32, a padded size that is not a whole
  * number of 128-row tiles); negative status on error.  The plan must be uploaded. */
 int bg_band_uses_tensor_cores(const bg_plan* plan, bg_dtype dtype, int32_t H);
+/* 1 when a single propagation of this kind (op BG_OP_PROPAGATE_FWD or BG_OP_PROPAGATE_BWD) sums
+ * the plan's edges from lists, 0 when it multiplies the band's bit tiles (or runs on the SIMT
+ * kernels); the GGNN steps always multiply the tiles.  Negative status on error.  The plan must be
+ * uploaded. */
+int bg_band_uses_lists(const bg_plan* plan, bg_dtype dtype, int32_t H, int32_t op);
 
 #ifdef __cplusplus
 }

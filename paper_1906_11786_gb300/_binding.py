@@ -110,6 +110,7 @@ def load(path: str = LIB_PATH):
         "bg_profile_read": (c.c_int, [i32, vp, vp, i32]),
         "bg_launch_count": (i64, []),
         "bg_band_uses_tensor_cores": (c.c_int, [vp, c.c_int, i32]),
+        "bg_band_uses_lists": (c.c_int, [vp, c.c_int, i32, i32]),
         "bg_reach_filter": (c.c_int, [vp, vp, i32, i32, vp, vp, vp, vp, vp, vp]),
         "bg_plan_partition": (c.c_int, [vp, i32, i32, vp, vp]),
     }
@@ -389,6 +390,14 @@ def profile_read(kid, reset=False):
 
 def band_uses_tensor_cores(plan, dtype, H) -> bool:
     rc = load().bg_band_uses_tensor_cores(plan.handle, dtype_code(dtype), H)
+    if rc < 0:
+        _check(rc)
+    return rc == 1
+
+
+def band_uses_lists(plan, dtype, H, op) -> bool:
+    """Whether a single propagation (op BG_OP_PROPAGATE_FWD or _BWD) sums the edges from lists."""
+    rc = load().bg_band_uses_lists(plan.handle, dtype_code(dtype), H, op)
     if rc < 0:
         _check(rc)
     return rc == 1

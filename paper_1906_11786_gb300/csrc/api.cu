@@ -657,6 +657,15 @@ extern "C" int bg_band_uses_tensor_cores(const bg_plan* p, bg_dtype dt, int32_t 
   return bg::band_tc_supported(p, (int)dt, H) ? 1 : 0;
 }
 
+extern "C" int bg_band_uses_lists(const bg_plan* p, bg_dtype dt, int32_t H, int32_t op) {
+  bg_clear_error();
+  BG_TRY(check_plan_dev(p));
+  BG_TRY(check_shape(p, dt, H));
+  if (op != BG_OP_PROPAGATE_FWD && op != BG_OP_PROPAGATE_BWD)
+    return bg_fail(BG_EINVAL, "op must be BG_OP_PROPAGATE_FWD or BG_OP_PROPAGATE_BWD");
+  return bg::band_tc_uses_lists(p, (int)dt, H, op == BG_OP_PROPAGATE_BWD) ? 1 : 0;
+}
+
 // ---------------------------------------------------------------------------------- pack
 extern "C" int bg_pack_states(const bg_plan* p, bg_dtype dt, int32_t H, const void* Eo, void* Eb,
                               void* stream) {

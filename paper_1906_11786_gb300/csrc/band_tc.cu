@@ -1736,6 +1736,10 @@ namespace {
 bool use_lists(const bg_plan* p, int H, bool bwd) { return p->list_h[bwd] >> (H / 32) & 1; }
 }  // namespace
 
+bool band_tc_uses_lists(const bg_plan* p, int dtype, int H, bool bwd) {
+  return band_tc_supported(p, dtype, H) && use_lists(p, H, bwd);
+}
+
 size_t band_tc_w_bytes(const bg_plan* p, int H) {
   return al256((size_t)p->P * H * H * 4);
 }

@@ -10,6 +10,8 @@ namespace bg {
 
 // True when the fused tensor-core kernels handle (dtype, H, S, P) for this plan.
 bool band_tc_supported(const bg_plan* p, int dtype, int H);
+// Whether band_tc_fwd (bwd = false) or band_tc_bwd with `lists` runs the gathered kernel.
+bool band_tc_uses_lists(const bg_plan* p, int dtype, int H, bool bwd);
 size_t band_tc_fwd_ws_bytes(const bg_plan* p, int dtype, int H);
 size_t band_tc_bwd_ws_bytes(const bg_plan* p, int dtype, int H);
 // Y = sum_p A_p (E W_p + b_p), bf16 operands, fp32 accumulation and output.  `lists` allows the

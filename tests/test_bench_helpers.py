@@ -90,3 +90,43 @@ def test_l2_statement_follows_the_working_set():
     assert cfg["parallelism"].startswith("dp2") and "all-reduce" in cfg["parallelism"]
     for k in ("workload", "graphs", "packed", "n_real", "n_pad", "K", "S", "P", "H", "T"):
         assert k in cfg
+
+
+class _FakeBinding:
+    """The library calls the roofline makes, on a plan that uses lists in one direction only."""
+    BG_KID_BAND_FWD, BG_KID_BAND_BWD = 0, 1
+    BG_OP_PROPAGATE_FWD, BG_OP_PROPAGATE_BWD = 0, 1
+    BG_FLOPS_BAND, BG_FLOPS_XFORM, BG_FLOPS_NNZ = "band", "xform", "nnz"
+
+    @staticmethod
+    def band_uses_tensor_cores(plan, dtype, H):
+        return True
+
+    @classmethod
+    def band_uses_lists(cls, plan, dtype, H, op):
+        return op == cls.BG_OP_PROPAGATE_FWD
+
+
+class _FakePlan:
+    def flops(self, H, kind):
+        return {"band": 4e12, "xform": 1e12, "nnz": 1e10}[kind]
+
+    def info(self):
+        return {"S": 512}
+
+
+@pytest.mark.parametrize("slow,gru,count,flops", [
+    ("band_fwd", False, "edges and transforms", 1.01e12),
+    ("band_bwd", False, "band-dense and transforms", 5e12),   # a plan beyond the lists' range
+    ("band_fwd", True, "band-dense and transforms", 5e12)])   # GGNN steps multiply the tiles
+def test_roofline_counts_the_operations_of_the_kernel_that_ran(slow, gru, count, flops):
+    import types
+    st = types.SimpleNamespace(plan=_FakePlan())
+    fwd, bwd = (2.0, 1.0) if slow == "band_fwd" else (1.0, 2.0)
+    kt = [(fwd, 1), (bwd, 1), (0, 0), (0, 0), (0, 0)]
+    pk = {"bf16": 1880.7, "bf16_sustained": 1713.8, "src": "measured", "sm_max_mhz": 2070.0}
+    r = bench.roofline(_FakeBinding, st, {"H": 64, "dtype": "bf16", "gru": gru}, kt, pk, "none")
+    assert r["kernel"] == slow and r["flops_counted"] == count
+    assert r["achieved"] == pytest.approx(flops / 2e-3 / 1e12)
+    assert bench._band_flops(_FakeBinding, st.plan, "bf16", 64, slow, gru)[2] == (
+        "k_band_gather" if count.startswith("edges") else "k_band_tc")
