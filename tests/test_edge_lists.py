@@ -129,3 +129,50 @@ def test_propagation_on_lists_matches_the_oracle(S, H, P, F, lam, sizes):
     for got, ref, what in ((dE, rE, "dE"), (dW, rW, "dW"), (db, rb, "db")):
         assert_close(got.cpu().numpy(), ref, TOL["bf16"], what)
     assert float(Y[c.n_real:].abs().max() if c.N > c.n_real else 0.0) == 0.0
+
+
+# (S, H, P, F, lam, sizes, lists forward, lists backward): the first three as their rule says, several
+# blocks of four steps for many (group, type) pairs (51 steps a tile and type at lam = 20); then a plan
+# beyond the rule, one at a narrow band, one at a state size without lists
+ROUTES = [(256, 64, 3, 3, 20.0, [1100], True, True), (512, 128, 3, 3, 45.0, [900, 700], True, True),
+          (512, 32, 20, 10, 3.0, [1800, 700], True, True), (256, 64, 3, 3, 70.0, [1100], False, False),
+          (128, 64, 20, 10, 3.0, [900], False, False), (512, 96, 20, 10, 3.0, [600], False, False)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("S,H,P,F,lam,sizes,fwd,bwd", ROUTES)
+def test_lists_run_where_their_rule_says_and_accumulate(S, H, P, F, lam, sizes, fwd, bwd):
+    import oracle
+    import torch
+    from gpu_common import Case, L, TOL, assert_close, ensure_built, f32_dev
+    ensure_built()
+    graphs = [synth.gen_graph(n, F, P == 2 * F, 3 * S // 8, 3 * S // 8, lam, 300 + i)
+              for i, n in enumerate(sizes)]
+    c = Case(graphs, P, S, H, "bf16", seed=S + H)
+    assert L.band_uses_lists(c.plan, "bf16", H, L.BG_OP_PROPAGATE_FWD) == fwd
+    assert L.band_uses_lists(c.plan, "bf16", H, L.BG_OP_PROPAGATE_BWD) == bwd
+    assert not L.band_uses_lists(c.plan, "f32", H, L.BG_OP_PROPAGATE_FWD)
+    Y = torch.empty((c.N, H), device="cuda")
+    L.band_propagate_fwd(c.plan, "bf16", H, c.E_band_dev, c.dprm["W"], c.dprm["b"], Y,
+                         c.ws(L.BG_OP_PROPAGATE_FWD))
+    dY = np.zeros((c.N, H))
+    dY[: c.n_real] = np.random.default_rng(7).standard_normal((c.n_real, H)).astype(np.float32)
+    got = [torch.empty(s, device="cuda") for s in ((c.N, H), (P, H, H), (P, H))]
+    ws = c.ws(L.BG_OP_PROPAGATE_BWD)
+    L.band_propagate_bwd(c.plan, "bf16", H, c.E_band_dev, c.dprm["W"], f32_dev(dY), *got, ws)
+    # the same gradients added to what the arrays hold
+    start = [torch.from_numpy(np.random.default_rng(i).standard_normal(tuple(x.shape)).astype(np.float32))
+             .cuda() * x.abs().max() for i, x in enumerate(got)]
+    acc = [x.clone() for x in start]
+    L.band_propagate_bwd(c.plan, "bf16", H, c.E_band_dev, c.dprm["W"], f32_dev(dY), *acc, ws,
+                         flags=L.BG_ACCUM)
+    torch.cuda.synchronize()
+    L.check_device()
+    args = (c.N, P, H, *c.edges, c.E_band, c.prm["W"])
+    assert_close(Y.cpu().numpy(), oracle.propagate_fwd(*args, c.prm["b"]), TOL["bf16"], "Y")
+    for x, a, s, ref, what in zip(got, acc, start, oracle.propagate_bwd(*args, dY), ("dE", "dW", "db")):
+        assert_close(x.cpu().numpy(), ref, TOL["bf16"], what)
+        # one fp32 addition per sum beyond the plain call's, of values up to five times its largest, and
+        # the split's partial sums added in another order: a few units of 2^-24
+        d = (a.double() - s.double() - x.double()).abs().max() / x.abs().max()
+        assert float(d) < 1e-5, what
