@@ -69,6 +69,11 @@ constexpr int kTile = 128;     // rows per tile = UMMA M
 //   S <= 64: C1 = 2 (the tile spans 128 / S block-rows);  S = 128: 3;  S = 256: 6;  S = 512: 12.
 __host__ __device__ constexpr int band_chunks(int S) { return S <= 64 ? 2 : 3 * (S / 128); }
 
+// Shapes (block size, state columns per pass) whose forward adds the bias in its epilogue, in-degree
+// times b in fp32, dense and gathered alike; at the others it is a product of in-degrees and the bias
+// split into two 16-bit parts.
+__host__ __device__ constexpr bool bias_in_fp32(int S, int SW) { return S == 512 && SW == 64; }
+
 template <int H, int S, bool BWD = false>
 struct Cfg {
   // H > SW runs as H / SW passes over SW-column slices of the state: pass hh contracts the band
@@ -79,7 +84,7 @@ struct Cfg {
   // size in shared memory: the expanders read their mask words straight from global memory (L2)
   // instead of a staged ring, W has one stage, and the bias is added in the epilogue (in-degree
   // times b in fp32) instead of by a product with staged operands
-  static constexpr bool GM = S == 512 && SW == 64;
+  static constexpr bool GM = bias_in_fp32(S, SW);
   static constexpr int NH = H / SW;
   static constexpr int C1 = band_chunks(S);                   // 128-column chunks per type
   static constexpr int XROW = SW * 2;                         // bytes of one node's slice
@@ -751,8 +756,8 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 // from the row-major window in shared memory), and T holds a 1 where an edge ends in a row.  The
 // accumulator fragment is the register layout of tcgen05.st.16x256b, so pre_p goes to TMEM as the A
 // operand of the second product, which is issued exactly as in k_band_tc.  A sum of a few bf16 values
-// is nearly always exact in fp32, so the results agree with the dense kernel's but for the rare sum
-// that is not (1e-10 to 1e-6 of the norm).  A GGNN step rounds Y to bf16 and feeds it back, where even
+// is nearly always exact in fp32, and the bias is added as the dense kernel adds it, so the results
+// agree with the dense kernel's but for the rare sum that is not exact (1e-10 to 3e-7 of the norm).  A GGNN step rounds Y to bf16 and feeds it back, where even
 // that grows through the layers; its saved activations and gradients do not depend on how dense a
 // plan is, so the GGNN steps stay on the dense kernel.
 //
@@ -1143,6 +1148,31 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
           const float* ad = sc.addend + (size_t)asl * H + h0;
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ad[j]);
+        }
+        if (!BWD && sc.bias && part <= 0) {
+          // the bias in fp32, as the dense kernel adds it at these shapes: the in-degrees of two types
+          // per load (0 beyond the last), each times b_p
+          const uint16_t* dr = sc.deg + (size_t)row * 64;
+#pragma unroll 1
+          for (int q = 0; q < P; q += 2) {
+            const uint32_t two = *reinterpret_cast<const uint32_t*>(dr + q);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const uint32_t bits = (two >> (16 * t)) & 0xFFFFu;
+              if (!bits) continue;
+              const float d = sc.bias_f16 ? __half2float(__ushort_as_half((unsigned short)bits))
+                                          : __uint_as_float(bits << 16);
+              const float4* bq = reinterpret_cast<const float4*>(sc.bias + (size_t)(q + t) * H + h0);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const float4 b4 = bq[j];
+                v[4 * j] = __float_as_uint(fmaf(d, b4.x, __uint_as_float(v[4 * j])));
+                v[4 * j + 1] = __float_as_uint(fmaf(d, b4.y, __uint_as_float(v[4 * j + 1])));
+                v[4 * j + 2] = __float_as_uint(fmaf(d, b4.z, __uint_as_float(v[4 * j + 2])));
+                v[4 * j + 3] = __float_as_uint(fmaf(d, b4.w, __uint_as_float(v[4 * j + 3])));
+              }
+            }
+          }
         }
         if (part >= 0) {
           // a slice of a split tile: its partial Y, summed with the other slices' by the fix-up
@@ -1572,6 +1602,7 @@ struct GaOps {
   const __nv_bfloat16* X;
   const void* Wk;
   const __nv_bfloat16* b2T;
+  const float* b32;
   float* out;
   __nv_bfloat16 *outb, *outT;
   int64_t ld_outT;
@@ -1591,7 +1622,9 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   if (!make_map_ld(&tx, o.X, n, H, H, lay.box_rows) ||
       !make_map_w(&tw, o.Wk, P, H))
     return cudaErrorInvalidValue;
-  const bool bias_mma = C::BIAS && o.b2T != nullptr;
+  // the bias in fp32 from the epilogue wherever the dense kernel adds it so (Cfg::GM), else as a product
+  const bool bias32 = !BWD && o.b32 && bias_in_fp32(p->S, C::SW);
+  const bool bias_mma = C::BIAS && o.b2T != nullptr && !bias32;
   tdeg = tb2 = tx;
   if (bias_mma && (!make_map(&tdeg, p->d_deg2, n, 64, kTile) || !make_map(&tb2, o.b2T, H, 64, H)))
     return cudaErrorInvalidValue;
@@ -1604,6 +1637,9 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   sc.part = o.split;
   sc.addend = BWD ? nullptr : o.addend;
   sc.slot = p->d_sin_slot;
+  sc.deg = reinterpret_cast<const uint16_t*>(p->d_deg2);
+  sc.bias = bias32 ? o.b32 : nullptr;
+  sc.bias_f16 = p->max_deg > 256 ? 1 : 0;
   e = launch_pdl(k_band_gather<H, BWD>, dim3(std::min(sc.n_items, sms)), dim3(C::THREADS),
                  smem, st, tx, tw, tdeg, tb2, (const uint32_t*)p->d_glist[BWD],
                  (const uint32_t*)p->d_goff[BWD], o.out, o.outb, o.outT, o.ld_outT, o.dM, sc, lay, n, P,
@@ -1786,7 +1822,7 @@ cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, co
   const int n = p->n_pad(), P = p->P;
   if (lists && use_lists(p, H, false))
     return launch_gather_h<false>(
-        p, H, GaOps{X, Wk, b2T, out, outb, outT, ld_outT, nullptr, 0, split, addend}, status, st);
+        p, H, GaOps{X, Wk, b2T, b32, out, outb, outT, ld_outT, nullptr, 0, split, addend}, status, st);
   CUtensorMap tx, tw, tdeg, tb2;
   if (!make_map_box(&tx, X, n, H, H, H < 64 ? 32 : 64, kTile) ||
       !make_map_w(&tw, Wk, P, H) || !make_map(&tdeg, p->d_deg2, n, 64, kTile) ||
@@ -1811,7 +1847,7 @@ cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, c
   const int n = p->n_pad(), P = p->P;
   if (lists && use_lists(p, H, true))
     return launch_gather_h<true>(
-        p, H, GaOps{dY, Wk, nullptr, dE, nullptr, nullptr, 0, dM, accumulate, split, nullptr},
+        p, H, GaOps{dY, Wk, nullptr, nullptr, dE, nullptr, nullptr, 0, dM, accumulate, split, nullptr},
         status, st);
   CUtensorMap tx, tw, tdm;
   const int sw = H < 64 ? 32 : 64;

@@ -176,3 +176,76 @@ def test_lists_run_where_their_rule_says_and_accumulate(S, H, P, F, lam, sizes, 
         # the split's partial sums added in another order: a few units of 2^-24
         d = (a.double() - s.double() - x.double()).abs().max() / x.abs().max()
         assert float(d) < 1e-5, what
+
+
+def _bias_case(H, P, hub, seed):
+    """A plan whose propagation runs on lists at S = 512: program graphs, or one graph with a node of 300
+    in-edges (in-degrees above 256 put the in-degree table and the bias split in fp16)."""
+    from gpu_common import Case
+    if not hub:
+        graphs = [synth.gen_graph(n, P // 2, True, 192, 192, 3.0, seed + i) for i, n in enumerate([900, 333])]
+    else:
+        r = np.random.default_rng(seed)
+        n, m = 400, 500
+        src = np.concatenate([np.arange(1, 301), r.integers(0, n, m)])
+        dst = np.concatenate([np.zeros(300, np.int64), r.integers(1, n, m)])
+        et = np.concatenate([np.zeros(300, np.int64), r.integers(0, P, m)])
+        graphs = [synth.Graph(n, src.astype(np.int32), dst.astype(np.int32), et.astype(np.int32), P)]
+    return Case(graphs, P, 512, H, "bf16", seed=seed)
+
+
+def _bias_run(c, b):
+    """Y of zero states with bias b (so Y = sum_p in-degree_p b_p), by the workspace entry point and the
+    allocation-free one, and the in-degrees [n_pad][P]."""
+    import torch
+    from gpu_common import L, f32_dev
+    assert L.band_uses_lists(c.plan, "bf16", c.H, L.BG_OP_PROPAGATE_FWD)
+    E = torch.zeros((c.N, c.H), dtype=torch.bfloat16, device="cuda")
+    Y, Yn = (torch.full((c.N, c.H), 7.0, device="cuda") for _ in range(2))
+    L.band_propagate_fwd(c.plan, "bf16", c.H, E, c.dprm["W"], f32_dev(b), Y, c.ws(L.BG_OP_PROPAGATE_FWD))
+    L.band_propagate_fwd_noalloc(c.plan, "bf16", c.H, E, c.dprm["W"], f32_dev(b), Yn)
+    torch.cuda.synchronize()
+    deg = np.zeros((c.N, c.P))
+    np.add.at(deg, (c.edges[0], c.edges[2]), 1.0)
+    assert torch.equal(Y.view(torch.int32), Yn.view(torch.int32))
+    return Y.cpu().numpy().astype(np.float64), deg
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H,P,hub,scale", [(64, 20, False, 1.0), (128, 20, False, 1.0), (64, 6, True, 1.0),
+                                           (64, 6, True, 1e-6), (128, 3, True, 1e5)])
+def test_bias_on_lists_is_added_in_fp32(H, P, hub, scale):
+    """At S = 512 and H = 64 or 128 the bias is in-degree times b in fp32, P fused multiply-adds: each
+    entry of Y is within P 2^-24 sum_p in-degree_p |b_p| of the exact sum.  A bias split into two
+    16-bit parts is off by up to 2^-17 (bf16), and as fp16 loses small biases and those above 65504."""
+    from gpu_common import L, ensure_built
+    ensure_built()
+    c = _bias_case(H, P, hub, 41 + H)
+    b = (scale * np.random.default_rng(H + P).standard_normal((P, H))).astype(np.float32)
+    Y, deg = _bias_run(c, b)
+    assert (deg.max() > 256) == hub
+    if scale > 6e4:
+        with pytest.raises(L.BandGGNNError):  # the split, made beside it, still reports |b| > 65504
+            L.check_device()
+    else:
+        L.check_device()
+    want, bound = deg @ b.astype(np.float64), P * 2.0**-24 * (deg @ np.abs(b.astype(np.float64)))
+    assert (np.abs(Y - want) <= bound).all(), float((np.abs(Y - want) - bound).max())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("H", [64, 128])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_non_finite_bias_on_lists_reaches_only_the_rows_with_such_edges(H, value):
+    from gpu_common import L, ensure_built
+    ensure_built()
+    c = _bias_case(H, 20, False, 53 + H)
+    b = np.random.default_rng(3).standard_normal((20, H)).astype(np.float32)
+    b[7, 5] = value
+    Y, deg = _bias_run(c, b)
+    L.check_device()
+    hit = deg[:, 7] > 0
+    assert hit.any() and not hit.all()
+    np.testing.assert_array_equal(Y[hit, 5], value)
+    Y[hit, 5] = 0.0
+    assert np.isfinite(Y).all() and (Y[c.n_real:] == 0.0).all()
