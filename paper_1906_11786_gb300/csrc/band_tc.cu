@@ -62,6 +62,7 @@ using namespace tc;
 namespace {
 
 constexpr int kTile = 128;     // rows per tile = UMMA M
+constexpr int kSmemLimit = 232448;  // dynamic shared memory one block can have
 
 // Block size S: a 128-row tile sees a window of C1 128-column chunks of the state (and of its
 // bit tiles): rows [row0, row0 + 128) only couple to columns in block-rows kr - 1 .. kr + 1 of
@@ -144,7 +145,7 @@ struct Cfg {
   static_assert(NT / G >= NB, "barrier ring");
   static_assert(NA >= CG + 1 && NA <= 8, "one group of A tiles and one more must fit");
   static_assert(GM || (NM >= 2 && NM <= 8), "mask ring");
-  static_assert(SMEM <= 232448, "shared memory");
+  static_assert(SMEM <= kSmemLimit, "shared memory");
 };
 
 struct Bars {
@@ -827,7 +828,7 @@ GaLayout ga_layout(int lo, int rows) {
   // from L2); where that does not fit, the stages before the second window.
   constexpr int kTry[8][2] = {{2, 4}, {2, 3}, {1, 4}, {1, 3}, {2, 2}, {1, 2}, {2, 1}, {1, 1}};
   for (auto& t : kTry)
-    if (t[0] * win + t[1] * C::WSTAGE + C::FIXED <= 232448) {
+    if (t[0] * win + t[1] * C::WSTAGE + C::FIXED <= kSmemLimit) {
       g.nxb = t[0];
       g.nw = t[1];
       break;
@@ -1629,8 +1630,10 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   if (bias_mma && (!make_map(&tdeg, p->d_deg2, n, 64, kTile) || !make_map(&tb2, o.b2T, H, 64, H)))
     return cudaErrorInvalidValue;
   const int smem = lay.nxb * (lay.rows + 8) * 128 + lay.nw * C::WSTAGE + C::FIXED;
+  // the attribute belongs to the kernel, not to this launch: with the plan's own size, a thread with a
+  // smaller plan could lower it between another thread's setting and launch
   cudaError_t e = cudaFuncSetAttribute(k_band_gather<H, BWD>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (e != cudaSuccess) return e;
   const int n_tiles = (n + kTile - 1) / kTile, sms = num_sms();
   Sched sc = make_sched(n_tiles, C::NH * P, sms, o.split != nullptr && n % kTile == 0);

@@ -249,3 +249,53 @@ def test_non_finite_bias_on_lists_reaches_only_the_rows_with_such_edges(H, value
     np.testing.assert_array_equal(Y[hit, 5], value)
     Y[hit, 5] = 0.0
     assert np.isfinite(Y).all() and (Y[c.n_real:] == 0.0).all()
+
+
+@pytest.mark.gpu
+def test_two_threads_with_plans_of_different_windows():
+    """Two host threads propagate on plans whose windows, and so whose shared memory, differ: every call
+    of both succeeds and gives the bits it gives alone."""
+    import threading
+    import torch
+    from gpu_common import Case, L, ensure_built
+    ensure_built()
+    jobs = []
+    for reach, sizes, seed in ((8, [700, 500], 1), (300, [1500, 900], 2)):
+        graphs = [synth.gen_graph(n, 3, False, reach, reach, 3.0, seed + i) for i, n in enumerate(sizes)]
+        c = Case(graphs, 3, 512, 64, "bf16", seed=seed)
+        assert L.band_uses_lists(c.plan, "bf16", 64, L.BG_OP_PROPAGATE_FWD)
+        jobs.append((c, c.ws(L.BG_OP_PROPAGATE_FWD), torch.cuda.Stream()))
+
+    def propagate(c, ws, stream):
+        Y = torch.empty((c.N, 64), device="cuda")
+        L.band_propagate_fwd(c.plan, "bf16", 64, c.E_band_dev, c.dprm["W"], c.dprm["b"], Y, ws,
+                             stream=stream)
+        return Y
+
+    torch.cuda.synchronize()
+    alone = [propagate(c, ws, torch.cuda.current_stream()) for c, ws, _ in jobs]
+    torch.cuda.synchronize()
+    errors, last = [], [None, None]
+    start = threading.Barrier(2)
+
+    def work(i):
+        try:
+            c, ws, stream = jobs[i]
+            with torch.cuda.stream(stream):
+                start.wait()
+                for _ in range(1500):
+                    last[i] = propagate(c, ws, stream)
+                stream.synchronize()
+        except Exception as e:  # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors[0]
+    L.check_device()
+    for a, b in zip(alone, last):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))

@@ -71,6 +71,26 @@ def test_every_device_wait_is_bounded():
     assert re.search(r"for\s*\(\s*uint32_t\s+\w+\s*=\s*0\s*;\s*\w+\s*<\s*kSpinLimit", util)
 
 
+def test_shared_memory_limits_are_constants_of_the_kernel():
+    """cudaFuncSetAttribute changes the kernel for every thread of the process, so the limit it sets
+    must not depend on the plan of one launch: between two threads' settings and launches the smaller
+    one would make the larger one's launch fail.  It is a named constant, or (gru_tc.cu) chosen with
+    the kernel from the state size alone."""
+    seen = 0
+    for f, s in _device_sources().items():
+        s = _strip_comments(s).replace("\\\n", " ")
+        for m in re.finditer(r"cudaFuncSetAttribute\(([^;]*?)\);", s):
+            kernel, attr, value = re.fullmatch(r"(.+),\s*(\w+),\s*(.+)", m.group(1), re.S).groups()
+            assert attr == "cudaFuncAttributeMaxDynamicSharedMemorySize"
+            value = value.strip()
+            if not re.fullmatch(r"(k\w+|\w+(<\w+>)?::SMEM)", value):
+                assert f == "gru_tc.cu" and value == "smem" and kernel == "kern", (f, value)
+                for use in re.findall(r"\bsmem = ([^;]*);", s):
+                    assert not re.search(r"n_pad|n_tiles|->", use), use
+            seen += 1
+    assert seen >= 7
+
+
 def test_no_closed_copy_calls():
     """The batched memcpy entry points are closed on the target machines: no source, header or
     script of the product names them."""
