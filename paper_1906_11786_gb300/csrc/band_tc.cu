@@ -1948,13 +1948,73 @@ bool upload_to(const std::vector<T>& v, T** d, cudaStream_t st) {
 }
 }  // namespace
 
+// Edge lists for the orientations and state sizes that are faster on them and fit.
+static int band_tc_upload_lists(bg_plan* p, int64_t edges, cudaStream_t st) {
+  const int S = p->S;
+  const double cells = (double)(p->n_pad() / kTile) * p->P;  // (tile, type) pairs
+  uint32_t want[2] = {0, 0};
+  // state sizes whose rule `steps` gather steps per (tile, type) meet
+  auto rule = [&](int d, double steps) {
+    uint32_t w = 0;
+    for (int H : {32, 64, 128, 256})
+      if (steps <= gather_max_steps(S, H, d)) w |= 1u << (H / 32);
+    return w;
+  };
+  unsigned dirs = 0;
+  for (int d = 0; d < 2; ++d)
+    if (rule(d, std::max(8.0, (double)edges / 16 / cells))) dirs |= 1u << d;  // full steps at best
+  if (!dirs) return 0;
+  ListScan scan[2];
+  band_tc_scan_lists(p, dirs, scan);
+  std::unique_ptr<uint32_t[]> words[2];
+  uint32_t* to[2] = {nullptr, nullptr};
+  size_t at[2][2], bytes = 0;  // words and offsets of each orientation in one allocation
+  for (int d = 0; d < 2; ++d) {
+    if (!(dirs >> d & 1)) continue;
+    const ListScan& s = scan[d];
+    want[d] = (s.blocks >> 31) ? 0 : rule(d, (double)s.steps / cells);
+    for (int H : {32, 64, 128, 256})
+      if (!(d ? gather_fits<true>(s.lo, s.rows, H) : gather_fits<false>(s.lo, s.rows, H)))
+        want[d] &= ~(1u << (H / 32));
+    if (!want[d]) {
+      dirs &= ~(1u << d);
+      continue;
+    }
+    words[d].reset(to[d] = new uint32_t[(size_t)s.blocks * 32 * kGatherBlock]);
+    at[d][0] = bytes;
+    bytes += al256((size_t)s.blocks * 32 * kGatherBlock * 4);
+    at[d][1] = bytes;
+    bytes += al256(s.off.size() * 4);
+  }
+  if (!dirs) return 0;
+  band_tc_emit_lists(p, dirs, scan, to);
+  if (cudaMalloc(&p->d_lists, bytes) != cudaSuccess) return -1;
+  for (int d = 0; d < 2; ++d) {
+    if (!(dirs >> d & 1)) continue;
+    const ListScan& s = scan[d];
+    p->d_glist[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d][0]);
+    p->d_goff[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d][1]);
+    p->g_lo[d] = s.lo;
+    p->g_rows[d] = s.rows;
+    if (cudaMemcpyAsync(p->d_glist[d], to[d], (size_t)s.blocks * 32 * kGatherBlock * 4,
+                        cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyAsync(p->d_goff[d], s.off.data(), s.off.size() * 4, cudaMemcpyHostToDevice, st) !=
+            cudaSuccess)
+      return -1;
+  }
+  if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
+  for (int d = 0; d < 2; ++d) p->list_h[d] = want[d];
+  return 0;
+}
+
 int band_tc_upload(bg_plan* p, cudaStream_t st) {
   const int S = p->S;
   if (p->P > 32 || (S != 32 && S != 64 && S != 128 && S != 256 && S != 512)) return 0;
   const size_t n = (size_t)p->K * S;
   if (n % kTile) return 0;
   std::vector<uint16_t> deg;
-  p->max_deg = band_tc_host_degrees(p, deg);
+  int64_t edges = 0;
+  p->max_deg = band_tc_host_degrees(p, deg, &edges);
   if (!upload_to(deg, &p->d_deg2, st)) return -1;
   const size_t words = n / kTile * p->P * band_chunks(S) * kTile * 4;
   for (int d = 0; d < 2; ++d) {
@@ -1966,29 +2026,7 @@ int band_tc_upload(bg_plan* p, cudaStream_t st) {
         cudaStreamSynchronize(st) != cudaSuccess)
       return -1;
   }
-  GatherLists lists[2];
-  for (int d = 0; d < 2; ++d) {
-    // each orientation: lists for the state sizes that are faster on them and fit
-    if (gather_max_steps(S, 64, d) == 0) break;
-    const double per = (double)band_tc_list_steps(p, d) / ((double)(n / kTile) * p->P);
-    uint32_t want = 0;
-    for (int H : {32, 64, 128, 256})
-      if (per <= gather_max_steps(S, H, d)) want |= 1u << (H / 32);
-    if (!want) continue;
-    GatherLists& l = lists[d];
-    band_tc_host_lists(p, d, l);
-    for (int H : {32, 64, 128, 256})
-      if ((l.blocks >> 31) ||
-          !(d ? gather_fits<true>(l.lo, l.rows, H) : gather_fits<false>(l.lo, l.rows, H)))
-        want &= ~(1u << (H / 32));
-    if (!want) continue;
-    p->g_lo[d] = l.lo;
-    p->g_rows[d] = l.rows;
-    if (!upload_to(l.words, &p->d_glist[d], st) || !upload_to(l.off, &p->d_goff[d], st)) return -1;
-    p->list_h[d] = want;
-  }
-  if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
-  return 0;
+  return band_tc_upload_lists(p, edges, st);
 }
 
 cudaError_t band_tc_preload_fwd(const bg_plan* p) {
@@ -2021,11 +2059,9 @@ void band_tc_release(bg_plan* p) {
   cudaFree(p->d_maskI);
   cudaFree(p->d_maskTI);
   cudaFree(p->d_deg2);
-  for (int d = 0; d < 2; ++d) {
-    cudaFree(p->d_glist[d]);
-    cudaFree(p->d_goff[d]);
-    p->d_glist[d] = p->d_goff[d] = nullptr;
-  }
+  cudaFree(p->d_lists);
+  p->d_lists = nullptr;
+  for (int d = 0; d < 2; ++d) p->d_glist[d] = p->d_goff[d] = nullptr;
   p->list_h[0] = p->list_h[1] = 0;
   p->d_maskI = p->d_maskTI = nullptr;
   p->d_deg2 = nullptr;

@@ -63,7 +63,8 @@ int band_tc_upload(bg_plan* p, cudaStream_t st);
 // orientations, and the per-row in-degrees [n_pad][64] as bf16; returns the largest in-degree.
 int band_tc_host_tiles(const bg_plan* p, int C1, std::vector<uint32_t>& mi,
                        std::vector<uint32_t>& mti, std::vector<uint16_t>& deg);
-int band_tc_host_degrees(const bg_plan* p, std::vector<uint16_t>& deg);
+// (`edges`, if not NULL: the number of edges in the tiles)
+int band_tc_host_degrees(const bg_plan* p, std::vector<uint16_t>& deg, int64_t* edges = nullptr);
 void band_tc_host_chunks(const bg_plan* p, int C1, bool transposed, uint32_t* out);
 // Edge lists of the gathered band kernel, one orientation.  Per 128-row tile, 16-row group and edge
 // type: steps of 16 edges (at least one) in blocks of kGatherBlock, each step 32 words, one per lane of
@@ -81,7 +82,20 @@ struct GatherLists {
   int lo = 0, rows = 0;
   int64_t steps = 0, blocks = 0;
 };
-// Steps the lists of one orientation would have.
+// Building them takes two passes on host threads, for the orientations (bit 1: transposed) asked for: the
+// edges of every tile with the sizes that follow, then the words themselves (32 kGatherBlock per block,
+// every one written).
+struct ListScan {
+  int lo = 0, rows = 0;
+  int64_t steps = 0, blocks = 0;
+  std::vector<uint32_t> off;                 // as GatherLists::off
+  int unit = 1;                              // tiles that share an array of edges
+  std::vector<std::vector<uint32_t>> edges;  // by tile / unit
+  std::vector<uint32_t> start;               // [n_tiles][8 P + 1]: ranges of (group, type) in them
+};
+void band_tc_scan_lists(const bg_plan* p, unsigned orientations, ListScan* out);
+void band_tc_emit_lists(const bg_plan* p, unsigned orientations, const ListScan* s, uint32_t* const* out);
+// Both at once for one orientation, and the number of steps alone.
 int64_t band_tc_list_steps(const bg_plan* p, bool transposed);
 void band_tc_host_lists(const bg_plan* p, bool transposed, GatherLists& out);
 // Loads (CUDA lazy loading) every kernel band_tc_fwd can launch for this plan's block size, at
