@@ -352,6 +352,12 @@ extern "C" int bg_plan_upload(bg_plan* p, void* stream) {
     free_device(p);
     return rc;
   }
+  // last, so that what is left of the device's memory is all they can take
+  const cudaError_t e = bg::band_tc_upload_lists(p, st);
+  if (e != cudaSuccess) {
+    free_device(p);
+    return bg_fail(BG_ECUDA, std::string("upload of the edge lists: ") + cudaGetErrorString(e));
+  }
   return BG_OK;
 }
 

@@ -1948,8 +1948,7 @@ bool upload_to(const std::vector<T>& v, T** d, cudaStream_t st) {
 }
 }  // namespace
 
-// Edge lists for the orientations and state sizes that are faster on them and fit.
-static int band_tc_upload_lists(bg_plan* p, int64_t edges, cudaStream_t st) {
+static cudaError_t upload_lists(bg_plan* p, cudaStream_t st) {
   const int S = p->S;
   const double cells = (double)(p->n_pad() / kTile) * p->P;  // (tile, type) pairs
   uint32_t want[2] = {0, 0};
@@ -1962,8 +1961,8 @@ static int band_tc_upload_lists(bg_plan* p, int64_t edges, cudaStream_t st) {
   };
   unsigned dirs = 0;
   for (int d = 0; d < 2; ++d)
-    if (rule(d, std::max(8.0, (double)edges / 16 / cells))) dirs |= 1u << d;  // full steps at best
-  if (!dirs) return 0;
+    if (rule(d, std::max(8.0, (double)p->band_edges / 16 / cells))) dirs |= 1u << d;  // full steps at best
+  if (!dirs) return cudaSuccess;
   ListScan scan[2];
   band_tc_scan_lists(p, dirs, scan);
   std::unique_ptr<uint32_t[]> words[2];
@@ -1986,9 +1985,12 @@ static int band_tc_upload_lists(bg_plan* p, int64_t edges, cudaStream_t st) {
     at[d][1] = bytes;
     bytes += al256(s.off.size() * 4);
   }
-  if (!dirs) return 0;
+  if (!dirs) return cudaSuccess;
+  if (cudaMalloc(&p->d_lists, bytes) != cudaSuccess) {
+    p->d_lists = nullptr;
+    return cudaGetLastError();  // (taken off the runtime's record: the caller goes on without lists)
+  }
   band_tc_emit_lists(p, dirs, scan, to);
-  if (cudaMalloc(&p->d_lists, bytes) != cudaSuccess) return -1;
   for (int d = 0; d < 2; ++d) {
     if (!(dirs >> d & 1)) continue;
     const ListScan& s = scan[d];
@@ -1996,15 +1998,26 @@ static int band_tc_upload_lists(bg_plan* p, int64_t edges, cudaStream_t st) {
     p->d_goff[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d][1]);
     p->g_lo[d] = s.lo;
     p->g_rows[d] = s.rows;
-    if (cudaMemcpyAsync(p->d_glist[d], to[d], (size_t)s.blocks * 32 * kGatherBlock * 4,
-                        cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(p->d_goff[d], s.off.data(), s.off.size() * 4, cudaMemcpyHostToDevice, st) !=
-            cudaSuccess)
-      return -1;
+    cudaError_t e = cudaMemcpyAsync(p->d_glist[d], to[d], (size_t)s.blocks * 32 * kGatherBlock * 4,
+                                    cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(p->d_goff[d], s.off.data(), s.off.size() * 4, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
   }
-  if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
   for (int d = 0; d < 2; ++d) p->list_h[d] = want[d];
-  return 0;
+  return cudaSuccess;
+}
+
+cudaError_t band_tc_upload_lists(bg_plan* p, cudaStream_t st) {
+  if (!p->d_deg2 || p->max_deg >= 2048) return cudaSuccess;  // no tensor-core path
+  try {
+    const cudaError_t e = upload_lists(p, st);
+    return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+  } catch (const std::bad_alloc&) {
+    return cudaSuccess;
+  }
 }
 
 int band_tc_upload(bg_plan* p, cudaStream_t st) {
@@ -2013,8 +2026,7 @@ int band_tc_upload(bg_plan* p, cudaStream_t st) {
   const size_t n = (size_t)p->K * S;
   if (n % kTile) return 0;
   std::vector<uint16_t> deg;
-  int64_t edges = 0;
-  p->max_deg = band_tc_host_degrees(p, deg, &edges);
+  p->max_deg = band_tc_host_degrees(p, deg, &p->band_edges);
   if (!upload_to(deg, &p->d_deg2, st)) return -1;
   const size_t words = n / kTile * p->P * band_chunks(S) * kTile * 4;
   for (int d = 0; d < 2; ++d) {
@@ -2026,7 +2038,7 @@ int band_tc_upload(bg_plan* p, cudaStream_t st) {
         cudaStreamSynchronize(st) != cudaSuccess)
       return -1;
   }
-  return band_tc_upload_lists(p, edges, st);
+  return cudaStreamSynchronize(st) == cudaSuccess ? 0 : -1;
 }
 
 cudaError_t band_tc_preload_fwd(const bg_plan* p) {

@@ -58,6 +58,9 @@ cudaError_t prep_transpose_bf16(const void* in, int in_is_f32, __nv_bfloat16* ou
                                 int batch, cudaStream_t st, int64_t ld_out = 0);
 // Builds and uploads the tensor-core path's plan data (no-op where unsupported); 0 on success.
 int band_tc_upload(bg_plan* p, cudaStream_t st);
+// After it: edge lists for the orientations and state sizes that are faster on them and fit.  They are
+// an option: where host or device memory does not suffice, the plan stays without (not an error).
+cudaError_t band_tc_upload_lists(bg_plan* p, cudaStream_t st);
 // Host side of band_tc_upload (band_tiles.cpp): the bit-interleaved window chunks of every
 // 128-row tile, [n_pad / 128][P][C1][128][4] words for C1 128-column chunks per tile, in both
 // orientations, and the per-row in-degrees [n_pad][64] as bf16; returns the largest in-degree.

@@ -63,6 +63,7 @@ struct bg_plan {
   uint32_t* d_maskTI = nullptr;
   uint16_t* d_deg2 = nullptr;
   int32_t max_deg = 0;
+  int64_t band_edges = 0;  // edges in the bit tiles
   // gathered band kernel: edge lists of both orientations (band_tc.h, GatherLists), and the state
   // sizes (bit H / 32) that run on them instead of the chunks above
   uint32_t list_h[2] = {0, 0};

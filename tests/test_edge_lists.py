@@ -135,6 +135,36 @@ def test_building_lists_costs_little_beside_the_tiles(tmp_path):
     raise AssertionError(f"lists / (chunks and degrees): {ratios}")
 
 
+WRAPPED = ("cudaGetDevice", "cudaSetDevice", "cudaMalloc", "cudaFree", "cudaMemcpyAsync", "cudaMemset",
+           "cudaStreamSynchronize", "cudaGetLastError", "cudaGetSymbolAddress", "cudaFuncGetAttributes",
+           "cudaGetDriverEntryPointByVersion")
+
+
+def test_upload_goes_on_without_lists_when_they_find_no_memory(tmp_path):
+    """The edge lists are an option beside the bit tiles: a plan whose tiles fit the device and whose
+    lists do not uploads and runs on the tiles.  (On a fake of the CUDA runtime, each device allocation
+    of an upload failing in turn.)"""
+    B.build()
+    exe, pkg = str(tmp_path / "upload_probe"), os.path.join(ROOT, "paper_1906_11786_gb300")
+    objs = [os.path.join(B.BUILD, f) for f in sorted(os.listdir(B.BUILD)) if f.endswith(".o")]
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", os.path.join(ROOT, "include"),
+                    "-I", "/usr/local/cuda/include", os.path.join(ROOT, "tests", "upload_probe.cpp"), *objs,
+                    "-o", exe, "-L", "/usr/local/cuda/lib64", "-lcudart_static", "-lpthread", "-ldl", "-lrt",
+                    *[f"-Wl,--wrap={w}" for w in WRAPPED]], check=True)
+
+    def run(S, fail):
+        out = subprocess.run([exe, str(S), str(fail)], check=True, capture_output=True, text=True).stdout
+        return [int(x) for x in out.split()]
+
+    status, allocs, tc, fwd, bwd, left, held = run(256, 0)
+    assert (status, tc, fwd, bwd, left, held) == (0, 1, 1, 1, 0, 0)
+    for fail in range(1, allocs):
+        status, _, _, _, _, _, held = run(256, fail)
+        assert status != 0 and held == 0, fail
+    assert run(256, allocs)[:6] == [0, allocs, 1, 0, 0, 0] and run(256, allocs)[6] == 0
+    assert run(128, 0)[1:5] == [allocs - 1, 1, 0, 0]  # no lists at narrow bands
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("S,H,P,F,lam,sizes", [
     (256, 64, 20, 10, 3.0, [1500, 900]), (256, 128, 20, 10, 3.0, [2000]), (256, 32, 5, 5, 1.0, [257]),
