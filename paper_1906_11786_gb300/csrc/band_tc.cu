@@ -769,25 +769,25 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 // against the dense kernel's 457; S = 256, H = 128, 20k nodes backward: 61 us against 89 (ncu).
 //
 // Roles (24 warps, one CTA per SM, persistent over the same items as k_band_tc):
-//   warp 0       TMA producer: state windows, W tiles, deg, bias
+//   warp 0       TMA producer: W tiles
+//   warp 2       TMA producer: state windows, deg, bias
 //   warp 1       TMEM allocator and issuer of the second product and the bias product
-//   warps 4-7    epilogue, Y from TMEM (two accumulators up to H = 128, so it overlaps)
+//   warps 4-7    epilogue, Y from TMEM (two accumulators, so it overlaps) and the fp32 bias
 //   warps 8-23   gather: 8 warps of 16 rows for the even types, 8 for the odd ones
 template <int H, bool BWD>
 struct GaCfg {
+  static_assert(H == 32 || H == 64 || H == 128, "state sizes with wide bands");
   static constexpr int SW = H < 64 ? 32 : 64;
   static constexpr int NH = H / SW;
   static constexpr int NT = SW / 8;                     // accumulator n-tiles
   static constexpr int YC = H < 64 ? 64 : H;            // TMEM columns of one Y
-  static constexpr int NY = H <= 128 ? 2 : 1;
+  static constexpr int NY = 2;
   static constexpr int UC = 64;                         // columns of one pre_p unit
   static constexpr int UCOL = NY * YC;
   static constexpr int NU0 = (512 - UCOL) / UC;
   static constexpr int NU = NU0 > 6 ? 6 : NU0;
-  // W stages as in k_band_tc: fp32 K-columns of W_p^T in 32-column atoms of H rows
-  static constexpr int WK = H <= 128 ? SW : 32;
-  static constexpr int WJ = SW / WK;
-  static constexpr int WSTAGE = (WK / 32) * H * 128;
+  // a W stage as in k_band_tc: SW fp32 K-columns of W_p^T in 32-column atoms of H rows
+  static constexpr int WSTAGE = (SW / 32) * H * 128;
   static constexpr bool BIAS = !BWD;                    // bias as a product
   static constexpr int DEG = BIAS ? kTile * 128 : 0;
   static constexpr int B2 = BIAS ? H * 128 : 0;
@@ -935,9 +935,8 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
                   const __grid_constant__ CUtensorMap tm_deg,
                   const __grid_constant__ CUtensorMap tm_b2, const uint32_t* __restrict__ words,
                   const uint32_t* __restrict__ off, float* __restrict__ out,
-                  __nv_bfloat16* __restrict__ outb, __nv_bfloat16* __restrict__ outT,
-                  int64_t ld_outT, __nv_bfloat16* __restrict__ dM, const Sched sc, const GaLayout lay, int n, int P, int has_bias,
-                  int bias_f16, int accumulate, int* status) {
+                  __nv_bfloat16* __restrict__ dM, const Sched sc, const GaLayout lay, int P,
+                  int has_bias, int bias_f16, int accumulate, int* status) {
   using C = GaCfg<H, BWD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -999,18 +998,16 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
       item_of(sc, w, jobs, k, j0, j1, part);
       int hh = j0 / P, p = j0 - hh * P;
       for (int jb = j0; jb < j1 && ok; ++jb, p = p + 1 == P ? (++hh, 0) : p + 1) {
-        for (int wj = 0; wj < C::WJ; ++wj) {
-          if (!mbar_wait(&bars->w_empty[wi], (wph & 1) ^ 1, status, 153, abort)) {
-            ok = false;
-            break;
-          }
-          ++n_w[wi];
-          mbar_expect_tx(&bars->w_full[wi], C::WSTAGE);
-          for (int a = 0; a < C::WK / 32; ++a)
-            tma_load_2d(wring + wi * C::WSTAGE + a * H * 128, &tm_w, &bars->w_full[wi],
-                        C::SW * hh + C::WK * wj + 32 * a, p * H);
-          if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
+        if (!mbar_wait(&bars->w_empty[wi], (wph & 1) ^ 1, status, 153, abort)) {
+          ok = false;
+          break;
         }
+        ++n_w[wi];
+        mbar_expect_tx(&bars->w_full[wi], C::WSTAGE);
+        for (int a = 0; a < C::SW / 32; ++a)
+          tma_load_2d(wring + wi * C::WSTAGE + a * H * 128, &tm_w, &bars->w_full[wi],
+                      C::SW * hh + 32 * a, p * H);
+        if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
       }
     }
     if (*abort)
@@ -1079,24 +1076,20 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
           break;
         }
         const uint32_t ucol = tmem + C::UCOL + u * C::UC;
-        for (int wj = 0; wj < C::WJ; ++wj) {
-          if (!mbar_wait(&bars->w_full[wi], wph & 1, status, 252, abort)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t wbase = smem_u32(wring + wi * C::WSTAGE);
-          const bool first = jb == j0 && wj == 0;
-#pragma unroll
-          for (int kk = 0; kk < C::WK / 8; ++kk)
-            if (leader)
-              mma_ts_tf32(ycol, ucol + C::WK * wj + kk * 8,
-                          desc_sw128_kmajor(wbase + (kk / 4) * H * 128 + (kk % 4) * 32), idesc,
-                          (first && kk == 0) ? 0u : 1u);
-          if (leader) tc_commit(&bars->w_empty[wi]);
-          if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
+        if (!mbar_wait(&bars->w_full[wi], wph & 1, status, 252, abort)) {
+          ok = false;
+          break;
         }
-        if (!ok) break;
+        tc_fence_after();
+        const uint32_t wbase = smem_u32(wring + wi * C::WSTAGE);
+#pragma unroll
+        for (int kk = 0; kk < C::SW / 8; ++kk)
+          if (leader)
+            mma_ts_tf32(ycol, ucol + kk * 8,
+                        desc_sw128_kmajor(wbase + (kk / 4) * H * 128 + (kk % 4) * 32), idesc,
+                        (jb == j0 && kk == 0) ? 0u : 1u);
+        if (leader) tc_commit(&bars->w_empty[wi]);
+        if (++wi == (uint32_t)lay.nw) wi = 0, ++wph;
         if (leader) tc_commit(&bars->u_empty[u]);
         if (++u == (uint32_t)C::NU) u = 0, ++uph;
       }
@@ -1130,8 +1123,6 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
       int k, j0, j1, part;
       item_of(sc, w, jobs, k, j0, j1, part);
       const int row = k * kTile + r, yb = i % C::NY;
-      const bool live = row < n;
-      const int asl = (!BWD && sc.addend && part < 0 && live) ? sc.slot[row] : -1;
       if (!mbar_wait(&bars->y_full[yb], (i / C::NY) & 1, status, 452, abort, 64)) break;
       tc_fence_after();
 #pragma unroll 1
@@ -1143,12 +1134,6 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
         if (h0 + 32 >= H) {
           tc_fence_before();
           warp_arrive(&bars->y_empty[yb]);
-        }
-        if (!live) continue;
-        if (asl >= 0) {
-          const float* ad = sc.addend + (size_t)asl * H + h0;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + ad[j]);
         }
         if (!BWD && sc.bias && part <= 0) {
           // the bias in fp32, as the dense kernel adds it at these shapes: the in-degrees of two types
@@ -1185,45 +1170,23 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
                                __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
           continue;
         }
-        if (out) {
-          float4* o = reinterpret_cast<float4*>(out + (size_t)row * H + h0);
+        float4* o = reinterpret_cast<float4*>(out + (size_t)row * H + h0);
 #pragma unroll
-          for (int jh = 0; jh < 8; jh += 4) {
-            float4 prev[4];
+        for (int jh = 0; jh < 8; jh += 4) {
+          float4 prev[4];
+          if (accumulate) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) prev[j] = o[jh + j];
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t* vj = v + 4 * (jh + j);
+            float4 a = make_float4(__uint_as_float(vj[0]), __uint_as_float(vj[1]),
+                                   __uint_as_float(vj[2]), __uint_as_float(vj[3]));
             if (accumulate) {
-#pragma unroll
-              for (int j = 0; j < 4; ++j) prev[j] = o[jh + j];
+              a.x += prev[j].x; a.y += prev[j].y; a.z += prev[j].z; a.w += prev[j].w;
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const uint32_t* vj = v + 4 * (jh + j);
-              float4 a = make_float4(__uint_as_float(vj[0]), __uint_as_float(vj[1]),
-                                     __uint_as_float(vj[2]), __uint_as_float(vj[3]));
-              if (accumulate) {
-                a.x += prev[j].x; a.y += prev[j].y; a.z += prev[j].z; a.w += prev[j].w;
-              }
-              o[jh + j] = a;
-            }
-          }
-        }
-        if (outb || outT) {
-          uint32_t pk[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            pk[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-          if (outb) {
-            uint4* ob = reinterpret_cast<uint4*>(outb + (size_t)row * H + h0);
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              ob[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
-          }
-          if (outT) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              __nv_bfloat16* d = outT + (size_t)(h0 + 2 * j) * ld_outT + row;
-              d[0] = __ushort_as_bfloat16((unsigned short)(pk[j] & 0xFFFFu));
-              d[ld_outT] = __ushort_as_bfloat16((unsigned short)(pk[j] >> 16));
-            }
+            o[jh + j] = a;
           }
         }
       }
@@ -1605,12 +1568,9 @@ struct GaOps {
   const __nv_bfloat16* b2T;
   const float* b32;
   float* out;
-  __nv_bfloat16 *outb, *outT;
-  int64_t ld_outT;
   __nv_bfloat16* dM;
   int accumulate;
   float* split;
-  const float* addend;
 };
 
 template <int H, bool BWD>
@@ -1635,25 +1595,22 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   cudaError_t e = cudaFuncSetAttribute(k_band_gather<H, BWD>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
   if (e != cudaSuccess) return e;
-  const int n_tiles = (n + kTile - 1) / kTile, sms = num_sms();
-  Sched sc = make_sched(n_tiles, C::NH * P, sms, o.split != nullptr && n % kTile == 0);
+  const int sms = num_sms();
+  Sched sc = make_sched(n / kTile, C::NH * P, sms, o.split != nullptr);
   sc.part = o.split;
-  sc.addend = BWD ? nullptr : o.addend;
-  sc.slot = p->d_sin_slot;
   sc.deg = reinterpret_cast<const uint16_t*>(p->d_deg2);
   sc.bias = bias32 ? o.b32 : nullptr;
   sc.bias_f16 = p->max_deg > 256 ? 1 : 0;
   e = launch_pdl(k_band_gather<H, BWD>, dim3(std::min(sc.n_items, sms)), dim3(C::THREADS),
                  smem, st, tx, tw, tdeg, tb2, (const uint32_t*)p->d_glist[BWD],
-                 (const uint32_t*)p->d_goff[BWD], o.out, o.outb, o.outT, o.ld_outT, o.dM, sc, lay, n, P,
-                 bias_mma ? 1 : 0, p->max_deg > 256 ? 1 : 0, o.accumulate, status);
+                 (const uint32_t*)p->d_goff[BWD], o.out, o.dM, sc, lay, P, bias_mma ? 1 : 0, p->max_deg > 256 ? 1 : 0, o.accumulate, status);
   note_launch();
   if (e != cudaSuccess || sc.ksplit == 1) return e;
   const int64_t n4 = (int64_t)sc.part_rows * H / 4;
   e = launch_pdl(k_band_split_fixup, dim3((unsigned)std::min<int64_t>((n4 + 255) / 256, 2048)),
                  dim3(256), 0, st, (const float*)o.split, sc.ksplit, sc.part_rows,
-                 sc.n_full * kTile, H, o.out, o.outb, o.outT, o.ld_outT, o.accumulate, sc.addend,
-                 sc.slot);
+                 sc.n_full * kTile, H, o.out, (__nv_bfloat16*)nullptr, (__nv_bfloat16*)nullptr, (int64_t)0,
+                 o.accumulate, (const float*)nullptr, (const int32_t*)nullptr);
   note_launch();
   return e;
 }
@@ -1664,7 +1621,7 @@ cudaError_t launch_gather_h(const bg_plan* p, int H, const GaOps& o, int* status
     case 32: return launch_gather<32, BWD>(p, o, status, st);
     case 64: return launch_gather<64, BWD>(p, o, status, st);
     case 128: return launch_gather<128, BWD>(p, o, status, st);
-    default: return launch_gather<256, BWD>(p, o, status, st);
+    default: return cudaErrorInvalidValue;
   }
 }
 
@@ -1674,7 +1631,6 @@ bool gather_fits(int lo, int rows, int H) {
     case 32: return ga_layout<32, BWD>(lo, rows).nxb > 0;
     case 64: return ga_layout<64, BWD>(lo, rows).nxb > 0;
     case 128: return ga_layout<128, BWD>(lo, rows).nxb > 0;
-    case 256: return ga_layout<256, BWD>(lo, rows).nxb > 0;
     default: return false;
   }
 }
@@ -1691,9 +1647,9 @@ bool gather_fits(int lo, int rows, int H) {
 // 52 edges per node, and the lists are not built there.
 int gather_max_steps(int S, int H, bool bwd) {
   if (S != 256 && S != 512) return 0;
-  const int h = H == 32 ? 0 : H == 64 ? 1 : H == 128 ? 2 : 3;
-  static constexpr int kMax[2][2][4] = {{{100, 70, 80, 0}, {80, 60, 68, 0}},      // S = 256
-                                        {{200, 160, 200, 0}, {200, 110, 200, 0}}};  // S = 512
+  const int h = H == 32 ? 0 : H == 64 ? 1 : 2;
+  static constexpr int kMax[2][2][3] = {{{100, 70, 80}, {80, 60, 68}},      // S = 256
+                                        {{200, 160, 200}, {200, 110, 200}}};  // S = 512
   return kMax[S == 512][bwd][h];
 }
 
@@ -1823,9 +1779,8 @@ cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, co
                              float* split, const float* addend, int* status, cudaStream_t st,
                              bool lists) {
   const int n = p->n_pad(), P = p->P;
-  if (lists && use_lists(p, H, false))
-    return launch_gather_h<false>(
-        p, H, GaOps{X, Wk, b2T, b32, out, outb, outT, ld_outT, nullptr, 0, split, addend}, status, st);
+  if (lists && use_lists(p, H, false) && !outb && !outT && !addend)
+    return launch_gather_h<false>(p, H, GaOps{X, Wk, b2T, b32, out, nullptr, 0, split}, status, st);
   CUtensorMap tx, tw, tdeg, tb2;
   if (!make_map_box(&tx, X, n, H, H, H < 64 ? 32 : 64, kTile) ||
       !make_map_w(&tw, Wk, P, H) || !make_map(&tdeg, p->d_deg2, n, 64, kTile) ||
@@ -1849,9 +1804,8 @@ cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, c
                              int* status, cudaStream_t st, bool lists) {
   const int n = p->n_pad(), P = p->P;
   if (lists && use_lists(p, H, true))
-    return launch_gather_h<true>(
-        p, H, GaOps{dY, Wk, nullptr, nullptr, dE, nullptr, nullptr, 0, dM, accumulate, split, nullptr},
-        status, st);
+    return launch_gather_h<true>(p, H, GaOps{dY, Wk, nullptr, nullptr, dE, dM, accumulate, split},
+                                 status, st);
   CUtensorMap tx, tw, tdm;
   const int sw = H < 64 ? 32 : 64;
   if (!make_map_box(&tx, dY, n, H, H, sw, kTile) || !make_map_w(&tw, Wk, P, H) ||
@@ -1955,7 +1909,7 @@ static cudaError_t upload_lists(bg_plan* p, cudaStream_t st) {
   // state sizes whose rule `steps` gather steps per (tile, type) meet
   auto rule = [&](int d, double steps) {
     uint32_t w = 0;
-    for (int H : {32, 64, 128, 256})
+    for (int H : {32, 64, 128})
       if (steps <= gather_max_steps(S, H, d)) w |= 1u << (H / 32);
     return w;
   };
@@ -1972,7 +1926,7 @@ static cudaError_t upload_lists(bg_plan* p, cudaStream_t st) {
     if (!(dirs >> d & 1)) continue;
     const ListScan& s = scan[d];
     want[d] = (s.blocks >> 31) ? 0 : rule(d, (double)s.steps / cells);
-    for (int H : {32, 64, 128, 256})
+    for (int H : {32, 64, 128})
       if (!(d ? gather_fits<true>(s.lo, s.rows, H) : gather_fits<false>(s.lo, s.rows, H)))
         want[d] &= ~(1u << (H / 32));
     if (!want[d]) {
@@ -2063,7 +2017,6 @@ cudaError_t band_tc_preload_fwd(const bg_plan* p) {
   take(cudaFuncGetAttributes(&a, k_band_gather<32, false>));
   take(cudaFuncGetAttributes(&a, k_band_gather<64, false>));
   take(cudaFuncGetAttributes(&a, k_band_gather<128, false>));
-  take(cudaFuncGetAttributes(&a, k_band_gather<256, false>));
   return e;
 }
 

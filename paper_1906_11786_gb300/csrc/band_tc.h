@@ -46,7 +46,7 @@ cudaError_t band_tc_fwd_core(const bg_plan* p, int H, const __nv_bfloat16* X, co
                              const __nv_bfloat16* b2T, const float* b32, float* out,
                              __nv_bfloat16* outb, __nv_bfloat16* outT, int64_t ld_outT,
                              float* split, const float* addend, int* status, cudaStream_t st,
-                             bool lists = false);
+                             bool lists = false);  // (lists: with `out` alone)
 //   dY: [n_pad][H] bf16; Wk: band_tc_prep_w(bwd = 1); dE fp32 (+)=; dM: [n_pad][P*H] bf16, 16-byte
 //   aligned.
 cudaError_t band_tc_bwd_core(const bg_plan* p, int H, const __nv_bfloat16* dY, const void* Wk,
