@@ -232,6 +232,26 @@ __device__ __forceinline__ void item_of(const Sched& sc, int w, int jobs, int& t
   j1 = (part + 1) * jobs / sc.ksplit;
 }
 
+// Lane i of each group of eight holds 16-byte chunks 0 .. 7 (four words each) of its own row; afterwards
+// chunk i of the rows of lanes 0 .. 7.  Every lane of the warp calls it.
+__device__ __forceinline__ void transpose8(uint32_t (&v)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int m = 4; m; m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      if (!(c & m))
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t a = v[4 * c + k], b = v[4 * (c | m) + k];
+          const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? a : b, m);
+          v[4 * c + k] = up ? got : a;
+          v[4 * (c | m) + k] = up ? b : got;
+        }
+  }
+}
+
 template <int H, int S, bool BWD>
 __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
     k_band_tc(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
@@ -629,11 +649,17 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 #pragma unroll
         for (int j = 0; j < C::SW / 2; ++j)
           pk[j] = pack_bf16(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
-        if constexpr (!C::DMS) {
-          uint4* d = reinterpret_cast<uint4*>(dM + ((size_t)row * P + p) * H + C::SW * hh);
+        if constexpr (BWD && !C::DMS) {
+          // no room for a staging tile: eight lanes swap their rows' 16-byte chunks in registers, so that
+          // store j of the group writes row j's slice as one whole line.  (Each lane its own row, 16
+          // bytes at a time, was 6% of a GGNN backward: H = 128, 40k nodes, two steps 1,793 us a call;
+          // lane pairs swapping halves 1,720; so 1,694.)
+          transpose8(pk);
+          uint4* d = reinterpret_cast<uint4*>(dM + ((size_t)(row - (lane & 7)) * P + p) * H + C::SW * hh) +
+                     (lane & 7);
 #pragma unroll
-          for (int j = 0; j < C::SW / 8; ++j)
-            d[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+          for (int j = 0; j < 8; ++j)
+            d[(size_t)j * (P * H / 8)] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
           continue;
         }
         // dM_p (bf16, row-major) through this warp's 32-row staging tile, one bulk store per job

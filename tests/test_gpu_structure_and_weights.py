@@ -318,3 +318,31 @@ def test_block_row_split_on_one_gpu_matches_the_unsplit_launch(S, H, n_parts):
         sb += dbl.cpu().numpy()
     np.testing.assert_allclose(sW, dW, rtol=0, atol=1e-5 * np.abs(dW).max())
     np.testing.assert_allclose(sb, db, rtol=0, atol=1e-5 * np.abs(db).max())
+
+
+@pytest.mark.parametrize("H", [32, 64, 128])
+def test_ggnn_fwd_bwd_at_S512(H):
+    """GGNN steps at S = 512 multiply the bit tiles whatever single propagations do; at H = 128 the
+    backward has no staging tile for dM and writes whole lines after swapping chunks between lanes."""
+    gs = [synth.gen_graph(n, 3, True, 192, 192, 2.0, 70 + n) for n in (700, 450)]
+    c = Case(gs, 6, 512, H, "bf16", seed=H)
+    assert L.band_uses_tensor_cores(c.plan, "bf16", H)
+    T = 2
+    saved = torch.empty(L.ggnn_saved_bytes(c.plan, "bf16", H, T), dtype=torch.uint8, device="cuda")
+    ET = torch.empty((c.N, H), dtype=torch.bfloat16, device="cuda")
+    L.ggnn_step(c.plan, "bf16", H, T, c.dprm, c.E_band_dev, ET, saved, c.ws(L.BG_OP_GGNN_FWD, T))
+    dET = np.zeros((c.N, H))
+    dET[: c.n_real] = np.random.default_rng(8).standard_normal((c.n_real, H)).astype(np.float32)
+    grads = {"d" + k: torch.empty(tuple(c.dprm[k].shape), device="cuda")
+             for k in ("W", "b", "W_ih", "W_hh", "b_ih", "b_hh")}
+    dE0 = torch.empty((c.N, H), device="cuda")
+    L.ggnn_step_bwd(c.plan, "bf16", H, T, c.dprm, saved, f32_dev(dET), dE0, grads,
+                    c.ws(L.BG_OP_GGNN_BWD, T))
+    torch.cuda.synchronize()
+    L.check_device()
+    Es, Ys = oracle.ggnn_fwd(c.N, c.P, H, T, c.n_real, *c.edges, c.E_band, c.prm)
+    ref = oracle.ggnn_bwd(c.N, c.P, H, T, c.n_real, *c.edges, c.prm, Es, Ys, dET)
+    assert_close(ET.float().cpu().numpy(), Es[T], TOL["bf16"], "ET")
+    assert_close(dE0.cpu().numpy(), ref["dE0"], TOL["bf16"], "dE0")
+    for k, v in grads.items():
+        assert_close(v.cpu().numpy(), ref[k], TOL["bf16"], k)
