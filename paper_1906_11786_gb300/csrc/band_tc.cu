@@ -1943,61 +1943,78 @@ static cudaError_t upload_lists(bg_plan* p, cudaStream_t st) {
   for (int d = 0; d < 2; ++d)
     if (rule(d, std::max(8.0, (double)p->band_edges / 16 / cells))) dirs |= 1u << d;  // full steps at best
   if (!dirs) return cudaSuccess;
-  ListScan scan[2];
-  band_tc_scan_lists(p, dirs, scan);
-  std::unique_ptr<uint32_t[]> words[2];
-  uint32_t* to[2] = {nullptr, nullptr};
-  size_t at[2][2], bytes = 0;  // words and offsets of each orientation in one allocation
+  // the edges per (tile, group, type) counted on the device, in the place of their offsets
+  const size_t n_off = (size_t)p->n_pad() / 16 * (p->P + 1), off_bytes = al256(n_off * 4);
+  auto alloc = [](char** d, size_t bytes) {
+    if (cudaMalloc(d, bytes) == cudaSuccess) return true;
+    *d = nullptr;
+    cudaGetLastError();  // taken off the runtime's record: the caller goes on without lists
+    return false;
+  };
+  if (!alloc(&p->d_list_off, 2 * off_bytes + 256)) return cudaErrorMemoryAllocation;
+  int* d_reach = reinterpret_cast<int*>(p->d_list_off + 2 * off_bytes);
+  cudaError_t e = cudaMemsetAsync(d_reach, 0, 16, st);
+  int reach[4];
+  GatherLists l[2];
+  for (int d = 0; d < 2 && e == cudaSuccess; ++d) {
+    if (!(dirs >> d & 1)) continue;
+    p->d_goff[d] = reinterpret_cast<uint32_t*>(p->d_list_off + d * off_bytes);
+    l[d].off.resize(n_off);
+    e = list_count(p, d, p->d_goff[d], d_reach + 2 * d, st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(l[d].off.data(), p->d_goff[d], n_off * 4, cudaMemcpyDeviceToHost, st);
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(reach, d_reach, 16, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return e;
+  size_t at[2], bytes = 0;
   for (int d = 0; d < 2; ++d) {
     if (!(dirs >> d & 1)) continue;
-    const ListScan& s = scan[d];
-    want[d] = (s.blocks >> 31) ? 0 : rule(d, (double)s.steps / cells);
+    list_layout(p, reach + 2 * d, l[d]);
+    want[d] = (l[d].blocks >> 31) ? 0 : rule(d, (double)l[d].steps / cells);
     for (int H : {32, 64, 128})
-      if (!(d ? gather_fits<true>(s.lo, s.rows, H) : gather_fits<false>(s.lo, s.rows, H)))
+      if (!(d ? gather_fits<true>(l[d].lo, l[d].rows, H) : gather_fits<false>(l[d].lo, l[d].rows, H)))
         want[d] &= ~(1u << (H / 32));
     if (!want[d]) {
       dirs &= ~(1u << d);
       continue;
     }
-    words[d].reset(to[d] = new uint32_t[(size_t)s.blocks * 32 * kGatherBlock]);
-    at[d][0] = bytes;
-    bytes += al256((size_t)s.blocks * 32 * kGatherBlock * 4);
-    at[d][1] = bytes;
-    bytes += al256(s.off.size() * 4);
+    at[d] = bytes;
+    bytes += al256((size_t)l[d].blocks * 32 * kGatherBlock * 4);
   }
   if (!dirs) return cudaSuccess;
-  if (cudaMalloc(&p->d_lists, bytes) != cudaSuccess) {
-    p->d_lists = nullptr;
-    return cudaGetLastError();  // (taken off the runtime's record: the caller goes on without lists)
-  }
-  band_tc_emit_lists(p, dirs, scan, to);
-  for (int d = 0; d < 2; ++d) {
+  if (!alloc(&p->d_lists, bytes)) return cudaErrorMemoryAllocation;
+  for (int d = 0; d < 2 && e == cudaSuccess; ++d) {
     if (!(dirs >> d & 1)) continue;
-    const ListScan& s = scan[d];
-    p->d_glist[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d][0]);
-    p->d_goff[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d][1]);
-    p->g_lo[d] = s.lo;
-    p->g_rows[d] = s.rows;
-    cudaError_t e = cudaMemcpyAsync(p->d_glist[d], to[d], (size_t)s.blocks * 32 * kGatherBlock * 4,
-                                    cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(p->d_goff[d], s.off.data(), s.off.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
+    p->d_glist[d] = reinterpret_cast<uint32_t*>(p->d_lists + at[d]);
+    p->g_lo[d] = l[d].lo;
+    p->g_rows[d] = l[d].rows;
+    e = cudaMemcpyAsync(p->d_goff[d], l[d].off.data(), n_off * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = list_emit(p, d, p->d_goff[d], l[d].lo, l[d].rows, p->d_glist[d], st);
   }
-  const cudaError_t e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return e;
   for (int d = 0; d < 2; ++d) p->list_h[d] = want[d];
   return cudaSuccess;
 }
 
+static void free_lists(bg_plan* p) {
+  cudaFree(p->d_lists);
+  cudaFree(p->d_list_off);
+  p->d_lists = p->d_list_off = nullptr;
+  for (int d = 0; d < 2; ++d) p->d_glist[d] = p->d_goff[d] = nullptr;
+  p->list_h[0] = p->list_h[1] = 0;
+}
+
 cudaError_t band_tc_upload_lists(bg_plan* p, cudaStream_t st) {
   if (!p->d_deg2 || p->max_deg >= 2048) return cudaSuccess;  // no tensor-core path
+  cudaError_t e = cudaErrorMemoryAllocation;
   try {
-    const cudaError_t e = upload_lists(p, st);
-    return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    e = upload_lists(p, st);
   } catch (const std::bad_alloc&) {
-    return cudaSuccess;
   }
+  if (!p->list_h[0] && !p->list_h[1]) free_lists(p);
+  return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
 }
 
 int band_tc_upload(bg_plan* p, cudaStream_t st) {
@@ -2050,10 +2067,7 @@ void band_tc_release(bg_plan* p) {
   cudaFree(p->d_maskI);
   cudaFree(p->d_maskTI);
   cudaFree(p->d_deg2);
-  cudaFree(p->d_lists);
-  p->d_lists = nullptr;
-  for (int d = 0; d < 2; ++d) p->d_glist[d] = p->d_goff[d] = nullptr;
-  p->list_h[0] = p->list_h[1] = 0;
+  free_lists(p);
   p->d_maskI = p->d_maskTI = nullptr;
   p->d_deg2 = nullptr;
 }

@@ -85,20 +85,15 @@ struct GatherLists {
   int lo = 0, rows = 0;
   int64_t steps = 0, blocks = 0;
 };
-// Building them takes two passes on host threads, for the orientations (bit 1: transposed) asked for: the
-// edges of every tile with the sizes that follow, then the words themselves (32 kGatherBlock per block,
-// every one written).
-struct ListScan {
-  int lo = 0, rows = 0;
-  int64_t steps = 0, blocks = 0;
-  std::vector<uint32_t> off;                 // as GatherLists::off
-  int unit = 1;                              // tiles that share an array of edges
-  std::vector<std::vector<uint32_t>> edges;  // by tile / unit
-  std::vector<uint32_t> start;               // [n_tiles][8 P + 1]: ranges of (group, type) in them
-};
-void band_tc_scan_lists(const bg_plan* p, unsigned orientations, ListScan* out);
-void band_tc_emit_lists(const bg_plan* p, unsigned orientations, const ListScan* s, uint32_t* const* out);
-// Both at once for one orientation, and the number of steps alone.
+// On the device (band_lists.cu): the edges of each (tile, group, type) in the place of its offset, types in
+// the lists' order, with the window's reach before and behind the tile (two ints, cleared before); then,
+// with the offsets in place, the words (32 kGatherBlock per block, every one written).
+cudaError_t list_count(const bg_plan* p, bool transposed, uint32_t* d_off, int* d_reach, cudaStream_t st);
+cudaError_t list_emit(const bg_plan* p, bool transposed, const uint32_t* d_off, int lo, int rows,
+                      uint32_t* d_words, cudaStream_t st);
+// Their sizes: counts in `off` become offsets, `reach` becomes lo and rows.
+void list_layout(const bg_plan* p, const int* reach, GatherLists& out);
+// The same lists built on the host, and the number of their steps alone: what tests compare with.
 int64_t band_tc_list_steps(const bg_plan* p, bool transposed);
 void band_tc_host_lists(const bg_plan* p, bool transposed, GatherLists& out);
 // Loads (CUDA lazy loading) every kernel band_tc_fwd can launch for this plan's block size, at

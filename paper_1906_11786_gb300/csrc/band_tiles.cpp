@@ -178,230 +178,201 @@ int band_tc_host_degrees(const bg_plan* p, std::vector<uint16_t>& deg, int64_t* 
 
 
 namespace {
+// Gather steps of one type of a 16-row group (at least one).
+inline uint32_t list_steps(uint32_t edges) { return std::max<uint32_t>(1, (edges + 15) / 16); }
+}  // namespace
 
-constexpr int kListTile = 128, kGroups = kListTile / 16;  // rows of a tile, 16-row groups of one
-
-// Position of the i-th type in a group's order: the even types, then the odd ones (the kernel's two
-// classes of warps).
-inline int type_at(int i, int P) { return i < (P + 1) / 2 ? 2 * i : 2 * (i - (P + 1) / 2) + 1; }
-inline uint32_t steps_of(uint32_t edges) { return std::max<uint32_t>(1, (edges + 15) / 16); }
-
-// One 16-row group's edges of one type (row within the group << 16 | column - tile + 2048) as blocks of
-// gather steps of 16 edges at `out` (the format: band_tc.h).  `add` turns the low half into the window
-// row.  ldmatrix reads 8 window rows at once from one 16-byte column, so a set of 8 edges whose window
-// rows differ mod 8 reads all 32 banks and one whose rows agree serialises: the edges are dealt into
-// sets by taking the fullest residues first, and padding entries take a zero row of an unused residue.
-void emit_type(const uint32_t* e, int n, uint32_t add, uint32_t zero_row, uint32_t* out,
-               std::vector<uint32_t>& tmp) {
-  const int steps = (int)steps_of((uint32_t)n);
-  uint32_t cnt[8] = {0}, pos[8], at[8];
-  for (int i = 0; i < n; ++i) ++cnt[e[i] & 7];  // (add is a multiple of 8)
-  for (uint32_t r = 0, o = 0; r < 8; ++r) { pos[r] = at[r] = o; o += cnt[r]; }
-  if (tmp.size() < (size_t)n) tmp.resize((size_t)n);
-  for (int i = 0; i < n; ++i) tmp[at[e[i] & 7]++] = e[i] + add;
-  int rem = n;
-  uint32_t blk[32][kGatherBlock];
-  for (int s = 0; s < steps; ++s) {
-    const int in_blk = s % kGatherBlock;
-    if (in_blk == 0) std::memset(blk, 0, sizeof(blk));
-    uint32_t ent[16], bits[32] = {0};
-    for (int half = 0; half < 2; ++half) {
-      const int need = std::max(0, rem - 8 * (2 * (steps - s) - half - 1));
-      uint32_t* x = ent + 8 * half;
-      int k = 0;
-      unsigned used = 0;
-      auto take = [&](int r) {
-        const uint32_t v = x[k] = tmp[pos[r]++], row = v >> 16;
-        --cnt[r];
-        bits[(row & 7) * 4 + k / 2] |= 1u << (24 + (row >> 3) + 2 * half + 4 * (k & 1));
-        ++k;
-      };
-      if (rem) {
-        // one edge of every residue left, the fullest first (by residue where equal)
-        uint32_t key[8];
-        for (uint32_t r = 0; r < 8; ++r) key[r] = cnt[r] << 3 | (7 - r);
-        auto order = [&](int a, int b) {
-          const uint32_t hi = std::max(key[a], key[b]), lo = std::min(key[a], key[b]);
-          key[a] = hi, key[b] = lo;
-        };
-        order(0, 1); order(2, 3); order(4, 5); order(6, 7);
-        order(0, 2); order(1, 3); order(4, 6); order(5, 7);
-        order(1, 2); order(5, 6);
-        order(0, 4); order(1, 5); order(2, 6); order(3, 7);
-        order(2, 4); order(3, 5);
-        order(1, 2); order(3, 4); order(5, 6);
-        for (int i = 0; i < 8 && key[i] >= 8; ++i) {
-          const int r = 7 - (int)(key[i] & 7);
-          take(r);
-          used |= 1u << r;
-        }
-        while (k < need) take((int)(std::max_element(cnt, cnt + 8) - cnt));
-        rem -= k;
-      }
-      for (int r = 0; k < 8; r = (r + 1) & 7) {
-        if (!(used >> r & 1)) {
-          x[k++] = zero_row + r;
-          used |= 1u << r;
-        } else if (used == 0xFF) {
-          used = 0;
-        }
-      }
+void list_layout(const bg_plan* p, const int* reach, GatherLists& out) {
+  const int P = p->P;
+  auto up8 = [](int x) { return (x + 7) & ~7; };
+  out.lo = up8(reach[0]);
+  out.rows = out.lo + 128 + up8(reach[1]);
+  // a whole number of equal TMA boxes of at most 256 rows
+  const int boxes = (out.rows + 255) / 256;
+  out.rows = up8((out.rows + boxes - 1) / boxes) * boxes;
+  // per 16-row group: the even types, then the odd ones (the kernel's two classes of warps), each
+  // type's steps padded to whole blocks
+  uint64_t total = 0;
+  out.steps = 0;
+  for (size_t o = 0; o < out.off.size(); o += P + 1) {
+    for (int i = 0; i < P; ++i) {
+      const uint32_t ns = list_steps(out.off[o + i]);
+      out.off[o + i] = (uint32_t)total;
+      out.steps += ns;
+      total += (ns + kGatherBlock - 1) / kGatherBlock;
     }
-    const int s0 = s - in_blk, in = std::min(kGatherBlock, steps - s0);
-    const uint32_t flags = (uint32_t)(in - 1) * kGatherMore + (s0 + in == steps ? kGatherLast : 0u);
-    for (int k = 0; k < 16; ++k) {
-      const uint32_t row = ent[k] & 0xFFFFu, w = row * 128u + ((row & 7u) << 4);
-      blk[k][in_blk] = w | flags | bits[k];
-      blk[k + 16][in_blk] = (w ^ 16u) | flags | bits[k + 16];
-    }
-    if (in_blk == in - 1) std::memcpy(out + (size_t)(s / kGatherBlock) * 32 * kGatherBlock, blk, sizeof(blk));
+    out.off[o + P] = (uint32_t)total;
   }
+  out.blocks = (int64_t)total;
 }
 
-// The set bits of `words` 32-bit mask words, in order: f(bit).  Two words at a time where they pair up.
-template <typename F>
-inline void for_bits(const uint32_t* w, int words, F f) {
-  int j = 0;
-  for (; j + 1 < words; j += 2) {
-    uint64_t m;
-    std::memcpy(&m, w + j, 8);  // (both hosts are little-endian)
-    for (; m; m &= m - 1) f(32 * j + __builtin_ctzll(m));
+namespace {
+
+// One 16-row group's edges of one type (row within the group << 16 | window row) as gather steps of
+// 16: `words` gets 32 words per step (see band_tc_host_lists).  ldmatrix reads 8 window rows at
+// once from one 16-byte column, so a set of 8 edges whose window rows differ mod 8 reads all 32
+// banks and one whose rows agree serialises: the edges are dealt into sets by taking the fullest
+// residues first, and padding entries take a zero row of an unused residue.
+void emit_steps(const uint32_t* e, int n, int zero_row, uint32_t* words,
+                std::vector<uint32_t>& tmp) {
+  const int steps = (int)list_steps((uint32_t)n);
+  int cnt[8] = {0}, pos[8];
+  for (int i = 0; i < n; ++i) ++cnt[e[i] & 7];
+  for (int r = 0, o = 0; r < 8; ++r) { pos[r] = o; o += cnt[r]; }
+  tmp.resize((size_t)std::max(n, 1));
+  {
+    int at[8];
+    std::copy(pos, pos + 8, at);
+    for (int i = 0; i < n; ++i) tmp[at[e[i] & 7]++] = e[i];
   }
-  if (j < words)
-    for (uint32_t m = w[j]; m; m &= m - 1) f(32 * j + __builtin_ctz(m));
+  int rem = n;
+  for (int s = 0; s < steps; ++s) {
+    uint32_t ent[16];
+    bool real[16];
+    for (int half = 0; half < 2; ++half) {
+      const int sets_after = 2 * (steps - s) - half - 1;
+      const int need = std::max(0, rem - 8 * sets_after);
+      int order[8] = {0, 1, 2, 3, 4, 5, 6, 7};
+      for (int i = 1; i < 8; ++i)
+        for (int j = i; j > 0 && cnt[order[j]] > cnt[order[j - 1]]; --j) std::swap(order[j], order[j - 1]);
+      bool used[8] = {false};
+      int k = 0;
+      for (int i = 0; i < 8; ++i)
+        if (cnt[order[i]] > 0) {
+          const int r = order[i];
+          ent[8 * half + k] = tmp[pos[r]++];
+          real[8 * half + k++] = true;
+          --cnt[r];
+          used[r] = true;
+        }
+      while (k < need) {
+        const int r = (int)(std::max_element(cnt, cnt + 8) - cnt);
+        ent[8 * half + k] = tmp[pos[r]++];
+        real[8 * half + k++] = true;
+        --cnt[r];
+      }
+      rem -= k;
+      for (int r = 0; k < 8; r = (r + 1) & 7)
+        if (!used[r]) {
+          ent[8 * half + k] = (uint32_t)(zero_row + r);
+          real[8 * half + k++] = false;
+          used[r] = true;
+        } else if (std::all_of(used, used + 8, [](bool u) { return u; })) {
+          std::fill(used, used + 8, false);
+        }
+    }
+    uint32_t* w = words + (size_t)s * 32;
+    for (int l = 0; l < 32; ++l) {
+      const uint32_t row = ent[l & 15] & 0xFFFFu, hi = (uint32_t)(l >> 4);
+      w[l] = row * 128u + ((hi ^ (row & 7u)) << 4);
+    }
+    for (int k = 0; k < 16; ++k)
+      if (real[k]) {
+        const int r = (int)(ent[k] >> 16);
+        w[(r & 7) * 4 + (k & 7) / 2] |= 1u << (24 + (r >> 3) + 2 * (k >> 3) + 4 * (k & 1));
+      }
+  }
 }
 
 }  // namespace
 
-// Edges of one orientation by tile, 16-row group and type, and where their steps will stand.
-void band_tc_scan_lists(const bg_plan* p, unsigned orientations, ListScan* out) {
-  const int S = p->S, K = p->K, P = p->P, W32 = p->W32;
-  const int64_t n = (int64_t)K * S, n_tiles = (n + kListTile - 1) / kListTile;
-  // a unit of tiles shares one array of edges (row in the group << 16 | column - tile + 2048)
-  const int unit = (int)std::min<int64_t>(std::max<int64_t>(1, n_tiles / 64), 64);
-  const int64_t units = (n_tiles + unit - 1) / unit;
-  std::vector<int> todo;
-  for (int d = 0; d < 2; ++d)
-    if (orientations >> d & 1) {
-      todo.push_back(d);
-      out[d].unit = unit;
-      out[d].edges.resize((size_t)units);
-      out[d].start.resize((size_t)n_tiles * (kGroups * P + 1));
-    }
-  const int64_t jobs = units * (int64_t)todo.size();
-  std::vector<int> lo((size_t)jobs, 0), hi((size_t)jobs, 0);
-  parallel_ranges(jobs, [&](int64_t w0, int64_t w1) {
-    for (int64_t w = w0; w < w1; ++w) {
-      const int tr = todo[(size_t)(w / units)];
-      const int64_t u = w % units;
-      const std::vector<uint32_t>& masks = tr ? p->masksT : p->masks;
-      std::vector<uint32_t>& ed = out[tr].edges[(size_t)u];
-      int l = 0, h = 0;
-      for (int64_t t = u * unit; t < std::min(n_tiles, (u + 1) * unit); ++t) {
-        const int64_t row0 = t * kListTile;
-        uint32_t* st = &out[tr].start[(size_t)t * (kGroups * P + 1)];
-        for (int b = 0; b < kGroups; ++b)
-          for (int q = 0; q < P; ++q) {
-            *st++ = (uint32_t)ed.size();
-            for (int i = 0; i < 16; ++i) {
-              const int64_t R = row0 + 16 * b + i;
-              if (R >= n) break;
-              const int64_t kr = R / S;
-              for (int d = 0; d < 3; ++d) {
-                const int64_t kc = kr + d - 1;
-                if (kc < 0 || kc >= K) continue;
-                const int c0 = (int)(kc * S - row0);
-                for_bits(&masks[((((size_t)kr * 3 + d) * P + q) * S + R % S) * W32], W32, [&](int c) {
-                  const int rel = c0 + c;
-                  l = std::max(l, -rel);
-                  h = std::max(h, rel - (kListTile - 1));
-                  ed.push_back((uint32_t)i << 16 | (uint32_t)(rel + 2048));
-                });
-              }
-            }
-          }
-        *st = (uint32_t)ed.size();
-      }
-      lo[(size_t)w] = l;
-      hi[(size_t)w] = h;
-    }
-  }, grain_of((int64_t)unit * kListTile * P * 3 * W32 * 4));
-  auto up8 = [](int x) { return (x + 7) & ~7; };
-  for (size_t j = 0; j < todo.size(); ++j) {
-    ListScan& s = out[todo[j]];
-    const auto at = (int64_t)j * units;
-    s.lo = up8(*std::max_element(lo.begin() + at, lo.begin() + at + units));
-    s.rows = s.lo + kListTile + up8(*std::max_element(hi.begin() + at, hi.begin() + at + units));
-    // a whole number of equal TMA boxes of at most 256 rows
-    const int boxes = (s.rows + 255) / 256;
-    s.rows = up8((s.rows + boxes - 1) / boxes) * boxes;
-    // each type's steps padded to whole blocks
-    s.off.resize((size_t)n_tiles * kGroups * (P + 1));
-    uint64_t total = 0;
-    s.steps = 0;
-    uint32_t* o = s.off.data();
-    for (int64_t t = 0; t < n_tiles; ++t)
-      for (int b = 0; b < kGroups; ++b) {
-        const uint32_t* st = &s.start[(size_t)t * (kGroups * P + 1) + (size_t)b * P];
-        for (int i = 0; i <= P; ++i) {
-          *o++ = (uint32_t)total;
-          if (i == P) break;
-          const int q = type_at(i, P);
-          const uint32_t ns = steps_of(st[q + 1] - st[q]);
-          s.steps += ns;
-          total += (ns + kGatherBlock - 1) / kGatherBlock;
-        }
-      }
-    s.blocks = (int64_t)total;
-  }
-}
-
-void band_tc_emit_lists(const bg_plan* p, unsigned orientations, const ListScan* s,
-                        uint32_t* const* out) {
-  const int P = p->P;
-  const int64_t n_tiles = ((int64_t)p->K * p->S + kListTile - 1) / kListTile;
-  std::vector<int> todo;
-  int64_t steps = 0;
-  for (int d = 0; d < 2; ++d)
-    if (orientations >> d & 1) todo.push_back(d), steps += s[d].steps;
-  const int64_t jobs = n_tiles * (int64_t)todo.size();
-  parallel_ranges(jobs, [&](int64_t w0, int64_t w1) {
-    std::vector<uint32_t> tmp;
-    for (int64_t w = w0; w < w1; ++w) {
-      const int tr = todo[(size_t)(w / n_tiles)];
-      const int64_t t = w % n_tiles;
-      const ListScan& c = s[tr];
-      const uint32_t* ed = c.edges[(size_t)(t / c.unit)].data();
-      const uint32_t add = (uint32_t)(c.lo - 2048);
-      for (int b = 0; b < kGroups; ++b) {
-        const uint32_t* st = &c.start[(size_t)t * (kGroups * P + 1) + (size_t)b * P];
-        const uint32_t* off = &c.off[((size_t)t * kGroups + b) * (P + 1)];
-        for (int i = 0; i < P; ++i) {
-          const int q = type_at(i, P);
-          emit_type(ed + st[q], (int)(st[q + 1] - st[q]), add, (uint32_t)c.rows,
-                    out[tr] + (size_t)off[i] * 32 * kGatherBlock, tmp);
-        }
-      }
-    }
-  }, grain_of(jobs ? 512 * steps / jobs : 1));
-}
-
 int64_t band_tc_list_steps(const bg_plan* p, bool transposed) {
-  ListScan s[2];
-  band_tc_scan_lists(p, 1u << transposed, s);
-  return s[transposed].steps;
+  const int S = p->S, K = p->K, P = p->P, W32 = p->W32;
+  const std::vector<uint32_t>& masks = transposed ? p->masksT : p->masks;
+  std::vector<int64_t> part((size_t)K, 0);  // S is a multiple of 16: no group spans two block-rows
+  parallel_ranges(K, [&](int64_t k0, int64_t k1) {
+    for (int64_t k = k0; k < k1; ++k)
+      for (int q = 0; q < P; ++q)
+        for (int r0 = 0; r0 < S; r0 += 16) {
+          int m = 0;
+          for (int d = 0; d < 3; ++d) {
+            const uint32_t* w = &masks[((((size_t)k * 3 + d) * P + q) * S + r0) * W32];
+            for (int j = 0; j < 16 * W32; ++j) m += __builtin_popcount(w[j]);
+          }
+          part[(size_t)k] += list_steps((uint32_t)m);
+        }
+  }, grain_of((int64_t)12 * P * S * W32));
+  // the groups beyond the last row of a last tile that is not whole have one empty step per type
+  const int64_t n = (int64_t)K * S;
+  int64_t steps = ((n + 127) / 128 * 8 - n / 16) * P;
+  for (int64_t x : part) steps += x;
+  return steps;
 }
 
 void band_tc_host_lists(const bg_plan* p, bool transposed, GatherLists& out) {
-  ListScan s[2];
-  band_tc_scan_lists(p, 1u << transposed, s);
-  ListScan& c = s[transposed];
-  out.lo = c.lo, out.rows = c.rows, out.steps = c.steps, out.blocks = c.blocks;
-  if (c.blocks >> 31) return;  // the caller checks `blocks`
-  out.words.resize((size_t)c.blocks * 32 * kGatherBlock);
-  uint32_t* const to[2] = {out.words.data(), out.words.data()};
-  band_tc_emit_lists(p, 1u << transposed, s, to);
-  out.off = std::move(c.off);
+  constexpr int kTile = 128;
+  const int S = p->S, K = p->K, P = p->P, W32 = p->W32;
+  const int64_t n = (int64_t)K * S, n_tiles = (n + kTile - 1) / kTile;
+  const std::vector<uint32_t>& masks = transposed ? p->masksT : p->masks;
+  const int NB = kTile / 16;
+  // edges of every tile, as (16-row group, type), row in the group, column; reach beyond the tile
+  std::vector<std::vector<uint32_t>> edges((size_t)n_tiles);  // col - row0 + 2048 | row << 16
+  std::vector<std::vector<uint32_t>> start((size_t)n_tiles);  // (group, type) ranges, [NB * P + 1]
+  std::vector<int> lo((size_t)n_tiles, 0), hi((size_t)n_tiles, 0);
+  parallel_ranges(n_tiles, [&](int64_t t0, int64_t t1) {
+    for (int64_t t = t0; t < t1; ++t) {
+      const int64_t row0 = t * kTile;
+      auto& ed = edges[t];
+      auto& st = start[t];
+      st.reserve((size_t)NB * P + 1);
+      for (int b = 0; b < NB; ++b)
+        for (int q = 0; q < P; ++q) {
+          st.push_back((uint32_t)ed.size());
+          for (int i = 0; i < 16; ++i) {
+            const int64_t R = row0 + 16 * b + i;
+            if (R >= n) break;
+            const int64_t kr = R / S;
+            for (int d = 0; d < 3; ++d) {
+              const int64_t kc = kr + d - 1;
+              if (kc < 0 || kc >= K) continue;
+              const uint32_t* w = &masks[((((size_t)kr * 3 + d) * P + q) * S + R % S) * W32];
+              for (int j = 0; j < W32; ++j)
+                for (uint32_t m = w[j]; m; m &= m - 1) {
+                  const int rel = (int)(kc * S + 32 * j + __builtin_ctz(m) - row0);
+                  lo[t] = std::max(lo[t], -rel);
+                  hi[t] = std::max(hi[t], rel - (kTile - 1));
+                  ed.push_back((uint32_t)i << 16 | (uint32_t)(rel + 2048));
+                }
+            }
+          }
+        }
+      st.push_back((uint32_t)ed.size());
+    }
+  }, 1);
+  auto type_at = [&](int i) { return i < (P + 1) / 2 ? 2 * i : 2 * (i - (P + 1) / 2) + 1; };
+  out.off.assign((size_t)n_tiles * NB * (P + 1), 0);
+  for (int64_t t = 0; t < n_tiles; ++t)
+    for (int b = 0; b < NB; ++b)
+      for (int i = 0; i < P; ++i) {
+        const uint32_t* at = &start[t][(size_t)b * P + type_at(i)];
+        out.off[((size_t)t * NB + b) * (P + 1) + i] = at[1] - at[0];
+      }
+  const int reach[2] = {*std::max_element(lo.begin(), lo.end()), *std::max_element(hi.begin(), hi.end())};
+  list_layout(p, reach, out);
+  if (out.blocks >> 31) return;  // the caller checks `blocks`
+  out.words.assign((size_t)out.blocks * 32 * kGatherBlock, 0u);
+  parallel_ranges(n_tiles, [&](int64_t t0, int64_t t1) {
+    std::vector<uint32_t> tmp, words;
+    for (int64_t t = t0; t < t1; ++t) {
+      for (auto& e : edges[t]) e += (uint32_t)(out.lo - 2048);  // window row in the low half
+      for (int b = 0; b < NB; ++b)
+        for (int i = 0; i < P; ++i) {
+          const int q = type_at(i);
+          const uint32_t e0 = start[t][(size_t)b * P + q], e1 = start[t][(size_t)b * P + q + 1];
+          const int ns = (int)list_steps(e1 - e0);
+          words.assign((size_t)ns * 32, 0u);
+          emit_steps(edges[t].data() + e0, (int)(e1 - e0), out.rows, words.data(), tmp);
+          uint32_t* o = &out.words[(size_t)out.off[((size_t)t * NB + b) * (P + 1) + i] * 32 * kGatherBlock];
+          for (int s = 0; s < ns; ++s) {
+            const int s0 = s / kGatherBlock * kGatherBlock, in = std::min(kGatherBlock, ns - s0);
+            const uint32_t flags = (uint32_t)(in - 1) * kGatherMore + (s0 + in == ns ? kGatherLast : 0u);
+            for (int l = 0; l < 32; ++l)
+              o[((size_t)(s / kGatherBlock) * 32 + l) * kGatherBlock + s % kGatherBlock] =
+                  words[(size_t)s * 32 + l] | flags;
+          }
+        }
+    }
+  }, 1);
 }
 
 }  // namespace bg

@@ -67,7 +67,7 @@ struct bg_plan {
   // gathered band kernel: edge lists of both orientations (band_tc.h, GatherLists), and the state
   // sizes (bit H / 32) that run on them instead of the chunks above
   uint32_t list_h[2] = {0, 0};
-  char* d_lists = nullptr;  // holds the arrays below
+  char *d_lists = nullptr, *d_list_off = nullptr;  // hold the arrays below
   uint32_t* d_glist[2] = {nullptr, nullptr};
   uint32_t* d_goff[2] = {nullptr, nullptr};
   int32_t g_lo[2] = {0, 0}, g_rows[2] = {0, 0};

@@ -33,6 +33,7 @@ cudaError_t __wrap_cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t __wrap_cudaMalloc(void** p, size_t n) {
   if (++g_allocs == g_fail_alloc) return err(cudaErrorMemoryAllocation);
   char* q = static_cast<char*>(std::aligned_alloc(256, (n + 255) / 256 * 256));
+  std::memset(q, 0, n);
   g_held[q] = n;
   *p = q;
   return cudaSuccess;
@@ -42,14 +43,19 @@ cudaError_t __wrap_cudaFree(void* p) {
   std::free(p);
   return cudaSuccess;
 }
-cudaError_t __wrap_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
-  auto it = g_held.upper_bound(static_cast<char*>(d));
-  if (it == g_held.begin() || static_cast<char*>(d) + n > std::prev(it)->first + std::prev(it)->second)
+cudaError_t __wrap_cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  char* dev = static_cast<char*>(kind == cudaMemcpyDeviceToHost ? const_cast<void*>(s) : d);
+  auto it = g_held.upper_bound(dev);
+  if (it == g_held.begin() || dev + n > std::prev(it)->first + std::prev(it)->second)
     return err(cudaErrorInvalidValue);
   std::memcpy(d, s, n);
   return cudaSuccess;
 }
 cudaError_t __wrap_cudaMemset(void* d, int v, size_t n) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t __wrap_cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
+// kernels do nothing: the edge counts stay as the allocation is, 0
+cudaError_t __wrap_cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t __wrap_cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**) { return cudaSuccess; }
 cudaError_t __wrap_cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t __wrap_cudaGetLastError() { cudaError_t e = g_last; g_last = cudaSuccess; return e; }
 cudaError_t __wrap_cudaGetSymbolAddress(void** p, const void*) { *p = g_symbol; return cudaSuccess; }
