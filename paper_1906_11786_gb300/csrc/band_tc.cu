@@ -816,7 +816,7 @@ struct GaCfg {
   static constexpr int WSTAGE = (SW / 32) * H * 128;
   static constexpr bool BIAS = !BWD;                    // bias as a product
   static constexpr int DEG = BIAS ? kTile * 128 : 0;
-  static constexpr int B2 = BIAS ? H * 128 : 0;
+  static constexpr int B2 = BIAS ? H * 128 : 0;         // the bias split, or b in fp32
   static constexpr int DM = BWD ? 16 * 16 * SW * 2 : 0; // a 16-row staging tile per gather warp
   static constexpr int FIXED = DEG + B2 + DM + 1024 + 1024;
   static constexpr int THREADS = 32 * 24;
@@ -907,6 +907,22 @@ __device__ __forceinline__ void st_16x256b(uint32_t t, const float (&r)[16]) {
       "f"(r[8]), "f"(r[9]), "f"(r[10]), "f"(r[11]), "f"(r[12]), "f"(r[13]), "f"(r[14]), "f"(r[15])
       : "memory");
 }
+// 16 rows x 32 fp32 columns of TMEM in the same layout
+__device__ __forceinline__ void ld_16x256b(uint32_t t, float* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+        "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
+      : "r"(t)
+      : "memory");
+}
+// v[0], v[1] += d * b, as one instruction of two fused multiply-adds
+__device__ __forceinline__ void fma2(float* v, float d, const float2& b) {
+  asm("{\n.reg .b64 x, y, z;\nmov.b64 x, {%0, %1};\nmov.b64 y, {%2, %2};\nmov.b64 z, {%3, %4};\n"
+      "fma.rn.f32x2 x, y, z, x;\nmov.b64 {%0, %1}, x;\n}"
+      : "+f"(v[0]), "+f"(v[1])
+      : "f"(d), "f"(b.x), "f"(b.y));
+}
 // One gather warp's blocks of four steps in the order of their use: the passes of the CTA's items, one
 // per slice of the state.  Lane l holds the block range of pass `held` + l, so that moving on to the
 // next pass touches no memory.
@@ -977,6 +993,8 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
   volatile int* abort = &bars->abort;
   const int jobs = C::NH * P;
   const bool bias_mma = C::BIAS && has_bias;
+  // the bias in fp32, added by the epilogue: b2s then holds b [P][H] (launch_gather decides)
+  const bool bias32 = C::BIAS && C::SW == 64 && sc.bias != nullptr;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -987,7 +1005,7 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
     for (int i = 0; i < 6; ++i) { mbar_init(&bars->u_full[i], 8); mbar_init(&bars->u_empty[i], 1); }
     mbar_init(&bars->b2_full, 1);
     mbar_init(&bars->deg_full, 1);
-    mbar_init(&bars->deg_empty, 1);
+    mbar_init(&bars->deg_empty, bias32 ? 4 : 1);
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
     fence_mbar_init();
@@ -1048,6 +1066,9 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
     if (bias_mma) {
       mbar_expect_tx(&bars->b2_full, C::B2);
       tma_load_2d(b2s, &tm_b2, &bars->b2_full, 0, 0);
+    } else if (bias32) {
+      mbar_expect_tx(&bars->b2_full, (uint32_t)(P * H * 4));  // (P <= 32: no more than C::B2)
+      bulk_load(b2s, sc.bias, (uint32_t)(P * H * 4), &bars->b2_full);
     }
     uint32_t xi = 0, di = 0;  // windows and deg tiles so far
     uint32_t n_x[2] = {0, 0}, n_deg = 0;
@@ -1068,7 +1089,7 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
           tma_load_2d(xwin + xb * xbytes + r * 128, &tm_x, &bars->x_full[xb], C::SW * (jb / P),
                       row0 - lay.lo + r);
       }
-      if (ok && bias_mma && part <= 0) {
+      if (ok && (bias_mma || bias32) && part <= 0) {
         if (!mbar_wait(&bars->deg_empty, (di & 1) ^ 1, status, 152, abort, 32)) break;
         ++n_deg;
         ++di;
@@ -1079,7 +1100,7 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
     if (*abort) {
       for (int q = 0; q < 2; ++q) settle(&bars->x_full[q], n_x[q]);
       settle(&bars->deg_full, n_deg);
-      if (bias_mma) settle(&bars->b2_full, 1);
+      if (bias_mma || bias32) settle(&bars->b2_full, 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ issuer
@@ -1141,82 +1162,96 @@ __global__ void __launch_bounds__(GaCfg<H, BWD>::THREADS, 1)
     drain_mmas(leader, &bars->drain);
   } else if (warp >= 4 && warp < 8) {
     // ------------------------------------------------------------------ epilogue
+    // Y leaves TMEM 16 rows at a time in the fragment layout: lane l holds rows l / 4 and l / 4 + 8 and of
+    // each 8 columns the pair 2 (l % 4).  Stores (and the loads of an accumulated dE) then fill whole
+    // sectors, and a lane reads the bias of 8 columns for two rows from shared memory instead of 32 for
+    // one.  131k nodes, S = 512, H = 64: 115 us a call with a bias and 109 without; with a row per lane 130
+    // and 115, and 70 us more when the in-degrees and b came from global memory, where L1 has no room.
+    // Accumulating backward at H = 64: 267 us, with a row per lane 296.
     grid_dep_wait();  // outputs (and the accumulated dE) may still be in use by the previous kernel
-    const int r = (warp & 3) * 32 + lane;
+    const int r0 = (warp & 3) * 32 + (lane >> 2), c0 = 2 * (lane & 3);
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     int i = 0;
+    uint32_t di = 0;  // in-degree tiles so far
     for (int w = blockIdx.x; w < sc.n_items && !*abort; w += gridDim.x, ++i) {
       int k, j0, j1, part;
       item_of(sc, w, jobs, k, j0, j1, part);
-      const int row = k * kTile + r, yb = i % C::NY;
+      const int yb = i % C::NY;
       if (!mbar_wait(&bars->y_full[yb], (i / C::NY) & 1, status, 452, abort, 64)) break;
       tc_fence_after();
+      const bool biased = bias32 && part <= 0;
+      if (biased) {
+        if (!mbar_wait(&bars->deg_full, di & 1, status, 453, abort, 32)) break;
+        if (di == 0 && !mbar_wait(&bars->b2_full, 0, status, 454, abort, 32)) break;
+        ++di;
+      }
+      // a slice of a split tile writes its partial Y, summed with the other slices' by the fix-up
+      float* dst = part >= 0
+          ? sc.part + ((size_t)part * sc.part_rows + (size_t)(k - sc.n_full) * kTile + r0) * H + c0
+          : out + ((size_t)k * kTile + r0) * H + c0;
+      const bool add = accumulate && part < 0;
 #pragma unroll 1
-      for (int h0 = 0; h0 < H; h0 += 32) {
+      for (int g = 0; g < H / 16; ++g) {  // 16 rows x 32 columns at a time
+        const int h0 = (g >> 1) * 32, rb = (g & 1) * 16;
         __syncwarp();
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_base + yb * C::YC + h0, v);
+        float v[16];  // [8-column group][row / 8][pair]
+        ld_16x256b(tmem + lane_base + ((uint32_t)rb << 16) + yb * C::YC + h0, v);
         tmem_wait_ld();
-        if (h0 + 32 >= H) {
+        if (g == H / 16 - 1) {
           tc_fence_before();
           warp_arrive(&bars->y_empty[yb]);
         }
-        if (!BWD && sc.bias && part <= 0) {
-          // the bias in fp32, as the dense kernel adds it at these shapes: the in-degrees of two types
-          // per load (0 beyond the last), each times b_p
-          const uint16_t* dr = sc.deg + (size_t)row * 64;
-#pragma unroll 1
-          for (int q = 0; q < P; q += 2) {
-            const uint32_t two = *reinterpret_cast<const uint32_t*>(dr + q);
+        if (biased) {
+          // in-degree times b_p, type by type, each a fused multiply-add (an infinite b_p reaches only the
+          // rows with such an edge): two types' in-degrees per word of the swizzled tile, 0 beyond the last
+          const uint8_t* dr = degs + (r0 + rb) * 128;
+          const uint8_t* br = b2s + (h0 + c0) * 4;
+#pragma unroll 2
+          for (int q = 0; q < P; q += 2, br += 2 * H * 4) {
+            uint32_t dw[2];
+            float2 b[2][4];
 #pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              const uint32_t bits = (two >> (16 * t)) & 0xFFFFu;
-              if (!bits) continue;
-              const float d = sc.bias_f16 ? __half2float(__ushort_as_half((unsigned short)bits))
-                                          : __uint_as_float(bits << 16);
-              const float4* bq = reinterpret_cast<const float4*>(sc.bias + (size_t)(q + t) * H + h0);
+            for (int x = 0; x < 2; ++x)  // (row & 7 is the same for both rows)
+              dw[x] = *reinterpret_cast<const uint32_t*>(dr + 1024 * x + (((q >> 3) ^ (r0 & 7)) << 4) + 2 * (q & 7));
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const float4 b4 = bq[j];
-                v[4 * j] = __float_as_uint(fmaf(d, b4.x, __uint_as_float(v[4 * j])));
-                v[4 * j + 1] = __float_as_uint(fmaf(d, b4.y, __uint_as_float(v[4 * j + 1])));
-                v[4 * j + 2] = __float_as_uint(fmaf(d, b4.z, __uint_as_float(v[4 * j + 2])));
-                v[4 * j + 3] = __float_as_uint(fmaf(d, b4.w, __uint_as_float(v[4 * j + 3])));
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) b[t][j] = *reinterpret_cast<const float2*>(br + t * H * 4 + 32 * j);
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+              for (int x = 0; x < 2; ++x) {
+                const uint32_t bits = (dw[x] >> (16 * t)) & 0xFFFFu;
+                if (bits) {
+                  const float d = bias_f16 ? __half2float(__ushort_as_half((unsigned short)bits))
+                                           : __uint_as_float(bits << 16);
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) fma2(v + 4 * j + 2 * x, d, b[t][j]);
+                }
               }
-            }
           }
+          if (g == H / 16 - 1) warp_arrive(&bars->deg_empty);
         }
-        if (part >= 0) {
-          // a slice of a split tile: its partial Y, summed with the other slices' by the fix-up
-          float4* o = reinterpret_cast<float4*>(
-              sc.part + ((size_t)part * sc.part_rows + (size_t)(k - sc.n_full) * kTile + r) * H + h0);
+        float* o = dst + (size_t)rb * H + h0;
+        float2 prev[2][4];
+        if (add) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            o[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                               __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-          continue;
+          for (int x = 0; x < 2; ++x)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) prev[x][j] = *reinterpret_cast<const float2*>(o + 8 * x * H + 8 * j);
         }
-        float4* o = reinterpret_cast<float4*>(out + (size_t)row * H + h0);
 #pragma unroll
-        for (int jh = 0; jh < 8; jh += 4) {
-          float4 prev[4];
-          if (accumulate) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) prev[j] = o[jh + j];
-          }
+        for (int x = 0; x < 2; ++x)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const uint32_t* vj = v + 4 * (jh + j);
-            float4 a = make_float4(__uint_as_float(vj[0]), __uint_as_float(vj[1]),
-                                   __uint_as_float(vj[2]), __uint_as_float(vj[3]));
-            if (accumulate) {
-              a.x += prev[j].x; a.y += prev[j].y; a.z += prev[j].z; a.w += prev[j].w;
-            }
-            o[jh + j] = a;
+            float2 a = make_float2(v[4 * j + 2 * x], v[4 * j + 2 * x + 1]);
+            if (add) a.x += prev[x][j].x, a.y += prev[x][j].y;
+            *reinterpret_cast<float2*>(o + 8 * x * H + 8 * j) = a;
           }
-        }
       }
     }
+    // (as in the issuer: the bias this CTA loaded and never used must land before it ends)
+    if (bias32 && di == 0) mbar_wait(&bars->b2_full, 0, status, 455, abort, 32);
   } else if (warp >= 8) {
     // ------------------------------------------------------------------ gather
     const int gw = warp - 8, g = gw >> 3;            // types of parity g
@@ -1613,8 +1648,8 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   const bool bias32 = !BWD && o.b32 && bias_in_fp32(p->S, C::SW);
   const bool bias_mma = C::BIAS && o.b2T != nullptr && !bias32;
   tdeg = tb2 = tx;
-  if (bias_mma && (!make_map(&tdeg, p->d_deg2, n, 64, kTile) || !make_map(&tb2, o.b2T, H, 64, H)))
-    return cudaErrorInvalidValue;
+  if ((bias_mma || bias32) && !make_map(&tdeg, p->d_deg2, n, 64, kTile)) return cudaErrorInvalidValue;
+  if (bias_mma && !make_map(&tb2, o.b2T, H, 64, H)) return cudaErrorInvalidValue;
   const int smem = lay.nxb * (lay.rows + 8) * 128 + lay.nw * C::WSTAGE + C::FIXED;
   // the attribute belongs to the kernel, not to this launch: with the plan's own size, a thread with a
   // smaller plan could lower it between another thread's setting and launch
@@ -1624,12 +1659,11 @@ cudaError_t launch_gather(const bg_plan* p, const GaOps& o, int* status, cudaStr
   const int sms = num_sms();
   Sched sc = make_sched(n / kTile, C::NH * P, sms, o.split != nullptr);
   sc.part = o.split;
-  sc.deg = reinterpret_cast<const uint16_t*>(p->d_deg2);
   sc.bias = bias32 ? o.b32 : nullptr;
-  sc.bias_f16 = p->max_deg > 256 ? 1 : 0;
   e = launch_pdl(k_band_gather<H, BWD>, dim3(std::min(sc.n_items, sms)), dim3(C::THREADS),
                  smem, st, tx, tw, tdeg, tb2, (const uint32_t*)p->d_glist[BWD],
-                 (const uint32_t*)p->d_goff[BWD], o.out, o.dM, sc, lay, P, bias_mma ? 1 : 0, p->max_deg > 256 ? 1 : 0, o.accumulate, status);
+                 (const uint32_t*)p->d_goff[BWD], o.out, o.dM, sc, lay, P, bias_mma ? 1 : 0,
+                 p->max_deg > 256 ? 1 : 0, o.accumulate, status);
   note_launch();
   if (e != cudaSuccess || sc.ksplit == 1) return e;
   const int64_t n4 = (int64_t)sc.part_rows * H / 4;
