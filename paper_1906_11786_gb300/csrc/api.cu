@@ -538,9 +538,9 @@ size_t saved_Y_off(const bg_plan* p, bg_dtype dt, int H, int T, int t) {
   return saved_E_off(p, dt, H, T + 1) + (size_t)t * al(sizeof(float) * (size_t)p->n_pad() * H);
 }
 // With the band kernel and bf16 Y (H = 256): after E(0..T) and Y(0..T-1), E(0..T-1)^T and
-// Y(0..T-1)^T in [H+16][T n] bf16 arrays, written by the forward's GRU and band kernels: the band
-// products' operands and the weight-gradient GEMMs', which read the first H rows and append the
-// ones row (-> bias gradient) in shared memory; the last 16 rows are not written.
+// Y(0..T-1)^T in [H+16][T n] bf16 arrays, written by the forward's GRU and band kernels: the
+// weight-gradient GEMMs' operands, which read the first H rows and append the ones row (-> bias
+// gradient) in shared memory; the last 16 rows are not written.
 struct YbSaved {
   size_t ETa, YTa, total;
 };
@@ -567,8 +567,8 @@ bool tc_ggnn(const bg_plan* p, bg_dtype dt, int H) {
 
 // Saved activations: E(0..T) [n][H]; E(0..T-1)^T in an [H+16][T n] array; Y(0..T-1) [n][H];
 // Y(0..T-1)^T in an [H+16][T n] array (all bf16).  The transposed copies are the operands of the
-// band products (TMA, K contiguous) and of the weight-gradient GEMMs, which append the ones row
-// (-> bias gradient) in shared memory; the last 16 rows of each array are not written.
+// weight-gradient GEMMs (TMA, K contiguous), which append the ones row (-> bias gradient) in shared
+// memory; the last 16 rows of each array are not written.
 struct TcSaved {
   size_t E, ETa, Y, YTa, total;
 };
@@ -801,7 +801,7 @@ static int propagate_bwd_band(const bg_plan* p, bg_dtype dt, int H, const void* 
                                accum, status, st));
     }
     KTimer t(BG_KID_DW, st);
-    // dW_p, db_p from one split-K product of dM^T with E^T and the GEMM's appended ones row
+    // dW_p, db_p from one split-K product of dM (MN-major) with E^T and the GEMM's appended ones row
     BG_CUDA(bg::prep_transpose_bf16(E, 0, ETa, (int)n, H, 1, st));
     BG_CUDA(bg::gemm_tn(dMb, PH, 1, ETa, (int64_t)n, PH, H, (int64_t)n, 1, dW, db, accum, tpart, tpf,
                         status, st));
@@ -953,8 +953,7 @@ extern "C" int bg_ggnn_step(const bg_plan* p, bg_dtype dt, int32_t H, int32_t T,
   BG_CUDA(cudaMemcpyAsync(sv + saved_E_off(p, dt, H, 0), E0, ebytes, cudaMemcpyDeviceToDevice, st));
   if (y_bf16_path(p, dt, H)) {
     // band kernel (bf16 Y and Y^T) and the fused GRU forward (E(t+1) and E(t+1)^T): the
-    // transposed copies go to the saved E^T and Y^T arrays for the band products of the next
-    // step and for the backward's weight gradients
+    // transposed copies go to the saved E^T and Y^T arrays for the backward's weight gradients
     int* status = nullptr;
     BG_TRY(status_word_ptr(&status));
     const size_t n = (size_t)p->n_pad(), TN = (size_t)T * n;
@@ -1111,9 +1110,9 @@ extern "C" int bg_ggnn_step_bwd(const bg_plan* p, bg_dtype dt, int32_t H, int32_
   float* part = reinterpret_cast<float*>(wsc + w.part);
   const size_t pf = part_floats(p, H);
   if (y_bf16_path(p, dt, H)) {
-    // H = 256 with the band kernel: per step the gate gradients (one kernel), dX^T = (dgi W_ih)^T
+    // H = 256 with the band kernel: per step the gate gradients (one kernel), dX = dgi W_ih
     // straight into the band backward's operand, g += dgh W_hh, the transposed-band backward and
-    // the band's weight gradients from its dM_p^T (one step's K range of E^T stays in L2
+    // the band's weight gradients from its dM_p (one step's K range of E^T stays in L2
     // across the M tiles, which a product over all T steps at once does not); the GRU's weight
     // gradients in one grouped product over all T steps at the end (operands E^T, Y^T
     // saved by the forward).  The running state gradient alternates between two buffers.

@@ -50,9 +50,10 @@ int resolve_scratch(int dev, char** out) {
 
 inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Scratch this entry point uses for (plan, dtype, H): the tensor-core kernels' operands (E^T, the
-// second-product weights, the bias split and the split-tile partials), or the SIMT path's
-// messages M_p = E W_p + b_p for every type.
+// Scratch this entry point uses for (plan, dtype, H): the tensor-core kernels' operands (the
+// second-product weights, the bias split and the split-tile partials, and n_pad H 2 bytes that the
+// transposed states once took and the limit still counts), or the SIMT path's messages
+// M_p = E W_p + b_p for every type.
 size_t need_bytes(const bg_plan* p, bg_dtype dt, int H) {
   if (bg::band_tc_supported(p, (int)dt, H)) return bg::band_tc_fwd_ws_bytes(p, (int)dt, H);
   return al(sizeof(float) * (size_t)p->P * p->n_pad() * H);
