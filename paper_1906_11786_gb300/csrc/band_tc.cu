@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(Cfg<H, S, BWD>::THREADS, 1)
 // Bound: latency along each warp's chain (words, ldmatrix, products, TMEM store), with the shared-memory
 // and tensor pipes each about half busy at 16 warps of 80 registers.  A step (4 ldmatrix.x4, 8 mma.sync)
 // takes 26 cycles of the SM with conflict-free rows, 44 with random ones, which is why the plan deals
-// edges into sets of 8 whose rows differ mod 8.  S = 512, H = 64, 131k nodes, 52 edges per node: 112 us
+// edges into sets of 8 whose rows differ mod 8.  S = 512, H = 64, 131k nodes, 52 edges per node: 113 us
 // against the dense kernel's 457; S = 256, H = 128, 20k nodes backward: 61 us against 89 (ncu).
 //
 // Roles (24 warps, one CTA per SM, persistent over the same items as k_band_tc):
@@ -1703,7 +1703,9 @@ bool gather_fits(int lo, int rows, int H) {
 // against 103, 125 and 238 against 222; S = 512 forward 37 and 74 against 183, 50 and 107 against 225,
 // 100 and 214 against 495, backward 50 and 82 against 186, 68 and 120 against 187, 146 and 241 against
 // 560.  The entries lie where the measured lines cross, or at S = 512 at half the distance beyond the
-// last measured point (about 80 steps).  At S = 128 the two are within 7% of one another at H = 64 and
+// last measured point (about 80 steps); there, at 20k nodes and about 150 steps, the lists still take 60 us
+// a call against 80 at H = 32, 87 against 105 at H = 64 and 158 against 218 at H = 128 forward, 89 against
+// 107 and 238 against 300 backward at H = 32 and 128.  At S = 128 the two are within 7% of one another at H = 64 and
 // 52 edges per node, and the lists are not built there.
 int gather_max_steps(int S, int H, bool bwd) {
   if (S != 256 && S != 512) return 0;
