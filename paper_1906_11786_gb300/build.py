@@ -47,13 +47,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = _nvcc()
     hdrs = _headers()
     common = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-lineinfo", "-I", INCLUDE, "-I", CSRC]
+    # device code stored as it is: nvcc compresses objects above a size by itself, and unpacking the band
+    # kernels' then took 8 ms of a process's first upload, which loads them
+    device = ARCH + ["--compress-mode=none"]
     jobs = []
     objs = []
     for src in _sources():
         obj = os.path.join(BUILD, os.path.basename(src) + ".o")
         objs.append(obj)
         if force or _stale(obj, [src] + hdrs):
-            cmd = [nvcc] + ARCH + common + ["-c", src, "-o", obj]
+            cmd = [nvcc] + device + common + ["-c", src, "-o", obj]
             if src.endswith(".cpp"):
                 cmd = [nvcc] + common + ["-x", "c++", "-c", src, "-o", obj]
             jobs.append(cmd)
